@@ -184,6 +184,15 @@ int pkd_range_count(const pkd_tree* tree, const int32_t* lo, const int32_t* hi, 
 int pkd_range_report(const pkd_tree* tree, const int32_t* lo, const int32_t* hi, uint64_t q, uint64_t* offsets,
                      uint32_t* ids, uint64_t ids_cap, uint64_t* total, void* stream);
 
+/* The ids of a range report whose offsets are known: offsets (device, [q + 1])
+ * are those that pkd_range_report (with ids NULL, ids_cap 0) gave for the same
+ * boxes on the unchanged tree.  Saves the second counting of a caller that
+ * sizes its buffer first.  Box i's ids are written below offsets[i + 1] and
+ * ids_cap only: other offsets leave ids incomplete.  Asynchronous like
+ * pkd_knn. */
+int pkd_range_report_ids(const pkd_tree* tree, const int32_t* lo, const int32_t* hi, uint64_t q,
+                         const uint64_t* offsets, uint32_t* ids, uint64_t ids_cap, void* stream);
+
 /* Stored bounding boxes: the paper's Pkd-bb variant (Sec. 6, the study of
  * bounding boxes).  With enable = 1 every node keeps the tight box of the
  * points in its subtree (8d bytes per node slot, computed bottom-up now and

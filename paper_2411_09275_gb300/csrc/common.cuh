@@ -66,6 +66,7 @@ struct DevStatus {
   int detail;
   uint32_t max_depth;
   int idflags;  // id-table flags of the running call (IDF_* in ids.cuh)
+  unsigned long long refused;  // number of the last query call whose coordinates were out of range
   unsigned long long counters[8];
 };
 

@@ -165,6 +165,21 @@ void dfree(T*& p, cudaStream_t s) {
   p = nullptr;
 }
 
+// Scratch buffers of one call, freed in stream order when it returns.
+struct Scratch {
+  cudaStream_t s;
+  std::vector<void*> ptrs;
+  ~Scratch() {
+    for (void* p : ptrs) cudaFreeAsync(p, s);
+  }
+  template <class T>
+  int get(T** p, size_t n) {
+    int e = dalloc(p, n, s);
+    if (e == PKD_OK) ptrs.push_back(*p);
+    return e;
+  }
+};
+
 // Pinned host blocks of PINNED_BLOCK bytes from a library-owned pool that
 // grows by whole chunks and is never returned (pinning and unpinning memory
 // are slow, synchronising driver calls).  nullptr when pinning fails.
@@ -187,6 +202,7 @@ struct PinnedBlock {
 
 // Reads the device status word; PKD_OK or the mapped error.
 int check_status(TreeMem& t, cudaStream_t s);
+int status_code(int err, int detail);
 
 // Kernel timing (CUDA events on the launching stream).
 struct KTimer {

@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(QTHREADS) k_knn(QueryArgs a) {
   constexpr int U = 32 / G;  // points per lane and step
   static_assert(D <= G, "a lane per dimension");
   extern __shared__ __align__(16) unsigned char sm[];
+  if (query_refused(a)) return;
   const int lane = threadIdx.x & (G - 1);
   const int gshift = (threadIdx.x & 31) & ~(G - 1);
   const uint64_t qi = (uint64_t)blockIdx.x * (QTHREADS / G) + threadIdx.x / G;
@@ -295,11 +296,10 @@ int pkd::knn_on(TreeMem& t, uint32_t root, const int32_t* queries, uint64_t q, i
   if (q == 0) return PKD_OK;
   if (!queries || !out_ids || !out_d2) return PKD_EINVAL;
   TreeTouch touch{&t, s};
-  bool ok;
-  PKD_TRY_(validate_coords(queries, q * (uint64_t)t.p.d, s, &ok));
-  if (!ok) return PKD_EINVAL;
-  PKD_TRY_(check_status(t, s));
+  QueryCheck check(t, s);
+  PKD_TRY_(check.begin(queries, q * (uint64_t)t.p.d, nullptr, 0));
   QueryArgs a{};
+  a.call = check.call;
   a.nodes = t.nodes;
   a.ndim = t.ndim;
   a.A = t.A;
@@ -317,7 +317,7 @@ int pkd::knn_on(TreeMem& t, uint32_t root, const int32_t* queries, uint64_t q, i
     PKD_QDISPATCH(t.p.d, launch_knn, ac, s);
   }));
   PKD_CUDA(cudaGetLastError());
-  return PKD_OK;
+  return check.end();
 }
 
 

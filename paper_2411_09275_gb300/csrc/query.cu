@@ -15,6 +15,9 @@
 // thread per box (before) walked node after node with the subspace's 2d
 // bounds in a local-memory stack; 1e4 boxes of about 300 points in 3e6
 // clustered 2-D points: count 0.45-0.60 -> 0.033 ms, report 3.2 -> 0.13 ms.
+#include <atomic>
+
+#include "coords.cuh"
 #include "query.cuh"
 
 namespace pkd {
@@ -101,6 +104,7 @@ __device__ __forceinline__ bool range_in(const Pts& A, uint64_t g, const int32_t
 #define RANGE_PROLOGUE                                                                              \
   constexpr unsigned FULL = 0xffffffffu;                                                            \
   extern __shared__ __align__(16) unsigned char sm[];                                               \
+  if (query_refused(a)) return;                                                                     \
   const int lane = threadIdx.x & 31;                                                                \
   const uint64_t qi = (uint64_t)blockIdx.x * (QTHREADS / 32) + threadIdx.x / 32;                    \
   if (qi >= a.nq) return;                                                                           \
@@ -172,11 +176,12 @@ __global__ void __launch_bounds__(QTHREADS) k_range_count(QueryArgs a) {
 // walked to its leaves too: after updates its points need not be contiguous
 // in the arena.)
 template <int D, bool DEEP>
-__global__ void __launch_bounds__(QTHREADS) k_range_report(QueryArgs a, const uint64_t* offsets, uint32_t* out_ids) {
+__global__ void __launch_bounds__(QTHREADS) k_range_report(QueryArgs a, const uint64_t* offsets, uint32_t* out_ids,
+                                                             uint64_t ids_cap) {
   RANGE_PROLOGUE
   const int g = lane >> 3, gl = lane & 7;
   uint64_t pos = offsets[qi];
-  const uint64_t end = offsets[qi + 1];
+  const uint64_t end = min(offsets[qi + 1], ids_cap);
   while (sp > 0) {
     const int p = sp > RANGE_WIDE ? 1 : min(sp, 32);
     const uint2 e = lane < p ? st[sp - 1 - lane] : make_uint2(0, 0);
@@ -237,8 +242,8 @@ __global__ void __launch_bounds__(QTHREADS) k_range_report(QueryArgs a, const ui
           if (k < g) before += t;
           tot += t;
         }
-        if (pos + (uint64_t)tot > end) {  // more points than counted: the tree changed
-          if (lane == 0) set_error(a.st, DERR_STATE, 902);
+        if (pos > end || (uint64_t)tot > end - pos) {  // more points than counted: the tree changed
+          if (lane == 0 && !a.given_offsets) set_error(a.st, DERR_STATE, 902);
           return;
         }
 #pragma unroll
@@ -256,8 +261,8 @@ __global__ void __launch_bounds__(QTHREADS) k_range_report(QueryArgs a, const ui
           const uint32_t b = b0 + lane;
           const bool in = b < s0 && (all0 || range_in<D>(a.A, (uint64_t)a0 + b, lo, hi));
           const unsigned m = __ballot_sync(FULL, in);
-          if (pos + (uint64_t)__popc(m) > end) {
-            if (lane == 0) set_error(a.st, DERR_STATE, 902);
+          if (pos > end || (uint64_t)__popc(m) > end - pos) {
+            if (lane == 0 && !a.given_offsets) set_error(a.st, DERR_STATE, 902);
             return;
           }
           if (in) out_ids[pos + __popc(m & ((1u << lane) - 1u))] = a.A.id[(uint64_t)a0 + b];
@@ -269,9 +274,12 @@ __global__ void __launch_bounds__(QTHREADS) k_range_report(QueryArgs a, const ui
   }
 }
 
-// Exclusive scan of q 64-bit counts into offsets[0..q] (offsets[q] = total):
-// per-block sums, one block over the sums, then the blocks again.
+// Exclusive scan of q 64-bit counts into offsets[0..q] (offsets[q] = total,
+// also stored to host_total): one block for up to SCAN64_ONE counts (a launch
+// instead of three and, with the total stored to pinned memory, no copy back),
+// else per-block sums, one block over the sums, then the blocks again.
 constexpr int SCAN64_THREADS = 256, SCAN64_PER = 8, SCAN64_TILE = SCAN64_THREADS * SCAN64_PER;
+constexpr uint64_t SCAN64_ONE = 16 * SCAN64_TILE;
 
 __device__ __forceinline__ uint64_t block_scan64(uint64_t v, uint64_t* sh, uint64_t* total) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -318,31 +326,89 @@ __global__ void k_scan64_partials(uint64_t* partial, uint64_t nb) {
   if (threadIdx.x == 0) partial[nb] = carry;
 }
 
-__global__ void k_scan64_apply(const uint64_t* in, uint64_t n, const uint64_t* partial, uint64_t* out) {
+// Tile blockIdx.x + k * gridDim.x of the scan; `partial` null: one block over all tiles.
+__global__ void k_scan64_apply(QueryArgs a, const uint64_t* in, uint64_t n, const uint64_t* partial, uint64_t* out,
+                               uint64_t* host_total) {
   __shared__ uint64_t sh[SCAN64_THREADS / 32];
-  const uint64_t base = (uint64_t)blockIdx.x * SCAN64_TILE + (uint64_t)threadIdx.x * SCAN64_PER;
-  uint64_t v[SCAN64_PER], s = 0;
-  for (int k = 0; k < SCAN64_PER; ++k) {
-    v[k] = base + k < n ? in[base + k] : 0;
-    s += v[k];
+  if (__syncthreads_or(threadIdx.x < 32 && query_refused(a))) return;  // no counts were written
+  uint64_t carry = partial ? partial[blockIdx.x] : 0;
+  for (uint64_t tile = blockIdx.x; tile * SCAN64_TILE < n; tile += gridDim.x) {
+    const uint64_t base = tile * SCAN64_TILE + (uint64_t)threadIdx.x * SCAN64_PER;
+    uint64_t v[SCAN64_PER], s = 0;
+    for (int k = 0; k < SCAN64_PER; ++k) {
+      v[k] = base + k < n ? in[base + k] : 0;
+      s += v[k];
+    }
+    uint64_t tot;
+    uint64_t run = carry + block_scan64(s, sh, &tot);
+    for (int k = 0; k < SCAN64_PER; ++k) {
+      if (base + k < n) out[base + k] = run;
+      run += v[k];
+    }
+    carry += tot;
   }
-  uint64_t tot;
-  uint64_t run = partial[blockIdx.x] + block_scan64(s, sh, &tot);
-  for (int k = 0; k < SCAN64_PER; ++k) {
-    if (base + k < n) out[base + k] = run;
-    run += v[k];
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+    out[n] = carry;
+    *(volatile uint64_t*)host_total = carry;
   }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = partial[gridDim.x];
+}
+
+__global__ void k_query_check(const int32_t* c1, uint64_t n1, const int32_t* c2, uint64_t n2, DevStatus* st,
+                              unsigned long long call, QueryHost* h) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    h->err = st->err;
+    h->detail = st->detail;
+  }
+  const unsigned b = coord_bits(c1, n1) | (c2 ? coord_bits(c2, n2) : 0);
+  if (__any_sync(0xffffffffu, (b >> 30) != 0) && (threadIdx.x & 31) == 0) {
+    *(volatile unsigned long long*)&st->refused = call;
+    *(volatile int*)&h->bad = 1;
+  }
+}
+
+int QueryCheck::begin(const int32_t* c1, uint64_t n1, const int32_t* c2, uint64_t n2) {
+  static std::atomic<unsigned long long> calls{0};
+  h = (volatile QueryHost*)pinned_get();
+  if (!h) return PKD_ENOMEM;
+  h->bad = 0;
+  call = ++calls;
+  KTimer kt;
+  ktimer_begin(kt, "validate", n1 + (c2 ? n2 : 0), s);
+  PKD_LAUNCH(k_query_check<<<coord_blocks(n1), 256, 0, s>>>(c1, n1, c2, n2, t.st, call, (QueryHost*)h));
+  ktimer_end(kt);
+  if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess || cudaEventRecord(ev, s) != cudaSuccess) {
+    cudaGetLastError();
+    PKD_CUDA(cudaStreamSynchronize(s));
+    if (ev) cudaEventDestroy(ev);
+    ev = nullptr;
+  }
+  return PKD_OK;
+}
+
+int QueryCheck::end() {
+  if (ev) PKD_CUDA(cudaEventSynchronize(ev));
+  if (h->bad) return PKD_EINVAL;
+  return status_code(h->err, h->detail);
+}
+
+QueryCheck::~QueryCheck() {
+  if (ev) {
+    cudaEventSynchronize(ev);  // the check writes to the block until then
+    cudaEventDestroy(ev);
+  }
+  if (h) pinned_put((void*)h);
 }
 
 template <int D>
-static void launch_report(const QueryArgs& a, const uint64_t* offsets, uint32_t* ids, cudaStream_t s) {
+static void launch_report(const QueryArgs& a, const uint64_t* offsets, uint32_t* ids, uint64_t ids_cap,
+                          cudaStream_t s) {
   constexpr int WPB = QTHREADS / 32;
   const uint64_t g = (a.nq + WPB - 1) / WPB;
   KTimer kt;
   ktimer_begin(kt, "range_report", a.nq, s);
-  if (a.deep) launch_query(k_range_report<D, true>, g, 0, s, a, offsets, ids);
-  else launch_query(k_range_report<D, false>, g, (size_t)WPB * a.cap * sizeof(uint2), s, a, offsets, ids);
+  if (a.deep) launch_query(k_range_report<D, true>, g, 0, s, a, offsets, ids, ids_cap);
+  else launch_query(k_range_report<D, false>, g, (size_t)WPB * a.cap * sizeof(uint2), s, a, offsets, ids,
+                    ids_cap);
   ktimer_end(kt);
 }
 
@@ -361,6 +427,40 @@ static void launch_rc(const QueryArgs& a, cudaStream_t s) {
 
 using namespace pkd;
 
+namespace {
+
+// A box query's arguments.
+QueryArgs range_args(const TreeMem& t, const QueryCheck& check, const int32_t* lo, const int32_t* hi, uint64_t q) {
+  QueryArgs a{};
+  a.call = check.call;
+  a.nodes = t.nodes;
+  a.ndim = t.ndim;
+  a.A = t.A;
+  a.root = t.root;
+  a.q = lo;
+  a.hi = hi;
+  a.nq = q;
+  a.st = t.st;
+  a.box = t.bbox_on ? t.bbox : nullptr;
+  return a;
+}
+
+int range_counts(const TreeMem& t, const QueryArgs& a, uint64_t* counts, cudaStream_t s) {
+  return for_query_chunks(t, a, 2, RANGE_EXTRA, s, [&](QueryArgs ac, uint64_t c0) {
+    ac.out_cnt = counts + c0;
+    PKD_QDISPATCH(t.p.d, launch_rc, ac, s);
+  });
+}
+
+int range_ids(const TreeMem& t, const QueryArgs& a, const uint64_t* offsets, uint32_t* ids, uint64_t cap,
+              cudaStream_t s) {
+  return for_query_chunks(t, a, 2, RANGE_EXTRA, s, [&](QueryArgs ac, uint64_t c0) {
+    PKD_QDISPATCH(t.p.d, launch_report, ac, offsets + c0, ids, cap, s);
+  });
+}
+
+}  // namespace
+
 extern "C" {
 
 int pkd_range_count(const pkd_tree* tc, const int32_t* lo, const int32_t* hi, uint64_t q,
@@ -371,28 +471,12 @@ int pkd_range_count(const pkd_tree* tc, const int32_t* lo, const int32_t* hi, ui
   TreeMem& t = const_cast<TreeMem&>(tc->m);
   cudaStream_t s = (cudaStream_t)stream;
   TreeTouch touch{&t, s};
-  bool ok1, ok2;
-  PKD_TRY_(validate_coords(lo, q * (uint64_t)t.p.d, s, &ok1));
-  PKD_TRY_(validate_coords(hi, q * (uint64_t)t.p.d, s, &ok2));
-  if (!ok1 || !ok2) return PKD_EINVAL;
-  PKD_TRY_(check_status(t, s));
-  QueryArgs a{};
-  a.nodes = t.nodes;
-  a.ndim = t.ndim;
-  a.A = t.A;
-  a.root = t.root;
-  a.q = lo;
-  a.hi = hi;
-  a.nq = q;
-  a.out_cnt = out_counts;
-  a.st = t.st;
-  a.box = t.bbox_on ? t.bbox : nullptr;
-  PKD_TRY_(for_query_chunks(t, a, 2, RANGE_EXTRA, s, [&](QueryArgs ac, uint64_t c0) {
-    ac.out_cnt = out_counts + c0;
-    PKD_QDISPATCH(t.p.d, launch_rc, ac, s);
-  }));
+  const uint64_t nc = q * (uint64_t)t.p.d;
+  QueryCheck check(t, s);
+  PKD_TRY_(check.begin(lo, nc, hi, nc));
+  PKD_TRY_(range_counts(t, range_args(t, check, lo, hi, q), out_counts, s));
   PKD_CUDA(cudaGetLastError());
-  return PKD_OK;
+  return check.end();
 }
 
 int pkd_range_report(const pkd_tree* tc, const int32_t* lo, const int32_t* hi, uint64_t q, uint64_t* offsets,
@@ -404,58 +488,50 @@ int pkd_range_report(const pkd_tree* tc, const int32_t* lo, const int32_t* hi, u
   TreeMem& t = const_cast<TreeMem&>(tc->m);
   cudaStream_t s = (cudaStream_t)stream;
   TreeTouch touch{&t, s};
-  bool ok1, ok2;
-  PKD_TRY_(validate_coords(lo, q * (uint64_t)t.p.d, s, &ok1));
-  PKD_TRY_(validate_coords(hi, q * (uint64_t)t.p.d, s, &ok2));
-  if (!ok1 || !ok2) return PKD_EINVAL;
-  PKD_TRY_(check_status(t, s));
-  // pass 1: counts (into offsets[0..q)), scanned in place into offsets[0..q]
-  uint64_t* counts = nullptr;
-  uint64_t* partial = nullptr;
-  const uint64_t nb = (q + SCAN64_TILE - 1) / SCAN64_TILE;
-  PKD_TRY_(dalloc(&counts, q, s));
-  int e = dalloc(&partial, nb + 1, s);
-  if (e) {
-    dfree(counts, s);
-    return e;
+  const uint64_t nc = q * (uint64_t)t.p.d;
+  QueryCheck check(t, s);
+  PKD_TRY_(check.begin(lo, nc, hi, nc));
+  // pass 1: counts, scanned into offsets[0..q]
+  const uint64_t nb = q <= SCAN64_ONE ? 1 : (q + SCAN64_TILE - 1) / SCAN64_TILE;
+  Scratch sc{s, {}};
+  uint64_t *counts, *partial = nullptr;
+  PKD_TRY_(sc.get(&counts, q));
+  if (nb > 1) PKD_TRY_(sc.get(&partial, nb + 1));
+  PinnedBlock tot(s);
+  if (!tot.p) return PKD_ENOMEM;
+  const QueryArgs a = range_args(t, check, lo, hi, q);
+  PKD_TRY_(range_counts(t, a, counts, s));
+  if (nb > 1) {
+    PKD_LAUNCH(k_scan64_reduce<<<(unsigned)nb, SCAN64_THREADS, 0, s>>>(counts, q, partial));
+    PKD_LAUNCH(k_scan64_partials<<<1, SCAN64_THREADS, 0, s>>>(partial, nb));
   }
-  QueryArgs a{};
-  a.nodes = t.nodes;
-  a.ndim = t.ndim;
-  a.A = t.A;
-  a.root = t.root;
-  a.q = lo;
-  a.hi = hi;
-  a.nq = q;
-  a.out_cnt = counts;
-  a.st = t.st;
-  a.box = t.bbox_on ? t.bbox : nullptr;
-  e = for_query_chunks(t, a, 2, RANGE_EXTRA, s, [&](QueryArgs ac, uint64_t c0) {
-    ac.out_cnt = counts + c0;
-    PKD_QDISPATCH(t.p.d, launch_rc, ac, s);
-  });
-  if (e) {
-    dfree(counts, s);
-    dfree(partial, s);
-    return e;
-  }
-  PKD_LAUNCH(k_scan64_reduce<<<(unsigned)nb, SCAN64_THREADS, 0, s>>>(counts, q, partial));
-  PKD_LAUNCH(k_scan64_partials<<<1, SCAN64_THREADS, 0, s>>>(partial, nb));
-  PKD_LAUNCH(k_scan64_apply<<<(unsigned)nb, SCAN64_THREADS, 0, s>>>(counts, q, partial, offsets));
-  dfree(counts, s);
-  dfree(partial, s);
-  uint64_t tot = 0;
-  PKD_CUDA(cudaMemcpyAsync(&tot, offsets + q, 8, cudaMemcpyDeviceToHost, s));
+  PKD_LAUNCH(k_scan64_apply<<<(unsigned)nb, SCAN64_THREADS, 0, s>>>(a, counts, q, partial, offsets, (uint64_t*)tot.p));
   PKD_CUDA(cudaStreamSynchronize(s));
-  *total = tot;
-  if (tot > ids_cap || (tot > 0 && !ids)) return PKD_EINVAL;
+  PKD_TRY_(check.end());  // a refused call's counts were not written
+  *total = *(volatile uint64_t*)tot.p;
+  if (*total > ids_cap || (*total > 0 && !ids)) return PKD_EINVAL;
   // pass 2: the ids
-  PKD_TRY_(for_query_chunks(t, a, 2, RANGE_EXTRA, s, [&](QueryArgs ac, uint64_t c0) {
-    PKD_QDISPATCH(t.p.d, launch_report, ac, offsets + c0, ids, s);
-  }));
+  PKD_TRY_(range_ids(t, a, offsets, ids, ids_cap, s));
   PKD_CUDA(cudaGetLastError());
   return PKD_OK;
 }
 
-}  // extern "C"
+int pkd_range_report_ids(const pkd_tree* tc, const int32_t* lo, const int32_t* hi, uint64_t q, const uint64_t* offsets,
+                         uint32_t* ids, uint64_t ids_cap, void* stream) {
+  if (!tc) return PKD_EINVAL;
+  if (q == 0) return PKD_OK;
+  if (!lo || !hi || !offsets || (ids_cap > 0 && !ids)) return PKD_EINVAL;
+  TreeMem& t = const_cast<TreeMem&>(tc->m);
+  cudaStream_t s = (cudaStream_t)stream;
+  TreeTouch touch{&t, s};
+  const uint64_t nc = q * (uint64_t)t.p.d;
+  QueryCheck check(t, s);
+  PKD_TRY_(check.begin(lo, nc, hi, nc));
+  QueryArgs a = range_args(t, check, lo, hi, q);
+  a.given_offsets = true;
+  PKD_TRY_(range_ids(t, a, offsets, ids, ids_cap, s));
+  PKD_CUDA(cudaGetLastError());
+  return check.end();
+}
 
+}  // extern "C"

@@ -596,20 +596,6 @@ static Pts shifted(const Pts& p, uint64_t base) {
   return q;
 }
 
-struct Scratch {
-  cudaStream_t s;
-  std::vector<void*> ptrs;
-  ~Scratch() {
-    for (void* p : ptrs) cudaFreeAsync(p, s);
-  }
-  template <class T>
-  int get(T** p, size_t n) {
-    int e = dalloc(p, n, s);
-    if (e == PKD_OK) ptrs.push_back(*p);
-    return e;
-  }
-};
-
 #define PKD_TRY(x)               \
   do {                           \
     int _r = (x);                \

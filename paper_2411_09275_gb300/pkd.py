@@ -71,6 +71,7 @@ def lib():
         L.pkd_range_count.argtypes = [vp, vp, vp, u64, vp, vp]
         L.pkd_knn_ids_noalloc.argtypes = [vp, vp, u64, i32, vp, vp]
         L.pkd_range_report.argtypes = [vp, vp, vp, u64, vp, vp, u64, P(u64), vp]
+        L.pkd_range_report_ids.argtypes = [vp, vp, vp, u64, vp, vp, u64, vp]
         L.pkd_build_forest.argtypes = [vp, vp, P(u64), C.c_uint32, P(pkd_params), vp, P(vp)]
         L.pkd_forest_trees.restype = C.c_uint32
         L.pkd_forest_trees.argtypes = [vp]
@@ -95,7 +96,7 @@ def lib():
         L.pkd_kernel_timing.argtypes = [i32]
         L.pkd_kernel_stats.argtypes = [C.c_char_p, P(u64), P(C.c_double), P(u64)]
         for f in ("pkd_build", "pkd_batch_insert", "pkd_batch_delete", "pkd_knn", "pkd_range_count",
-                  "pkd_knn_ids_noalloc", "pkd_range_report", "pkd_set_bounding_boxes", "pkd_export_boxes", "pkd_mem_info", "pkd_build_forest", "pkd_forest_export", "pkd_forest_knn", "pkd_export", "pkd_height", "pkd_set_option", "pkd_kernel_timing",
+                  "pkd_knn_ids_noalloc", "pkd_range_report", "pkd_range_report_ids", "pkd_set_bounding_boxes", "pkd_export_boxes", "pkd_mem_info", "pkd_build_forest", "pkd_forest_export", "pkd_forest_knn", "pkd_export", "pkd_height", "pkd_set_option", "pkd_kernel_timing",
                   "pkd_kernel_stats"):
             getattr(L, f).restype = i32
         _lib = L
@@ -195,8 +196,9 @@ def pkd_range_report(tree, lo: torch.Tensor, hi: torch.Tensor, stream=None):
     if r != PKD_OK and not (r == PKD_EINVAL and tot.value > 0):
         _check(r, "pkd_range_report")
     ids = torch.empty(max(int(tot.value), 1), dtype=torch.int32, device=lo.device)
-    _check(lib().pkd_range_report(tree, _dptr(lo), _dptr(hi), q, _dptr(offsets), _dptr(ids), ids.numel(),
-                                  C.byref(tot), _stream(stream)), "pkd_range_report")
+    if tot.value:
+        _check(lib().pkd_range_report_ids(tree, _dptr(lo), _dptr(hi), q, _dptr(offsets), _dptr(ids), ids.numel(),
+                                          _stream(stream)), "pkd_range_report")
     return offsets, ids[:int(tot.value)]
 
 

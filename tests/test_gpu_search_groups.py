@@ -79,3 +79,52 @@ def test_range_faces_and_leaf_order(kind, n, d, phi):
         gone = ex["leaf_ids"][::3].copy()
         assert t.delete(ids_dev(gone)) == o.delete(gone)
     t.close()
+
+
+def test_refused_queries_write_nothing_and_offsets_bound_the_ids():
+    # the search is queued behind its coordinate check: a refused call leaves
+    # its outputs alone, the next call is served
+    import ctypes as C
+
+    import torch
+
+    pkd, t, o, X = _tree("uniform", 5000, 3, 32, 61)
+    Q = I.uniform(700, 3, 62)
+    bad = Q.copy()
+    bad[699, 2] = 1 << 30
+    oi = torch.full((700, 5), -7, dtype=torch.int32, device="cuda")
+    od = torch.full((700, 5), -7, dtype=torch.int64, device="cuda")
+    cnt = torch.full((700,), -7, dtype=torch.int64, device="cuda")
+    hi = np.maximum(Q, TOP - 5)
+    for k in range(3):
+        with pytest.raises(pkd.PkdError) as e:
+            if k == 0:
+                pkd.pkd_knn(t._h, to_dev(bad), 5, oi, od)
+            elif k == 1:
+                pkd.pkd_range_count(t._h, to_dev(bad), to_dev(hi), cnt)
+            else:
+                pkd.pkd_range_count(t._h, to_dev(Q), to_dev(-hi), cnt)
+        assert e.value.code == pkd.PKD_EINVAL
+    torch.cuda.synchronize()
+    assert (oi == -7).all().item() and (od == -7).all().item() and (cnt == -7).all().item()
+    gi, gd = t.knn(to_dev(Q), 5)
+    wi, wd = o.knn(Q, 5)
+    assert np.array_equal(gd.cpu().numpy(), wd) and np.array_equal(gi.cpu().numpy().view(np.uint32), wi)
+    # more boxes than one block scans, and ids under offsets cut short
+    q = 40000
+    lo, hi = I.boxes(q, 3, 1 << 27, 63)
+    off, ids = pkd.pkd_range_report(t._h, to_dev(lo), to_dev(hi))
+    assert np.array_equal(off.cpu().numpy(), np.concatenate([[0], np.cumsum(o.range_count(lo, hi).astype(np.int64))]))
+    n = ids.numel()
+    out = torch.full((n + 64,), -7, dtype=torch.int32, device="cuda")
+    gl, gh = to_dev(lo), to_dev(hi)
+    for cap in (n, n // 2, 0):
+        out.fill_(-7)
+        r = pkd.lib().pkd_range_report_ids(t._h, pkd._dptr(gl), pkd._dptr(gh), C.c_uint64(q), pkd._dptr(off),
+                                           pkd._dptr(out), C.c_uint64(cap), pkd._stream(None))
+        torch.cuda.synchronize()
+        assert r == pkd.PKD_OK and (out[cap:] == -7).all().item()
+        if cap == n:
+            assert (out[:n] == ids).all().item()
+    assert np.array_equal(t.range_count(gl[:50], gh[:50]).cpu().numpy().astype(np.uint64), o.range_count(lo[:50], hi[:50]))
+    t.close()
