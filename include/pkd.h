@@ -287,11 +287,15 @@ const char* pkd_strerror(int code);
  *   "base_kernel" shared-memory base case: 0 sorts each subproblem once per
  *                dimension and splits by lookups (default), 1 selects every
  *                splitter by a radix select
- *   "graph_rounds" 1 (default): a build's rounds run from one CUDA graph whose
+ *   "graph_rounds" 1: a build's rounds run from one CUDA graph whose
  *                WHILE / IF nodes test device-side counts, and its base cases
  *                are persistent launches over device-side lists; 0: the same
  *                kernels with the host reading the counts after every step
- *                (one stream synchronisation per round and skeleton level)
+ *                (one stream synchronisation per round and skeleton level).
+ *                Until it is set, builds run as with 1, except that one whose
+ *                subproblems are known to fit shared memory (a single tree of
+ *                at most base_cap points, an update's rebuild of small
+ *                subtrees) has no rounds and launches its base cases directly
  *   "front_cap"  > 0: first capacity (entries) of the lists with which an
  *                update flattens the subtrees it rebuilds (testing; 0, the
  *                default, sizes them by the points of those subtrees).  A

@@ -137,7 +137,7 @@ int boxes_compute(TreeMem& t, cudaStream_t s) {
   uint32_t *all, *ctr;
   PKD_TRY(sc.get(&all, cap));
   PKD_TRY(sc.get(&ctr, 1));
-  PinnedBlock hb(s);
+  PinnedBlock hb;
   if (!hb.p) return PKD_ENOMEM;
   uint32_t* hn = (uint32_t*)hb.p;
   PKD_TRY_(dev_store(all, &t.root, 4, s));

@@ -556,8 +556,9 @@ static void launch_smem_warp(const SmemArgs& a, uint32_t nblocks, size_t smb, cu
 __global__ void k_classify(const RoundDyn* dyn, const uint32_t* sel, const uint32_t* ncur, uint32_t cur_cap,
                            uint32_t cap, Seg* big, uint32_t big_cap, uint32_t* ctr,
                            unsigned long long* pts, Seg* base, uint32_t* nbase, uint32_t base_cap,
-                           Seg* wbase, uint32_t* nwbase, uint32_t wcap, Seg* tbase, uint32_t* ntbase,
-                           uint32_t tcap, Seg* bbase, uint32_t* nbbase, uint32_t cap2, uint32_t tile,
+                           Seg* wbase, uint32_t* nwbase, uint32_t wbase_cap, uint32_t wcap, Seg* tbase,
+                           uint32_t* ntbase, uint32_t tbase_cap, uint32_t tcap, Seg* bbase, uint32_t* nbbase,
+                           uint32_t bbase_cap, uint32_t cap2, uint32_t tile,
                            unsigned long long* base_pts, DevStatus* st) {
   if (pkd_failed_block(st)) return;  // uniform: before the block-wide reservations
   const RoundDyn& dy = dyn[*sel];
@@ -591,7 +592,7 @@ __global__ void k_classify(const RoundDyn* dyn, const uint32_t* sel, const uint3
       if (first[0] < big_cap) big[first[0]] = s;
     } else if (kind > 0) {
       const uint32_t b = first[kind];
-      if (b < base_cap) (kind == 1 ? base : (kind == 2 ? wbase : (kind == 3 ? tbase : bbase)))[b] = s;
+      if (b < (kind == 1 ? base_cap : (kind == 2 ? wbase_cap : (kind == 3 ? tbase_cap : bbase_cap)))) (kind == 1 ? base : (kind == 2 ? wbase : (kind == 3 ? tbase : bbase)))[b] = s;
       else set_error(st, DERR_CAPACITY, 300 + kind);
     }
   }
@@ -1575,6 +1576,194 @@ struct BuildBufs {
   RoundDyn* dyn;
 };
 
+// The lists of the base cases, by how a segment is finished: a CTA of its own
+// per SM (longer than cap2, at most cap), one of two CTAs per SM (longer than
+// wcap), a warp (longer than tcap), a warp with a small slice.
+struct BaseLists {
+  Seg *one, *two, *warp, *tiny;
+  uint32_t n_one, n_two, n_warp, n_tiny;  // entries they can hold
+  uint32_t cap, cap2, wcap, tcap;
+
+  // Room for at most `segs` segments of `extent` points together: a list of
+  // segments longer than x points has at most extent / (x + 1) of them.
+  int alloc(Scratch& sc, uint64_t extent, uint64_t segs) {
+    auto most = [&](uint32_t over) { return (uint32_t)std::min<uint64_t>(segs, extent / (over + 1) + 1); };
+    n_one = most(cap2);
+    n_two = most(wcap);
+    n_warp = most(tcap);
+    n_tiny = (uint32_t)segs;
+    PKD_TRY(sc.get(&two, n_two));
+    PKD_TRY(sc.get(&warp, n_warp));
+    PKD_TRY(sc.get(&tiny, n_tiny));
+    return sc.get(&one, n_one);
+  }
+};
+
+static BaseLists base_limits(int d) {
+  BaseLists L{};
+  L.cap = (uint32_t)base_cap_for(d);
+  L.wcap = (uint32_t)warp_cap_for(d);
+  L.tcap = 128;
+  // the presorted base case runs two CTAs per SM up to cap2 points
+  L.cap2 = knobs().base_kernel == 0 ? std::min<uint32_t>(L.cap, (uint32_t)sorted_cap_two_per_sm(d)) : L.cap;
+  return L;
+}
+
+// Every small subproblem, in shared memory, one CTA (or warp) per entry of
+// the base lists: `q` is the stream, `list_blocks(w, per, max)` the grid of
+// the list whose length is control word w.
+template <class LB, class RC>
+static int base_stage(const SmemArgs& sa, const BaseLists& L, const uint32_t* dctr, const uint32_t* hctr, int d, int nsm,
+                      cudaStream_t q, cudaStream_t aux, LB&& list_blocks, RC&& recorded) {
+  const uint64_t cta_pts = *(unsigned long long*)(hctr + C_BASE_PTS);
+  const uint64_t warp_pts = *(unsigned long long*)(hctr + C_BASE_PTS + 2);
+  const uint64_t tiny_pts = *(unsigned long long*)(hctr + C_BASE_PTS + 4);
+  for (int pass = 0; pass < 2; ++pass) {
+    SmemArgs wa = sa;
+    const int w = pass == 0 ? C_NWBASE : C_NTBASE;
+    wa.segs = pass == 0 ? L.warp : L.tiny;
+    wa.nsegs = dctr + w;
+    wa.list_cap = pass == 0 ? L.n_warp : L.n_tiny;
+    wa.cap = pass == 0 ? (int)L.wcap : (int)L.tcap;
+    const size_t smb = warp_layout(wa.cap, d).per_warp * WK_WARPS;
+    const uint32_t blocks = list_blocks(w, WK_WARPS, (uint32_t)(nsm * 8));
+    if (blocks == 0) continue;
+    KTimer kt;
+    ktimer_begin(kt, "smem_warp", pass == 0 ? warp_pts : tiny_pts, q);
+    PKD_DISPATCH_D(d, launch_smem_warp, wa, blocks, smb, q);
+    ktimer_end(kt);
+    PKD_TRY(recorded(q, w, (uint32_t)WK_WARPS, (uint32_t)(nsm * 8)));
+  }
+  KTimer kt;
+  ktimer_begin(kt, "smem_build", cta_pts, q);
+  if (knobs().base_kernel == 0) {
+    // the one-CTA-per-SM segments run beside the two-CTA launch, on a
+    // second stream, so their long CTAs do not form a tail of their own
+    SmemArgs s1 = sa;
+    s1.segs = L.one;
+    s1.nsegs = dctr + C_NBBASE;
+    s1.list_cap = L.n_one;
+    s1.cap = (int)L.cap;
+    const uint32_t b1 = list_blocks(C_NBBASE, 1, 0);
+    cudaEvent_t fork = nullptr, join = nullptr;
+    if (b1) {
+      PKD_CUDA(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming));
+      PKD_CUDA(cudaEventCreateWithFlags(&join, cudaEventDisableTiming));
+      PKD_CUDA(cudaEventRecord(fork, q));
+      PKD_CUDA(cudaStreamWaitEvent(aux, fork, 0));
+      PKD_DISPATCH_D(d, launch_smem_sorted, s1, b1, sorted_layout((int)L.cap, d).total, aux);
+      PKD_TRY(recorded(aux, C_NBBASE, 1u, 0u));
+    }
+    SmemArgs s2 = sa;
+    s2.segs = L.two;
+    s2.nsegs = dctr + C_NBASE;
+    s2.list_cap = L.n_two;
+    s2.cap = (int)L.cap2;
+    const uint32_t b2 = list_blocks(C_NBASE, 1, 0);
+    if (b2) {
+      PKD_DISPATCH_D(d, launch_smem_sorted2, s2, b2, sorted_layout((int)L.cap2, d).total, q);
+      PKD_TRY(recorded(q, C_NBASE, 1u, 0u));
+    }
+    if (b1) {
+      PKD_CUDA(cudaEventRecord(join, aux));
+      PKD_CUDA(cudaStreamWaitEvent(q, join, 0));
+      cudaEventDestroy(fork);
+      cudaEventDestroy(join);
+    }
+  } else {
+    SmemArgs s2 = sa;
+    s2.segs = L.two;
+    s2.nsegs = dctr + C_NBASE;
+    s2.list_cap = L.n_two;
+    s2.cap = (int)L.cap;
+    const uint32_t b2 = list_blocks(C_NBASE, 1, 0);
+    if (b2) {
+      PKD_DISPATCH_D(d, launch_smem_build, s2, b2, smem_layout((int)L.cap, d).total, q);
+      PKD_TRY(recorded(q, C_NBASE, 1u, 0u));
+    }
+  }
+  ktimer_end(kt);
+  return PKD_OK;
+}
+
+static void launch_classify(const RoundDyn* dyn, uint32_t* dctr, uint64_t ncur, Seg* big, uint64_t nbig, uint32_t tile,
+                            const BaseLists& L, unsigned grid, DevStatus* st, cudaStream_t s) {
+  PKD_LAUNCH(k_classify<<<grid, 256, 0, s>>>(
+      dyn, dctr + C_SEL, dctr + C_NCUR, (uint32_t)ncur, L.cap, big, (uint32_t)nbig, dctr,
+      (unsigned long long*)(dctr + C_PTS), L.two, dctr + C_NBASE, L.n_two, L.warp, dctr + C_NWBASE, L.n_warp, L.wcap, L.tiny,
+      dctr + C_NTBASE, L.n_tiny, L.tcap, L.one, dctr + C_NBBASE, L.n_one, L.cap2, tile, (unsigned long long*)(dctr + C_BASE_PTS), st));
+}
+
+// A build whose segments all fit one CTA (job.max_len <= cap): no rounds, so
+// nothing depends on a count the host has not seen.  The base cases are
+// launched directly, on grids that bound their lists' lengths, instead of
+// from a graph: recording, instantiating and destroying one for every rebuild
+// of an update (its arena positions are new each time) took about 0.5 ms of
+// host time.
+static int build_flat(TreeMem& t, const BuildJob& job, Scratch& sc) {
+  cudaStream_t s = sc.s;
+  const int d = t.p.d, nsm = num_sms();
+  const uint64_t nroots = job.dsegs ? job.dsegs_n : job.segs.size();
+  if (nroots >= 0xFFFFFFF0ull) return PKD_EINVAL;
+  uint32_t* dctr;
+  PKD_TRY(sc.get(&dctr, C_WORDS));
+  Seg* roots = const_cast<Seg*>(job.dsegs);
+  if (!roots) {
+    PKD_TRY(sc.get(&roots, std::max<uint64_t>(nroots, 1)));
+    PKD_TRY(dev_store(roots, job.segs.data(), nroots * sizeof(Seg), s));
+  }
+  BaseLists L = base_limits(d);
+  PKD_TRY(L.alloc(sc, job.extent, nroots));
+  RoundDyn* dyn;
+  PKD_TRY(sc.get(&dyn, 1));
+  Src src{};
+  if (job.input_coords) {
+    src.aos = job.input_coords;
+    src.aos_ids = job.input_ids;
+    src.is_aos = 1;
+  } else {
+    src.soa = t.A;
+  }
+  const RoundDyn hd{src, Pts{}, (int)IN_B, job.input_coords ? (int)IN_INPUT : (int)IN_A, roots, nullptr};
+  PKD_TRY(dev_store(dyn, &hd, sizeof(hd), s));
+
+  SmemArgs sa{};
+  sa.p = t.p;
+  sa.A = t.A;
+  sa.in_coords = job.input_coords;
+  sa.in_ids = job.input_ids;
+  sa.nodes = t.nodes;
+  sa.ndim = t.ndim;
+  sa.st = t.st;
+  sa.shared_cap = t.shared_cap;
+
+  PKD_LAUNCH(k_ctl_init<<<1, 64, 0, s>>>(dctr, (uint32_t)nroots));
+  const unsigned g_cls = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((nroots + 255) / 256, (uint64_t)nsm * 8));
+  launch_classify(dyn, dctr, nroots, nullptr, 0, (uint32_t)std::max(knobs().tile, 256), L, g_cls, t.st, s);
+  if (job.before_base) job.before_base(nullptr);
+  alignas(8) uint32_t hctr[C_WORDS] = {};
+  bool counted = false;
+  auto bound = [&](int w, uint32_t per, uint32_t mx) {
+    // a list of segments longer than `over` points
+    const uint32_t over = w == C_NBBASE ? L.cap2 : (w == C_NBASE ? L.wcap : (w == C_NWBASE ? L.tcap : 0));
+    if (job.max_len <= over) return 0u;
+    const uint32_t c = counted ? hctr[w] : (uint32_t)std::min<uint64_t>(nroots, job.extent / (over + 1) + 1);
+    const uint32_t b = (c + per - 1) / per;
+    return mx ? std::min(b, mx) : b;
+  };
+  // A CTA past the end of its list costs little, 1e5 of them 0.7 ms: bounds
+  // that loose are replaced by the counts (and the timers report points).
+  if (ktiming_enabled() || bound(C_NBASE, 1, 0) > 2048 || bound(C_NBBASE, 1, 0) > 2048) {
+    PKD_CUDA(cudaMemcpyAsync(hctr, dctr, sizeof(hctr), cudaMemcpyDeviceToHost, s));
+    PKD_CUDA(cudaStreamSynchronize(s));
+    counted = true;
+  }
+  auto none = [](cudaStream_t, int, uint32_t, uint32_t) { return PKD_OK; };
+  PKD_TRY(base_stage(sa, L, dctr, hctr, d, nsm, s, aux_stream(), bound, none));
+  PKD_CUDA(cudaGetLastError());
+  return PKD_OK;
+}
+
 int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
   const Params& p = t.p;
   const int d = p.d;
@@ -1586,6 +1775,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
   const uint64_t base = job.base, extent = std::max<uint64_t>(job.extent, 1);
   const int nsm = num_sms();
   Scratch sc{s, {}};
+  if (job.max_len && job.max_len <= cap && knobs().graph_rounds != 1) return build_flat(t, job, sc);
 
   // scratch point buffer B and two sample buffers over [base, base + extent)
   int32_t *bc, *s0c, *s1c;
@@ -1600,7 +1790,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
 
   uint32_t* dctr;
   PKD_TRY(sc.get(&dctr, C_WORDS));
-  PinnedBlock hblk(s);  // host copy of the control block
+  PinnedBlock hblk;  // host copy of the control block
   uint32_t* hctr = (uint32_t*)hblk.p;
   if (!hctr) return PKD_ENOMEM;
   static_assert(C_WORDS * 4 <= PINNED_BLOCK, "control block");
@@ -1615,18 +1805,10 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
     PKD_TRY(sc.get(&roots, std::max<uint64_t>(nroots, 1)));
     PKD_TRY(dev_store(roots, job.segs.data(), nroots * sizeof(Seg), s));
   }
-  const uint32_t wcap = (uint32_t)warp_cap_for(d);
   // every base segment is a root or a non-empty bucket: at most extent + roots
   const uint64_t base_cap_segs = extent + nroots + 16;
-  Seg *base_list, *wbase_list, *tbase_list, *bbase_list;
-  PKD_TRY(sc.get(&base_list, base_cap_segs));
-  PKD_TRY(sc.get(&wbase_list, base_cap_segs));
-  PKD_TRY(sc.get(&tbase_list, base_cap_segs));
-  PKD_TRY(sc.get(&bbase_list, base_cap_segs));
-  const uint32_t tcap = 128;
-  // the presorted base case runs two CTAs per SM up to cap2 points
-  const uint32_t cap2 =
-      knobs().base_kernel == 0 ? std::min<uint32_t>(cap, (uint32_t)sorted_cap_two_per_sm(d)) : cap;
+  BaseLists L = base_limits(d);
+  PKD_TRY(L.alloc(sc, extent, base_cap_segs));
 
   // worst-case round buffers
   BuildBufs bb{};
@@ -1766,7 +1948,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
   const unsigned g_jtiles = grid_for(bb.jtiles, 1, 8);
   const unsigned g_sample = grid_for(bb.tiles, 1, SAMPLE_CTAS_PER_SM);
 
-  const bool graph = knobs().graph_rounds != 0;
+  const bool graph = knobs().graph_rounds != 0;  // 1, or not set
   Flow f;
   f.dctl = dctr;
   f.hctl = hctr;
@@ -1774,11 +1956,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
   f.s = s;
 
   auto classify = [&](Flow& g) {
-    PKD_LAUNCH(k_classify<<<g_cls, 256, 0, g.s>>>(
-        bb.dyn, dctr + C_SEL, dctr + C_NCUR, (uint32_t)bb.ncur, cap, bb.big, (uint32_t)bb.nbig, dctr,
-        (unsigned long long*)(dctr + C_PTS), base_list, dctr + C_NBASE, (uint32_t)base_cap_segs, wbase_list,
-        dctr + C_NWBASE, wcap, tbase_list, dctr + C_NTBASE, tcap, bbase_list, dctr + C_NBBASE, cap2,
-        (uint32_t)TILE, (unsigned long long*)(dctr + C_BASE_PTS), t.st));
+    launch_classify(bb.dyn, dctr, bb.ncur, bb.big, bb.nbig, (uint32_t)TILE, L, g_cls, t.st, g.s);
     PKD_LAUNCH(k_round_go<<<1, 1, 0, g.s>>>(dctr, (uint32_t)bb.nbig, (uint32_t)bb.tiles, t.st));
     return PKD_OK;
   };
@@ -1847,79 +2025,6 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
     return classify(g);
   };
 
-  // 5. every small subproblem, in shared memory, one CTA (or warp) per
-  //    entry of the base lists: `q` is the stream, `list_blocks(w, per,
-  //    max)` the grid of the list whose length is control word w.
-  auto base_stage = [&](cudaStream_t q, cudaStream_t aux, auto&& list_blocks, auto&& recorded) {
-    const uint64_t cta_pts = *(unsigned long long*)(hctr + C_BASE_PTS);
-    const uint64_t warp_pts = *(unsigned long long*)(hctr + C_BASE_PTS + 2);
-    const uint64_t tiny_pts = *(unsigned long long*)(hctr + C_BASE_PTS + 4);
-    for (int pass = 0; pass < 2; ++pass) {
-      SmemArgs wa = sa;
-      const int w = pass == 0 ? C_NWBASE : C_NTBASE;
-      wa.segs = pass == 0 ? wbase_list : tbase_list;
-      wa.nsegs = dctr + w;
-      wa.list_cap = (uint32_t)base_cap_segs;
-      wa.cap = pass == 0 ? (int)wcap : (int)tcap;
-      const size_t smb = warp_layout(wa.cap, d).per_warp * WK_WARPS;
-      const uint32_t blocks = list_blocks(w, WK_WARPS, (uint32_t)(nsm * 8));
-      if (blocks == 0) continue;
-      KTimer kt;
-      ktimer_begin(kt, "smem_warp", pass == 0 ? warp_pts : tiny_pts, q);
-      PKD_DISPATCH_D(d, launch_smem_warp, wa, blocks, smb, q);
-      ktimer_end(kt);
-      PKD_TRY(recorded(q, w, (uint32_t)WK_WARPS, (uint32_t)(nsm * 8)));
-    }
-    KTimer kt;
-    ktimer_begin(kt, "smem_build", cta_pts, q);
-    if (knobs().base_kernel == 0) {
-      // the one-CTA-per-SM segments run beside the two-CTA launch, on a
-      // second stream, so their long CTAs do not form a tail of their own
-      cudaEvent_t fork = nullptr, join = nullptr;
-      PKD_CUDA(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming));
-      PKD_CUDA(cudaEventCreateWithFlags(&join, cudaEventDisableTiming));
-      PKD_CUDA(cudaEventRecord(fork, q));
-      PKD_CUDA(cudaStreamWaitEvent(aux, fork, 0));
-      SmemArgs s1 = sa;
-      s1.segs = bbase_list;
-      s1.nsegs = dctr + C_NBBASE;
-      s1.list_cap = (uint32_t)base_cap_segs;
-      s1.cap = (int)cap;
-      const uint32_t b1 = list_blocks(C_NBBASE, 1, 0);
-      if (b1) {
-        PKD_DISPATCH_D(d, launch_smem_sorted, s1, b1, sorted_layout((int)cap, d).total, aux);
-        PKD_TRY(recorded(aux, C_NBBASE, 1u, 0u));
-      }
-      SmemArgs s2 = sa;
-      s2.segs = base_list;
-      s2.nsegs = dctr + C_NBASE;
-      s2.list_cap = (uint32_t)base_cap_segs;
-      s2.cap = (int)cap2;
-      const uint32_t b2 = list_blocks(C_NBASE, 1, 0);
-      if (b2) {
-        PKD_DISPATCH_D(d, launch_smem_sorted2, s2, b2, sorted_layout((int)cap2, d).total, q);
-        PKD_TRY(recorded(q, C_NBASE, 1u, 0u));
-      }
-      PKD_CUDA(cudaEventRecord(join, aux));
-      PKD_CUDA(cudaStreamWaitEvent(q, join, 0));
-      cudaEventDestroy(fork);
-      cudaEventDestroy(join);
-    } else {
-      SmemArgs s2 = sa;
-      s2.segs = base_list;
-      s2.nsegs = dctr + C_NBASE;
-      s2.list_cap = (uint32_t)base_cap_segs;
-      s2.cap = (int)cap;
-      const uint32_t b2 = list_blocks(C_NBASE, 1, 0);
-      if (b2) {
-        PKD_DISPATCH_D(d, launch_smem_build, s2, b2, smem_layout((int)cap, d).total, q);
-        PKD_TRY(recorded(q, C_NBASE, 1u, 0u));
-      }
-    }
-    ktimer_end(kt);
-    return PKD_OK;
-  };
-
   PKD_LAUNCH(k_ctl_init<<<1, 64, 0, s>>>(dctr, (uint32_t)nroots));
   if (!graph) {
     PKD_TRY(classify(f));
@@ -1933,7 +2038,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
       return mx ? std::min(b, mx) : b;
     };
     auto none = [](cudaStream_t, int, uint32_t, uint32_t) { return PKD_OK; };
-    PKD_TRY(base_stage(s, aux_stream(), host_blocks, none));
+    PKD_TRY(base_stage(sa, L, dctr, hctr, d, nsm, s, aux_stream(), host_blocks, none));
   } else {
     // One graph: WHILE(another round) { ... WHILE(another skeleton level)
     // { ... } ... IF(exact levels) { ... } ... }, then the base cases as
@@ -1945,7 +2050,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
     if (!cs) return PKD_ECUDA;
     BaseShape* dshape;
     PKD_TRY(sc.get(&dshape, MAX_SHAPES));
-    PinnedBlock shblk(s);
+    PinnedBlock shblk;
     if (!shblk.p) return PKD_ENOMEM;
     static_assert(MAX_SHAPES * sizeof(BaseShape) <= PINNED_BLOCK, "shape block");
     BaseShape* hshape = (BaseShape*)shblk.p;
@@ -1965,7 +2070,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
       put((uint64_t)p.d), put((uint64_t)p.phi), put((uint64_t)p.lambda), put((uint64_t)p.sigma_log2);
       put((uint64_t)p.sigma_os), put((uint64_t)p.count_mode), put((uint64_t)p.alpha_num), put((uint64_t)p.alpha_den);
       put(p.seed);
-      put((uint64_t)TILE), put(cap), put((uint64_t)scap), put(cap2), put(wcap), put((uint64_t)nsm);
+      put((uint64_t)TILE), put(cap), put((uint64_t)scap), put(L.cap2), put(L.wcap), put((uint64_t)nsm);
       put((uint64_t)knobs().sieve_kernel), put((uint64_t)knobs().base_kernel), put((uint64_t)knobs().wait_cycles);
       put((uint64_t)record_buckets(NB));
     }
@@ -2014,7 +2119,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
       ++nshape;
       return PKD_OK;
     };
-    if (e == PKD_OK) e = base_stage(cs, aux_stream(), dev_blocks, record_shape);
+    if (e == PKD_OK) e = base_stage(sa, L, dctr, hctr, d, nsm, cs, aux_stream(), dev_blocks, record_shape);
     flow_capturing() = false;
     cudaGraph_t graph_h = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(cs, &graph_h);

@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <functional>
 #include <string>
 #include <vector>
@@ -23,8 +24,9 @@ struct Knobs {
   int base_kernel = 0;  // base case: 0 presorted lists, 1 radix select per node
   int sieve_kernel = 0;  // sieve: 0 persistent with bulk copies and recorded
                          // buckets, 2 persistent re-walking, 1 one tile per CTA
-  int graph_rounds = 1;  // build rounds: 1 decided on the device (one CUDA graph
-                         // with conditional nodes), 0 sequenced by the host
+  int graph_rounds = -1;  // build rounds: 1 decided on the device (one CUDA graph
+                          // with conditional nodes), 0 sequenced by the host,
+                          // -1 (not set) a graph when there can be rounds
   long long front_cap = 0;  // > 0: first capacity of an update's flatten lists (testing)
 };
 Knobs& knobs();
@@ -165,18 +167,42 @@ void dfree(T*& p, cudaStream_t s) {
   p = nullptr;
 }
 
-// Scratch buffers of one call, freed in stream order when it returns.
+// Scratch buffers of one call, freed in stream order when it returns.  Small
+// buffers are cut from blocks of BLOCK bytes: an update asks for a few hundred
+// of them, at about 1.5 us of host time each when every one was an allocation.
 struct Scratch {
+  static constexpr size_t BLOCK = 256 << 10;
   cudaStream_t s;
-  std::vector<void*> ptrs;
+  std::vector<void*> ptrs;   // every buffer handed out, in order
+  std::vector<void*> owned;  // what has to be freed
+  char* cur = nullptr;
+  size_t left = 0;
   ~Scratch() {
-    for (void* p : ptrs) cudaFreeAsync(p, s);
+    for (void* p : owned) cudaFreeAsync(p, s);
   }
   template <class T>
   int get(T** p, size_t n) {
-    int e = dalloc(p, n, s);
-    if (e == PKD_OK) ptrs.push_back(*p);
-    return e;
+    *p = nullptr;
+    const size_t bytes = (std::max<size_t>(n, 1) * sizeof(T) + 255) & ~(size_t)255;
+    char* q = nullptr;
+    if (bytes > BLOCK / 4) {
+      const int e = dalloc(&q, bytes, s);
+      if (e != PKD_OK) return e;
+      owned.push_back(q);
+    } else {
+      if (left < bytes) {
+        const int e = dalloc(&cur, BLOCK, s);
+        left = e == PKD_OK ? BLOCK : 0;
+        if (e != PKD_OK) return e;
+        owned.push_back(cur);
+      }
+      q = cur;
+      cur += bytes;
+      left -= bytes;
+    }
+    *p = (T*)q;
+    ptrs.push_back(q);
+    return PKD_OK;
   }
 };
 
@@ -186,16 +212,15 @@ struct Scratch {
 constexpr size_t PINNED_BLOCK = 256;
 void* pinned_get();
 void pinned_put(void* p);
-// Return a block once the work queued on `s` so far has completed (a copy
-// into it may still be in flight).
-void pinned_put_after(cudaStream_t s, void* p);
 
-// A pinned block of PINNED_BLOCK bytes owned by one scope.
+// A pinned block of PINNED_BLOCK bytes owned by one scope.  Whoever lets the
+// device write to it waits for that write before the scope ends: the block
+// goes straight back to the pool.  (Handing it back by a host function queued
+// on the stream held the stream for about 25 us, twice in a build.)
 struct PinnedBlock {
   void* p = nullptr;
-  cudaStream_t s = nullptr;
-  explicit PinnedBlock(cudaStream_t st) : p(pinned_get()), s(st) {}
-  ~PinnedBlock() { pinned_put_after(s, p); }
+  PinnedBlock() : p(pinned_get()) {}
+  ~PinnedBlock() { pinned_put(p); }
   PinnedBlock(const PinnedBlock&) = delete;
   PinnedBlock& operator=(const PinnedBlock&) = delete;
 };
@@ -234,6 +259,7 @@ struct BuildJob {
   std::vector<Seg> segs;   // host list of root segments, or:
   const Seg* dsegs = nullptr;  // device list of root segments (dsegs_n of them)
   uint64_t dsegs_n = 0;
+  uint64_t max_len = 0;    // longest segment, when the caller knows it (0: unknown)
   // Called once on the host when the shared-memory base cases have been
   // queued or recorded (work that should overlap them, which are bound by
   // instruction issue rather than memory traffic, is queued from here).  The

@@ -497,7 +497,7 @@ int pkd_range_report(const pkd_tree* tc, const int32_t* lo, const int32_t* hi, u
   uint64_t *counts, *partial = nullptr;
   PKD_TRY_(sc.get(&counts, q));
   if (nb > 1) PKD_TRY_(sc.get(&partial, nb + 1));
-  PinnedBlock tot(s);
+  PinnedBlock tot;
   if (!tot.p) return PKD_ENOMEM;
   const QueryArgs a = range_args(t, check, lo, hi, q);
   PKD_TRY_(range_counts(t, a, counts, s));

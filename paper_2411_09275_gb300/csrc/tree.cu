@@ -342,17 +342,6 @@ void pinned_put(void* p) {
   g_pin_free.push_back(p);
 }
 
-static void CUDART_CB pinned_put_cb(void* p) { pinned_put(p); }
-
-void pinned_put_after(cudaStream_t s, void* p) {
-  if (!p) return;
-  if (cudaLaunchHostFunc(s, pinned_put_cb, p) != cudaSuccess) {
-    cudaGetLastError();
-    cudaStreamSynchronize(s);
-    pinned_put(p);
-  }
-}
-
 void tree_release(TreeMem& t) {
   cudaStream_t s = 0;
   for (void* p : {(void*)t.A.c, (void*)t.A.id, (void*)t.nodes, (void*)t.ndim, (void*)t.shared_next, (void*)t.st})
@@ -364,7 +353,7 @@ void tree_release(TreeMem& t) {
   big_free_zeroed(t.aux, clean ? t.node_cap * 4 : 0, s);
   ids_release(t.ids, s);
   big_free(t.bbox, s);
-  pinned_put_after(s, t.st_host);
+  pinned_put(t.st_host);  // every copy into it has been waited for
   t = TreeMem{};
 }
 
@@ -653,6 +642,7 @@ int pkd_build(const int32_t* coords, const uint32_t* ids, uint64_t n, const pkd_
   job.base = 0;
   job.extent = std::max<uint64_t>(n, 1);
   job.segs.push_back(Seg{0, (uint32_t)n, 0, 0, IN_INPUT});
+  job.max_len = n;
   trace_mark(s, "build: alloc tree");
   e = run_build(t->m, job, s);
   trace_mark(s, "build: run_build");

@@ -88,6 +88,8 @@ struct UpdArgs {
   RebuildItem* items_out;
   uint32_t* nitems_out;
   unsigned long long* items_total;
+  uint32_t* items_max;  // the largest of them
+  unsigned long long* inner_total;  // stored points (before the update) of the rebuilt interior nodes
   uint32_t items_cap;
   uint32_t* aux;  // [node slot] deleted points below (delete only)
   DevStatus* st;
@@ -610,7 +612,7 @@ __global__ void __launch_bounds__(ITEM_WARPS * 32) k_aggregate(UpdArgs a) {
   }
 }
 
-__device__ void push_rebuild(const UpdArgs& a, uint32_t slot, uint32_t depth, uint32_t size,
+__device__ void push_rebuild(const UpdArgs& a, uint32_t slot, uint32_t depth, uint32_t size, uint32_t old,
                              uint32_t old_live, uint64_t ws, uint64_t we) {
   const uint32_t k = atomicAdd(a.nitems_out, 1u);
   if (k >= a.items_cap) {
@@ -619,6 +621,8 @@ __device__ void push_rebuild(const UpdArgs& a, uint32_t slot, uint32_t depth, ui
   }
   a.items_out[k] = RebuildItem{slot, depth, size, old_live, ws, we, 0};
   atomicAdd(a.items_total, (unsigned long long)size);
+  atomicAdd(a.inner_total, (unsigned long long)old);
+  atomicMax(a.items_max, size);
 }
 
 // Top-down alpha test over every skeleton (rounds in forward order; within a
@@ -718,7 +722,7 @@ __global__ void __launch_bounds__(ITEM_WARPS * 32) k_decide(UpdArgs a) {
       const uint64_t kl = (uint64_t)i * a.NB + sk_bucket(sk[lv].y);
       const uint64_t kr = (uint64_t)i * a.NB + sk_bucket(sk[rv].y);
       const uint32_t depth = it.depth + (31 - __clz(v));
-      push_rebuild(a, slot, depth, N, a.insert ? old : old - c, a.bstart[kl], a.bstart[kr] + a.blen[kr]);
+      push_rebuild(a, slot, depth, N, old, a.insert ? old : old - c, a.bstart[kl], a.bstart[kr] + a.blen[kr]);
       atomicOr(&under[c0 >> 5], 3u << (c0 & 31));
     }
     __syncwarp();
@@ -755,6 +759,8 @@ __global__ void k_leaf_items(UpdArgs a, LeafGroup* groups, const uint32_t* ngrou
   const unsigned long long tv[1] = {push ? (unsigned long long)it.size : 0ull};
   unsigned long long* const tc[1] = {a.items_total};
   block_add64<1>(tv, tc);
+  const uint32_t mx = __reduce_max_sync(FULL_MASK, push ? it.size : 0u);
+  if (mx && lane_id() == 0) atomicMax(a.items_max, mx);
   const uint32_t bp = first[0], bc = first[1];
   if (push) {
     if (bp < a.items_cap) a.items_out[bp] = it;
@@ -1342,7 +1348,7 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
   uint32_t* dctr;
   PKD_TRY(sc.get(&dctr, 32));
   PKD_TRY(dev_fill(dctr, 0, 32 * 4, s));
-  PinnedBlock hblk(s);  // 128 bytes of host counters
+  PinnedBlock hblk;  // 128 bytes of host counters
   uint32_t* hctr = (uint32_t*)hblk.p;
   if (!hctr) return PKD_ENOMEM;
   uint32_t* d_ngroups = dctr + 4;
@@ -1373,6 +1379,8 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
   ua.items_out = items_out;
   ua.nitems_out = d_nitems;
   ua.items_total = d_total;
+  ua.items_max = dctr + 9;
+  ua.inner_total = (unsigned long long*)(dctr + 10);
   ua.items_cap = items_cap;
   ua.aux = t.aux;
   ua.st = t.st;
@@ -1593,11 +1601,12 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
   }
   trace_mark(s, "upd: match+count+decide");
   if (ngroups) PKD_LAUNCH(k_leaf_items<<<(ngroups + 255) / 256, 256, 0, s>>>(ua, groups, d_ngroups, compact, d_ncompact));
-  PKD_CUDA(cudaMemcpyAsync(hctr, dctr, 40, cudaMemcpyDeviceToHost, s));
+  PKD_CUDA(cudaMemcpyAsync(hctr, dctr, 48, cudaMemcpyDeviceToHost, s));
   PKD_CUDA(cudaStreamSynchronize(s));
   const uint32_t nitems = hctr[5];
   const uint64_t total = *(unsigned long long*)(hctr + 6);
   const uint32_t ncompact = hctr[8];
+  const uint64_t inner_total = *(unsigned long long*)(hctr + 10);
   stat_items(insert ? "rebuilt_insert" : "rebuilt_delete", total);
   trace_mark(s, "upd: leaf items");
 
@@ -1622,13 +1631,13 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
     PKD_TRY(sc.get(&saved_dims, nitems));
     PKD_TRY(sc.get(&saved_next, 1));
     // Capacity of the flatten's lists: every node of the old subtrees
-    // appears once.  A subtree of P stored points has at most 2P - 1 nodes
-    // unless deletes left empty leaves in it, so the first attempt is sized
-    // by the stored points of the rebuilt subtrees (at most their new sizes
-    // plus the points this batch deleted); when a level overflows it, the
-    // flatten is redone with four entries per stored point of the tree.
+    // appears once: a leaf item is one node, an interior item of P stored
+    // points has at most 2P - 1 nodes unless deletes left empty leaves in it.
+    // The first attempt is sized by that (an insert's items are mostly
+    // leaves); when a level overflows it, the flatten is redone with four
+    // entries per stored point of the tree.
     const uint64_t big_fcap = 4 * ((uint64_t)t.size + (uint64_t)nitems) + 1024;
-    uint64_t fcap = 2 * (total + (insert ? 0ull : (uint64_t)total_changed) + (uint64_t)nitems) + 1024;
+    uint64_t fcap = 2 * inner_total + (uint64_t)nitems + 1024;
     if (knobs().front_cap > 0) fcap = (uint64_t)knobs().front_cap;
     fcap = std::max<uint64_t>(std::min(fcap, big_fcap), (uint64_t)nitems + 1024);  // the roots always fit
     Front *fa = nullptr, *fb = nullptr, *leaves = nullptr, *bigleaves = nullptr;
@@ -1706,6 +1715,7 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
     job.extent = std::max<uint64_t>(total, 1);
     job.dsegs = segs;
     job.dsegs_n = nitems;
+    job.max_len = hctr[9];
     const int eb = run_build(t, job, s);
     if (eb != PKD_OK) {
       PKD_LAUNCH(k_restore_roots<<<gi, 128, 0, s>>>(items_out, d_nitems, t.nodes, t.ndim, saved_nodes, saved_dims));
@@ -1802,7 +1812,7 @@ int pkd_batch_delete(pkd_tree* tc, const uint32_t* ids, uint64_t m, uint64_t* n_
   PKD_TRY(dev_fill(cnt, 0, 4, s));
   Pts W{wc, wid, m};
   ids_take(t, ids, m, W, wslots, cnt, s);
-  PinnedBlock hb(s);
+  PinnedBlock hb;
   if (!hb.p) return PKD_ENOMEM;
   PKD_CUDA(cudaMemcpyAsync(hb.p, cnt, 4, cudaMemcpyDeviceToHost, s));
   int fl = 0;
