@@ -1,21 +1,13 @@
 // Batch updates of a Pkd-tree: BatchInsert (Alg. 2, Sec. 4.1) and the
 // two-round BatchDelete (Sec. 4.2).
 //
-//  route    the batch is sieved through the tree lambda levels at a time: the
-//           "skeleton at T" is fetched from the existing nodes (cut at
-//           leaves), and the same count / scan / scatter kernels as the build
-//           move every batch point to its external node.  Internal external
-//           nodes become the next round's items; leaves collect "leaf groups".
-//  match    (delete only) every stored point of a reached leaf is compared
-//           with the batch points routed there; matches are marked dead and
-//           points that match nothing are discarded (round 1 of Sec. 4.2).
-//  count    exact per-node counts of inserted / deleted points, aggregated
-//           bottom-up over the recorded skeletons.
-//  decide   top-down over every skeleton: a node that receives updates stays
-//           (its size is rewritten in place) when it is still alpha-balanced,
-//           otherwise it is rebuilt with Build on all its (live) points plus
-//           the new ones, and nothing below it is looked at.  A reached leaf
-//           is rebuilt (insert: Build(leaf + new)) or compacted (delete).
+//  route    the batch goes down the tree lambda levels a round (route.cuh); on
+//           the way a node that receives updates stays (its new size is
+//           recorded) when it is still alpha-balanced, otherwise it is rebuilt
+//           with Build on all its (live) points plus the new ones.  A reached
+//           leaf is rebuilt (insert: Build(leaf + new)) or compacted (delete).
+//  delete   every stored point of a reached leaf is compared with the batch
+//           points routed there; the matches go (round 1 of Sec. 4.2).
 //  rebuild  old subtrees are flattened by a parallel breadth-first walk into
 //           fresh arena ranges, new points appended, and every rebuild item
 //           becomes a root segment of one multi-segment build (build.cu).
@@ -23,400 +15,11 @@
 #include <cstdio>
 #include <vector>
 
-#include "sieve_tma.cuh"
+#include "query.cuh"
+#include "route.cuh"
 #include "tree_impl.hpp"
 
 namespace pkd {
-
-constexpr uint32_t LINK_NONE = 0xFFFFFFFFu;
-constexpr uint32_t LINK_LEAF = 0x80000000u;
-
-struct LeafGroup {
-  uint32_t slot;   // the leaf's node slot
-  uint32_t depth;  // its tree depth
-  uint64_t start;  // first routed batch point (position in the batch buffers)
-  uint32_t len;    // routed batch points
-  uint32_t found;  // insert: len; delete: stored points removed
-  uint32_t flag;   // 1: inside a subtree that is rebuilt
-  uint32_t pad;
-};
-
-struct RebuildItem {
-  uint32_t slot;
-  uint32_t depth;
-  uint32_t size;    // points after the update
-  uint32_t old_live;
-  uint64_t ws, we;  // batch points (insert) in the final batch buffer
-  uint64_t pos;     // arena position assigned
-};
-
-struct UpdArgs {
-  Params p;
-  int lam, NB, HN, TILE;
-  int insert;
-  const Node* nodes;
-  const uint8_t* ndim;
-  // this round
-  const Seg* items;
-  const uint32_t* nitems;
-  int2* skel;
-  uint32_t* slots;
-  uint32_t* nbk;
-  const uint32_t* tile0;
-  const uint32_t* hscan;
-  uint64_t* bstart;  // [item][NB]
-  uint32_t* blen;    // [item][NB]
-  uint32_t* link;    // [item][NB]
-  uint32_t* fnd;     // [item][HN]
-  uint32_t* nsz;     // [item][HN] new size of a node that stays, or ~0 (applied at the end)
-  uint32_t* iflag;   // [item]
-  // next round
-  Seg* next;
-  uint32_t* next_ctr;  // [0] items, [1] tiles of big items, [2] big items, [3] small items,
-                       // [16] points of the big items
-  Seg* next_big;       // big items (more than SMALL_ITEM points) and their item index
-  uint32_t* next_bigmap;
-  uint32_t* next_small;  // item index of the small items
-  uint32_t* next_iflag;
-  const uint32_t* next_fnd;  // found counts of the next round (aggregation)
-  int next_HN;
-  // leaf groups
-  LeafGroup* groups;
-  uint32_t* ngroups;
-  uint32_t group_cap;
-  // rebuild items
-  RebuildItem* items_out;
-  uint32_t* nitems_out;
-  unsigned long long* items_total;
-  uint32_t* items_max;  // the largest of them
-  unsigned long long* inner_total;  // stored points (before the update) of the rebuilt interior nodes
-  uint32_t items_cap;
-  uint32_t* aux;  // [node slot] deleted points below (delete only)
-  DevStatus* st;
-};
-
-// The per-item kernels (fetch, emit, aggregate, decide) give each item one
-// warp, whose lanes take the heap entries of one skeleton level at a time
-// (levels are ordered by __syncwarp); each CTA holds ITEM_WARPS items.
-constexpr int ITEM_WARPS = 4;
-__host__ __device__ inline unsigned item_blocks(uint64_t n) { return (unsigned)((n + ITEM_WARPS - 1) / ITEM_WARPS); }
-__device__ __forceinline__ uint32_t item_of_warp() { return blockIdx.x * ITEM_WARPS + warp_id(); }
-
-// The skeleton at each item: its node and lambda levels below, cut at leaves;
-// the external nodes are numbered left to right (the item's buckets).
-// The skeleton is assembled in shared memory (one level's node loads in
-// flight at a time, both of a node's records at once) and written out at
-// the end.
-__global__ void __launch_bounds__(ITEM_WARPS * 32) k_fetch(UpdArgs a) {
-  extern __shared__ __align__(16) uint8_t fetch_sm[];
-  __shared__ uint32_t bits_sh[ITEM_WARPS][32], pre_sh[ITEM_WARPS][32];
-  const uint32_t i = item_of_warp();
-  if (i >= *a.nitems) return;  // warp-uniform
-  const int lane = lane_id();
-  uint32_t* bits = bits_sh[warp_id()];
-  uint32_t* pre = pre_sh[warp_id()];
-  int2* sk = reinterpret_cast<int2*>(fetch_sm) + (size_t)warp_id() * a.HN;
-  uint32_t* sl = reinterpret_cast<uint32_t*>(reinterpret_cast<int2*>(fetch_sm) + (size_t)ITEM_WARPS * a.HN) +
-                 (size_t)warp_id() * a.HN;
-  for (int v = lane; v < a.HN; v += 32) {
-    sk[v] = make_int2(0, sk_meta(SK_NONE, 0, 0));
-    sl[v] = 0xFFFFFFFFu;
-  }
-  bits[lane] = 0;
-  __syncwarp();
-  if (lane == 0) {
-    sl[1] = a.items[i].root;
-    sk[1] = make_int2(0, sk_meta(SK_BUCKET, 0, 0));  // provisional: marks "defined"
-  }
-  __syncwarp();
-  for (int j = 0; j <= a.lam; ++j) {
-    for (int v = (1 << j) + lane; v < (2 << j); v += 32) {
-      if (sk_state(sk[v].y) == SK_NONE) continue;
-      const uint32_t slot = sl[v];
-      uint8_t dm = (uint8_t)PKD_LEAF;
-      Node nd{};
-      if (j < a.lam) {  // both loads issued together
-        dm = a.ndim[slot];
-        nd = a.nodes[slot];
-      }
-      if (dm == PKD_LEAF) {
-        // external: bit (its first position on level lambda) in the bitmap
-        const uint32_t lo = (uint32_t)(v - (1 << j)) << (a.lam - j);
-        atomicOr(&bits[lo >> 5], 1u << (lo & 31));
-        continue;
-      }
-      sk[v] = make_int2(nd.split, sk_meta(SK_INTERNAL, dm, 0));
-      sl[2 * v] = nd.a;
-      sl[2 * v + 1] = nd.b;
-      sk[2 * v] = make_int2(0, sk_meta(SK_BUCKET, 0, 0));
-      sk[2 * v + 1] = make_int2(0, sk_meta(SK_BUCKET, 0, 0));
-    }
-    __syncwarp();
-  }
-  // left-to-right number of an external node = set bits before its position
-  const uint32_t wc = (uint32_t)__popc(bits[lane]);
-  const uint32_t incl = (uint32_t)warp_incl_scan((int)wc);
-  pre[lane] = incl - wc;
-  __syncwarp();
-  for (int j = 0; j <= a.lam; ++j) {
-    for (int v = (1 << j) + lane; v < (2 << j); v += 32) {
-      if (sk_state(sk[v].y) != SK_BUCKET) continue;
-      const uint32_t lo = (uint32_t)(v - (1 << j)) << (a.lam - j);
-      const uint32_t nbk = pre[lo >> 5] + (uint32_t)__popc(bits[lo >> 5] & ((1u << (lo & 31)) - 1u));
-      sk[v].y = sk_meta(SK_BUCKET, 0, (int)nbk);
-    }
-  }
-  __syncwarp();
-  int2* gsk = a.skel + (uint64_t)i * a.HN;
-  uint32_t* gsl = a.slots + (uint64_t)i * a.HN;
-  for (int v = lane; v < a.HN; v += 32) {
-    gsk[v] = sk[v];
-    gsl[v] = sl[v];
-  }
-  if (lane == 31) a.nbk[i] = incl;
-}
-
-constexpr uint32_t SMALL_ITEM = 256;  // items up to this many points: one warp routes them
-
-// Bucket ranges of the big items from the bucket-major scan of the tile
-// histograms: one warp per item, its lanes over the buckets.
-__global__ void k_bucket_ranges(RoundArgs r, uint64_t* bstart, uint32_t* blen, const uint32_t* nbk) {
-  if (pkd_failed_block(r.st)) return;
-  const uint32_t s = (uint32_t)(((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  if (s >= *r.nbig) return;  // warp-uniform
-  const Seg it = r.big[s];
-  const uint32_t k = r.skel_map[s];
-  const uint32_t nb = nbk[k];
-  const uint32_t nt = (it.len + r.TILE - 1) / r.TILE;
-  const uint64_t hb = (uint64_t)r.tile0[s] * r.NB;
-  const uint32_t base = r.hscan[hb];
-  for (uint32_t b = lane_id(); b < (uint32_t)r.NB; b += 32) {
-    uint32_t b0 = it.len, b1 = it.len;
-    if (b < nb) {
-      b0 = r.hscan[hb + (uint64_t)b * nt] - base;
-      b1 = (b + 1 < nb) ? r.hscan[hb + (uint64_t)(b + 1) * nt] - base : it.len;
-    }
-    bstart[(uint64_t)k * r.NB + b] = it.start + b0;
-    blen[(uint64_t)k * r.NB + b] = b1 - b0;
-  }
-}
-
-// Small items: one warp walks every point through the item's skeleton,
-// counts and ranks the buckets in shared memory, and scatters the item in
-// one pass (no global histogram: the warp owns the whole item).  Points
-// also go to the final batch buffer F (see k_copy_round).
-template <int D>
-__global__ void __launch_bounds__(256, (D <= 3 ? 6 : 1)) k_route_small(RoundArgs r, const uint32_t* small, const uint32_t* nsmall,
-                                                     const Seg* items, const uint32_t* nbk, uint64_t* bstart,
-                                                     uint32_t* blen, Pts F) {
-  if (pkd_failed_block(r.st)) return;
-  extern __shared__ unsigned cnt_sm[];
-  const uint32_t gw = blockIdx.x * (blockDim.x / 32) + warp_id();
-  if (gw >= *nsmall) return;  // warp-uniform
-  unsigned* cnt = cnt_sm + (size_t)warp_id() * r.NB;
-  const uint32_t k = small[gw];
-  const Seg it = items[k];
-  const int2* sk = r.skel + (uint64_t)k * r.HN;
-  const uint32_t nb = nbk[k];
-  for (int b = lane_id(); b < r.NB; b += 32) cnt[b] = 0;
-  __syncwarp();
-  constexpr int PER = SMALL_ITEM / 32;
-  int32_t x[PER][D];
-  uint32_t id[PER];
-  int bk[PER], rk[PER];
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const uint32_t i = q * 32 + lane_id();
-    bk[q] = -1;
-    rk[q] = 0;
-    if (i < it.len) {
-      const uint64_t g = it.start + i;
-#pragma unroll
-      for (int j = 0; j < D; ++j) x[q][j] = r.src.x(D, j, g);
-      id[q] = r.src.id(g);
-      int h = 1;
-      for (int l = 0; l < r.lam; ++l) {
-        const int2 e = sk[h];
-        if (sk_state(e.y) != SK_INTERNAL) break;
-        h = 2 * h + (x[q][sk_dim(e.y)] >= e.x);
-      }
-      bk[q] = sk_bucket(sk[h].y);
-    }
-    const unsigned m = peer_mask(bk[q], r.lam);
-    const int leader = __ffs(m) - 1;
-    unsigned b0 = 0;
-    if (bk[q] >= 0 && lane_id() == leader) b0 = atomicAdd(&cnt[bk[q]], (unsigned)__popc(m));
-    rk[q] = (int)__shfl_sync(FULL_MASK, b0, leader) + __popc(m & lanemask_lt());
-  }
-  __syncwarp();
-  // bucket starts: exclusive scan of the counts, 32 buckets at a time
-  unsigned carry = 0;
-  for (int b0 = 0; b0 < r.NB; b0 += 32) {
-    const int b = b0 + lane_id();
-    const unsigned c = b < r.NB ? cnt[b] : 0;
-    const unsigned incl = (unsigned)warp_incl_scan((int)c);
-    if (b < r.NB) {
-      const uint64_t o = (uint64_t)k * r.NB + b;
-      bstart[o] = it.start + carry + incl - c;
-      blen[o] = (uint32_t)b < nb ? c : 0;
-    }
-    __syncwarp();
-    if (b < r.NB) cnt[b] = carry + incl - c;
-    carry += __shfl_sync(FULL_MASK, incl, 31);
-  }
-  __syncwarp();
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    if (bk[q] < 0) continue;
-    const uint64_t g = it.start + cnt[bk[q]] + (uint32_t)rk[q];
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-      r.dst.c[(uint64_t)j * r.dst.stride + g] = x[q][j];
-      F.c[(uint64_t)j * F.stride + g] = x[q][j];
-    }
-    r.dst.id[g] = id[q];
-    F.id[g] = id[q];
-  }
-}
-
-template <int D>
-static void launch_route_small(const RoundArgs& ra, const uint32_t* small, const uint32_t* nsmall, const Seg* items,
-                               const uint32_t* nbk, uint64_t* bstart, uint32_t* blen, Pts F, uint32_t n,
-                               cudaStream_t s) {
-  const size_t smb = (size_t)8 * ra.NB * 4;
-  PKD_LAUNCH(k_route_small<D><<<(n + 7) / 8, 256, smb, s>>>(ra, small, nsmall, items, nbk, bstart, blen, F));
-}
-
-// Next-round items and leaf groups from the bucket ranges.  Each lane takes
-// EMIT_PER heap positions at a time (v = v0 + 32u + lane): the loads of all
-// of them are issued before the first counter update, and the warp reserves
-// its outputs with one atomic per counter for all of them (warp scans give
-// each lane its offsets).
-constexpr int EMIT_PER = 4;
-__global__ void __launch_bounds__(ITEM_WARPS * 32) k_route_emit(UpdArgs a) {
-  if (pkd_failed_block(a.st)) return;
-  const uint32_t i = item_of_warp();
-  if (i >= *a.nitems) return;  // warp-uniform
-  const int lane = lane_id();
-  const Seg it = a.items[i];
-  const int2* sk = a.skel + (uint64_t)i * a.HN;
-  const uint32_t* sl = a.slots + (uint64_t)i * a.HN;
-  const uint64_t kb0 = (uint64_t)i * a.NB;
-  for (int b = lane; b < a.NB; b += 32) a.link[kb0 + b] = LINK_NONE;
-  __syncwarp();
-  for (int v0 = 1; v0 < a.HN; v0 += 32 * EMIT_PER) {
-    int bkt[EMIT_PER];
-#pragma unroll
-    for (int u = 0; u < EMIT_PER; ++u) {
-      const int v = v0 + 32 * u + lane;
-      bkt[u] = -1;
-      if (v < a.HN) {
-        const int m = sk[v].y;
-        if (sk_state(m) == SK_BUCKET) bkt[u] = sk_bucket(m);
-      }
-    }
-    uint32_t cnt[EMIT_PER], slot[EMIT_PER];
-    uint64_t b0[EMIT_PER];
-#pragma unroll
-    for (int u = 0; u < EMIT_PER; ++u) {
-      cnt[u] = 0;
-      slot[u] = 0;
-      b0[u] = 0;
-      if (bkt[u] >= 0) {
-        cnt[u] = a.blen[kb0 + bkt[u]];
-        b0[u] = a.bstart[kb0 + bkt[u]];
-        slot[u] = sl[v0 + 32 * u + lane];
-      }
-    }
-    bool leaf[EMIT_PER], big[EMIT_PER];
-    uint32_t nL = 0, nN = 0, nB = 0, tiles = 0, bigpts = 0;
-#pragma unroll
-    for (int u = 0; u < EMIT_PER; ++u) {
-      const bool reached = cnt[u] != 0;
-      leaf[u] = reached && a.ndim[slot[u]] == PKD_LEAF;
-      const bool inner = reached && !leaf[u];
-      big[u] = inner && cnt[u] > SMALL_ITEM;
-      nL += leaf[u];
-      nN += inner;
-      nB += big[u];
-      if (big[u]) {
-        tiles += (cnt[u] + a.TILE - 1) / a.TILE;
-        bigpts += cnt[u];
-      }
-    }
-    // one update of each counter per warp and batch
-    const uint32_t iL = (uint32_t)warp_incl_scan((int)nL);
-    const uint32_t iN = (uint32_t)warp_incl_scan((int)nN);
-    const uint32_t iB = (uint32_t)warp_incl_scan((int)nB);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      tiles += __shfl_xor_sync(FULL_MASK, tiles, o);
-      bigpts += __shfl_xor_sync(FULL_MASK, bigpts, o);
-    }
-    const uint32_t tL = __shfl_sync(FULL_MASK, iL, 31), tN = __shfl_sync(FULL_MASK, iN, 31);
-    const uint32_t tB = __shfl_sync(FULL_MASK, iB, 31);
-    uint32_t gB = 0, qB = 0, kB = 0, sB = 0;
-    if (lane == 0) {
-      if (tL) gB = atomicAdd(a.ngroups, tL);
-      if (tN) qB = atomicAdd(&a.next_ctr[0], tN);
-      if (tB) {
-        kB = atomicAdd(&a.next_ctr[2], tB);
-        atomicAdd(&a.next_ctr[1], tiles);
-        atomicAdd(&a.next_ctr[16], bigpts);
-      }
-      if (tN > tB) sB = atomicAdd(&a.next_ctr[3], tN - tB);
-    }
-    uint32_t g = __shfl_sync(FULL_MASK, gB, 0) + iL - nL;
-    uint32_t q = __shfl_sync(FULL_MASK, qB, 0) + iN - nN;
-    uint32_t kb = __shfl_sync(FULL_MASK, kB, 0) + iB - nB;
-    uint32_t sb = __shfl_sync(FULL_MASK, sB, 0) + (iN - iB) - (nN - nB);
-#pragma unroll
-    for (int u = 0; u < EMIT_PER; ++u) {
-      if (!cnt[u]) continue;
-      const int v = v0 + 32 * u + lane;
-      const uint64_t k = kb0 + bkt[u];
-      const uint32_t depth = it.depth + (31 - __clz(v));
-      if (leaf[u]) {
-        if (g >= a.group_cap) {
-          set_error(a.st, DERR_CAPACITY, 800);
-        } else {
-          a.groups[g] = LeafGroup{slot[u], depth, b0[u], cnt[u], a.insert ? cnt[u] : 0u, 0u, 0u};
-          a.link[k] = LINK_LEAF | g;
-        }
-        ++g;
-        continue;
-      }
-      const Seg c{b0[u], cnt[u], depth, slot[u], IN_B};
-      a.next[q] = c;
-      if (big[u]) {
-        a.next_big[kb] = c;
-        a.next_bigmap[kb] = q;
-        ++kb;
-      } else {
-        a.next_small[sb] = q;
-        ++sb;
-      }
-      a.link[k] = q;
-      ++q;
-    }
-  }
-}
-
-// Copy every point this round moved into the final batch buffer F.  Points
-// that go on to a deeper round are overwritten there later, so F ends with
-// every point at its final position (the points of a leaf group are never
-// moved again).  Same tiling as the sieve kernels: one block per tile.
-__global__ void k_copy_round(RoundArgs r, Pts F) {
-  if (pkd_failed_block(r.st)) return;
-  SieveTile t;
-  if (!sieve_tile(r, t, blockIdx.x)) return;
-  const int d = r.p.d;
-  for (int i = threadIdx.x; i < t.cnt; i += blockDim.x) {
-    const uint64_t p = t.seg.start + t.first + (uint64_t)i;
-    for (int j = 0; j < d; ++j) F.c[(uint64_t)j * F.stride + p] = r.dst.c[(uint64_t)j * r.dst.stride + p];
-    F.id[p] = r.dst.id[p];
-  }
-}
 
 // The per-leaf kernels below give each warp UPW leaves (or rebuild items):
 // lanes 0..UPW-1 fetch the descriptors together, and for leaves of at most
@@ -429,16 +32,22 @@ __host__ __device__ inline unsigned upw_blocks(uint32_t n) {
   return (unsigned)(((uint64_t)n + UPW * UPW_WARPS - 1) / (UPW * UPW_WARPS));
 }
 
-// Deletion round 1 at the leaves: mark stored points equal to a routed batch
-// point (coordinates and id); count them.
-template <int D>
-__global__ void __launch_bounds__(UPW_WARPS * 32, (D <= 3 ? 8 : 1)) k_match(LeafGroup* groups, const uint32_t* ngroups,
-                                                          const Node* nodes, Pts A, Pts F, uint8_t* dead,
-                                                          uint32_t* aux) {
+// Deletion round 1 at the leaves: stored points equal to a routed batch point
+// (coordinates and id) go.  MARK: the leaves of rebuilt subtrees, whose points
+// the flatten copies: they are only marked (dead).  Otherwise the survivors
+// move to the front of the leaf and its size is rewritten at once, in the pass
+// that has its points in registers (marking every leaf and compacting in a
+// second pass read each leaf twice: 0.55 + 0.89 ms for the 1e7 random deletes
+// in 1e8 points).  *total counts the points that go.
+template <int D, bool MARK>
+__global__ void __launch_bounds__(UPW_WARPS * 32, (D <= 3 ? 8 : 1)) k_delete_leaves(const LeafGroup* groups,
+                                                          const uint32_t* ngroups, Node* nodes, Pts A, Pts F,
+                                                          uint8_t* dead, uint32_t* total) {
+  __shared__ uint32_t sum_sh[UPW_WARPS];
   const uint32_t n = *ngroups;
   const uint32_t k0 = (blockIdx.x * UPW_WARPS + warp_id()) * UPW;
-  if (k0 >= n) return;
   const int lane = lane_id();
+  uint32_t gone = 0;  // of the warp
   uint32_t slot = 0, a = 0, sz = 0, glen = 0;
   unsigned long long gst = 0;
   if (lane < UPW && k0 + lane < n) {
@@ -450,423 +59,148 @@ __global__ void __launch_bounds__(UPW_WARPS * 32, (D <= 3 ? 8 : 1)) k_match(Leaf
     a = leaf.a;
     sz = leaf.size;
   }
-  {
-    // common case: every leaf of the warp holds at most 32 points and
-    // receives at most 32 / UPW batch points; all loads are issued at once
-    constexpr int PER = 32 / UPW;
-    uint32_t qa[UPW], qsz[UPW], qlen[UPW];
-    bool small = true;
-#pragma unroll
-    for (int q = 0; q < UPW; ++q) {
-      qa[q] = __shfl_sync(FULL_MASK, a, q);
-      qsz[q] = __shfl_sync(FULL_MASK, sz, q);
-      qlen[q] = __shfl_sync(FULL_MASK, glen, q);
-      small &= qsz[q] <= 32 && qlen[q] <= (uint32_t)PER;
-    }
-    if (small) {
-      int32_t x[UPW][D];
-      uint32_t id[UPW];
-#pragma unroll
-      for (int q = 0; q < UPW; ++q) {
-        id[q] = 0;
-        if ((uint32_t)lane < qsz[q]) {
-#pragma unroll
-          for (int j = 0; j < D; ++j) x[q][j] = A.c[(uint64_t)j * A.stride + qa[q] + lane];
-          id[q] = A.id[(uint64_t)qa[q] + lane];
-        }
-      }
-      // lane q * PER + e holds batch point e of leaf q
-      const int mq = lane / PER, me = lane % PER;
-      const unsigned long long myst = __shfl_sync(FULL_MASK, gst, mq);
-      const uint32_t mylen = __shfl_sync(FULL_MASK, glen, mq);
-      int32_t fx[D];
-      uint32_t fid = 0xFFFFFFFFu;
-      if ((uint32_t)me < mylen) {
-        const uint64_t r = myst + (uint64_t)me;
-#pragma unroll
-        for (int j = 0; j < D; ++j) fx[j] = F.c[(uint64_t)j * F.stride + r];
-        fid = F.id[r];
-      }
-#pragma unroll
-      for (int q = 0; q < UPW; ++q) {
-        bool hit = false;
-        for (int t = 0; t < (int)qlen[q]; ++t) {
-          const int src = q * PER + t;
-          bool same = __shfl_sync(FULL_MASK, fid, src) == id[q];
-#pragma unroll
-          for (int j = 0; j < D; ++j) same &= __shfl_sync(FULL_MASK, fx[j], src) == x[q][j];
-          hit |= same;
-        }
-        hit &= (uint32_t)lane < qsz[q];
-        if (hit) dead[(uint64_t)qa[q] + lane] = 1;
-        const int found = __popc(__ballot_sync(FULL_MASK, hit));
-        const uint32_t qslot = __shfl_sync(FULL_MASK, slot, q);
-        if (lane == 0 && k0 + q < n) {
-          groups[k0 + q].found = (uint32_t)found;
-          aux[qslot] = (uint32_t)found;
-        }
-      }
-      return;
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < UPW; ++q) {
-    if (k0 + q >= n) break;
-    const uint32_t qa = __shfl_sync(FULL_MASK, a, q), qsz = __shfl_sync(FULL_MASK, sz, q);
-    const uint32_t qlen = __shfl_sync(FULL_MASK, glen, q), qslot = __shfl_sync(FULL_MASK, slot, q);
-    const unsigned long long qst = __shfl_sync(FULL_MASK, gst, q);
-    int found = 0;
-    for (uint32_t base = 0; base < qsz; base += 32) {
-      const uint32_t i = base + lane;
-      bool hit = false;
-      int32_t x[D];
-      uint32_t id = 0;
-      if (i < qsz) {
-        const uint64_t p = (uint64_t)qa + i;
-#pragma unroll
-        for (int j = 0; j < D; ++j) x[j] = A.c[(uint64_t)j * A.stride + p];
-        id = A.id[p];
-      }
-      // the routed batch points, 32 at a time, broadcast lane by lane
-      for (uint32_t b0 = 0; b0 < qlen; b0 += 32) {
-        const uint32_t rb = b0 + lane;
-        int32_t fx[D];
-        uint32_t fid = 0xFFFFFFFFu;
-        if (rb < qlen) {
-          const uint64_t r = qst + rb;
-#pragma unroll
-          for (int j = 0; j < D; ++j) fx[j] = F.c[(uint64_t)j * F.stride + r];
-          fid = F.id[r];
-        }
-        const int cnt = (int)min(32u, qlen - b0);
-        for (int t = 0; t < cnt; ++t) {
-          bool same = __shfl_sync(FULL_MASK, fid, t) == id;
-#pragma unroll
-          for (int j = 0; j < D; ++j) same &= __shfl_sync(FULL_MASK, fx[j], t) == x[j];
-          hit |= same;
-        }
-      }
-      hit &= i < qsz;
-      if (hit) dead[(uint64_t)qa + i] = 1;
-      found += __popc(__ballot_sync(FULL_MASK, hit));
-    }
-    if (lane == 0) {
-      groups[k0 + q].found = (uint32_t)found;
-      aux[qslot] = (uint32_t)found;
-    }
-  }
-}
-
-// Exact counts per skeleton node, bottom-up (rounds in reverse order).  The
-// item's states and bucket counts are loaded first, AGG_PER heap positions
-// per lane at a time with all their loads in flight together; the interior
-// sums are then formed level by level in shared memory, from the deepest,
-// and the counts are written out at the end.
-constexpr int AGG_PER = 4;
-__global__ void __launch_bounds__(ITEM_WARPS * 32) k_aggregate(UpdArgs a) {
-  if (pkd_failed_block(a.st)) return;
-  extern __shared__ __align__(16) int agg_sm[];
-  const uint32_t i = item_of_warp();
-  if (i >= *a.nitems) return;  // warp-uniform
-  const int lane = lane_id();
-  int* ms = agg_sm + (size_t)warp_id() * 2 * a.HN;
-  uint32_t* fs = reinterpret_cast<uint32_t*>(ms + a.HN);
-  const int2* sk = a.skel + (uint64_t)i * a.HN;
-  const uint32_t* sl = a.slots + (uint64_t)i * a.HN;
-  uint32_t* f = a.fnd + (uint64_t)i * a.HN;
-  const uint64_t kb0 = (uint64_t)i * a.NB;
-  for (int v0 = 1; v0 < a.HN; v0 += 32 * AGG_PER) {
-    int m[AGG_PER];
-#pragma unroll
-    for (int u = 0; u < AGG_PER; ++u) {
-      const int v = v0 + 32 * u + lane;
-      m[u] = v < a.HN ? sk[v].y : sk_meta(SK_NONE, 0, 0);
-    }
-    uint32_t L[AGG_PER];
-#pragma unroll
-    for (int u = 0; u < AGG_PER; ++u)
-      L[u] = sk_state(m[u]) == SK_BUCKET ? a.link[kb0 + sk_bucket(m[u])] : LINK_NONE;
-#pragma unroll
-    for (int u = 0; u < AGG_PER; ++u) {
-      uint32_t c = 0;
-      if (L[u] != LINK_NONE)
-        c = (L[u] & LINK_LEAF) ? a.groups[L[u] & ~LINK_LEAF].found : a.next_fnd[(uint64_t)L[u] * a.next_HN + 1];
-      const int v = v0 + 32 * u + lane;
-      if (v < a.HN) {
-        ms[v] = m[u];
-        fs[v] = c;
-      }
-    }
-  }
-  __syncwarp();
-  for (int j = a.lam - 1; j >= 0; --j) {  // interior nodes sit above level lambda
-    for (int v = (1 << j) + lane; v < (2 << j); v += 32)
-      if (sk_state(ms[v]) == SK_INTERNAL) fs[v] = fs[2 * v] + fs[2 * v + 1];
-    __syncwarp();
-  }
-  for (int v = 1 + lane; v < a.HN; v += 32) {
-    if (sk_state(ms[v]) == SK_NONE) continue;
-    const uint32_t c = fs[v];
-    f[v] = c;
-    if (!a.insert && c) a.aux[sl[v]] = c;
-  }
-}
-
-__device__ void push_rebuild(const UpdArgs& a, uint32_t slot, uint32_t depth, uint32_t size, uint32_t old,
-                             uint32_t old_live, uint64_t ws, uint64_t we) {
-  const uint32_t k = atomicAdd(a.nitems_out, 1u);
-  if (k >= a.items_cap) {
-    set_error(a.st, DERR_CAPACITY, 810);
-    return;
-  }
-  a.items_out[k] = RebuildItem{slot, depth, size, old_live, ws, we, 0};
-  atomicAdd(a.items_total, (unsigned long long)size);
-  atomicAdd(a.inner_total, (unsigned long long)old);
-  atomicMax(a.items_max, size);
-}
-
-// Top-down alpha test over every skeleton (rounds in forward order; within a
-// skeleton, level by level from the root).  under: one bit per heap node
-// inside a subtree that is rebuilt.
-// The item's skeleton, slots, counts and the nodes' current sizes are staged
-// in shared memory first (DEC_PER heap positions per lane at a time, their
-// loads in flight together); the levels then read shared memory only.
-constexpr int DEC_PER = 4;
-__global__ void __launch_bounds__(ITEM_WARPS * 32) k_decide(UpdArgs a) {
-  if (pkd_failed_block(a.st)) return;
-  extern __shared__ __align__(16) uint8_t dec_sm[];
-  __shared__ uint32_t under_sh[ITEM_WARPS][64];
-  const uint32_t i = item_of_warp();
-  if (i >= *a.nitems) return;  // warp-uniform
-  const int lane = lane_id();
-  uint32_t* under = under_sh[warp_id()];
-  const Seg it = a.items[i];
-  int2* sk = reinterpret_cast<int2*>(dec_sm) + (size_t)warp_id() * a.HN;
-  uint32_t* sl = reinterpret_cast<uint32_t*>(reinterpret_cast<int2*>(dec_sm) + (size_t)ITEM_WARPS * a.HN) +
-                 (size_t)warp_id() * a.HN;
-  uint32_t* f = sl + (size_t)ITEM_WARPS * a.HN;
-  uint32_t* osz = f + (size_t)ITEM_WARPS * a.HN;
-  {
-    const int2* gsk = a.skel + (uint64_t)i * a.HN;
-    const uint32_t* gsl = a.slots + (uint64_t)i * a.HN;
-    const uint32_t* gf = a.fnd + (uint64_t)i * a.HN;
-    for (int v0 = 1; v0 < a.HN; v0 += 32 * DEC_PER) {
-      int2 e[DEC_PER];
-      uint32_t slv[DEC_PER], fv[DEC_PER], szv[DEC_PER];
-#pragma unroll
-      for (int u = 0; u < DEC_PER; ++u) {
-        const int v = v0 + 32 * u + lane;
-        e[u] = v < a.HN ? gsk[v] : make_int2(0, sk_meta(SK_NONE, 0, 0));
-      }
-#pragma unroll
-      for (int u = 0; u < DEC_PER; ++u) {
-        const int v = v0 + 32 * u + lane;
-        slv[u] = 0;
-        fv[u] = 0;
-        if (sk_state(e[u].y) != SK_NONE) {
-          slv[u] = gsl[v];
-          fv[u] = gf[v];
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < DEC_PER; ++u) szv[u] = sk_state(e[u].y) != SK_NONE ? a.nodes[slv[u]].size : 0u;
-#pragma unroll
-      for (int u = 0; u < DEC_PER; ++u) {
-        const int v = v0 + 32 * u + lane;
-        if (v >= a.HN) continue;
-        sk[v] = e[u];
-        sl[v] = slv[u];
-        f[v] = fv[u];
-        osz[v] = szv[u];
-      }
-    }
-  }
-  under[lane] = 0;
-  under[lane + 32] = 0;
-  __syncwarp();
-  if (lane == 0 && a.iflag[i]) under[0] = 2u;
-  __syncwarp();
-  for (int j = 0; j <= a.lam; ++j) {
-    for (int v = (1 << j) + lane; v < (2 << j); v += 32) {
-      const int m = sk[v].y;
-      const int st = sk_state(m);
-      if (st == SK_NONE) continue;
-      const bool u = (under[v >> 5] >> (v & 31)) & 1u;
-      if (st == SK_BUCKET) {
-        if (!u) continue;
-        const uint32_t L = a.link[(uint64_t)i * a.NB + sk_bucket(m)];
-        if (L == LINK_NONE) continue;
-        if (L & LINK_LEAF) a.groups[L & ~LINK_LEAF].flag = 1;
-        else a.next_iflag[L] = 1;
-        continue;
-      }
-      const int c0 = 2 * v;  // children c0 and c0 + 1 share a word of `under`
-      if (u) {
-        atomicOr(&under[c0 >> 5], 3u << (c0 & 31));
-        continue;
-      }
-      const uint32_t c = f[v];
-      if (c == 0) continue;  // nothing below changes
-      const uint32_t slot = sl[v];
-      const uint32_t old = osz[v], lold = osz[c0];
-      const uint32_t N = a.insert ? old + c : old - c;
-      const uint32_t L = a.insert ? lold + f[c0] : lold - f[c0];
-      if (N > 0 && is_balanced(L, N, a.p.alpha_num, a.p.alpha_den)) {
-        a.nsz[(uint64_t)i * a.HN + v] = N;  // written to the node once nothing can fail
-        continue;
-      }
-      // rebuild this subtree; the batch points below it are contiguous
-      int lv = v, rv = v;
-      while (sk_state(sk[lv].y) == SK_INTERNAL) lv = 2 * lv;
-      while (sk_state(sk[rv].y) == SK_INTERNAL) rv = 2 * rv + 1;
-      const uint64_t kl = (uint64_t)i * a.NB + sk_bucket(sk[lv].y);
-      const uint64_t kr = (uint64_t)i * a.NB + sk_bucket(sk[rv].y);
-      const uint32_t depth = it.depth + (31 - __clz(v));
-      push_rebuild(a, slot, depth, N, old, a.insert ? old : old - c, a.bstart[kl], a.bstart[kr] + a.blen[kr]);
-      atomicOr(&under[c0 >> 5], 3u << (c0 & 31));
-    }
-    __syncwarp();
-  }
-}
-
-// Reached leaves outside rebuilt subtrees: insert -> rebuild item
-// Build(leaf + new); delete -> compacted in place (a leaf minus some of its
-// points is a leaf again).
-__global__ void k_leaf_items(UpdArgs a, LeafGroup* groups, const uint32_t* ngroups, uint32_t* compact,
-                             uint32_t* ncompact) {
-  if (pkd_failed_block(a.st)) return;  // uniform: before the block-wide reservation
-  const uint32_t gi = blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t ng = *ngroups;
-  bool push = false, comp = false;
-  RebuildItem it{};
-  if (gi < ng) {
-    const LeafGroup G = groups[gi];
-    if (!G.flag) {
-      const uint32_t old = a.nodes[G.slot].size;
-      if (a.insert) {
-        push = true;
-        it = RebuildItem{G.slot, G.depth, old + G.len, old, G.start, G.start + G.len, 0};
-      } else if (G.found) {
-        comp = true;
-      }
-    }
-  }
-  // one counter update per block
-  const uint32_t c[2] = {push ? 1u : 0u, comp ? 1u : 0u};
-  uint32_t* const ctrs[2] = {a.nitems_out, ncompact};
-  uint32_t first[2];
-  block_reserve<2>(c, ctrs, first);
-  const unsigned long long tv[1] = {push ? (unsigned long long)it.size : 0ull};
-  unsigned long long* const tc[1] = {a.items_total};
-  block_add64<1>(tv, tc);
-  const uint32_t mx = __reduce_max_sync(FULL_MASK, push ? it.size : 0u);
-  if (mx && lane_id() == 0) atomicMax(a.items_max, mx);
-  const uint32_t bp = first[0], bc = first[1];
-  if (push) {
-    if (bp < a.items_cap) a.items_out[bp] = it;
-    else set_error(a.st, DERR_CAPACITY, 811);
-  }
-  if (comp) compact[bc] = gi;
-}
-
-template <int D>
-__global__ void __launch_bounds__(UPW_WARPS * 32) k_compact_leaves(const LeafGroup* groups, const uint32_t* list,
-                                                                   const uint32_t* n, Node* nodes, Pts A,
-                                                                   const uint8_t* dead) {
-  const uint32_t nn = *n;
-  const uint32_t k0 = (blockIdx.x * UPW_WARPS + warp_id()) * UPW;
-  if (k0 >= nn) return;
-  const int lane = lane_id();
-  uint32_t slot = 0, a = 0, sz = 0;
-  if (lane < UPW && k0 + lane < nn) {
-    slot = groups[list[k0 + lane]].slot;
-    const Node nd = nodes[slot];
-    a = nd.a;
-    sz = nd.size;
-  }
-  uint32_t qa[UPW], qsz[UPW], qslot[UPW];
+  // common case: every leaf of the warp holds at most 32 points and
+  // receives at most 32 / UPW batch points; all loads are issued at once
+  constexpr int PER = 32 / UPW;
+  uint32_t qa[UPW], qsz[UPW], qlen[UPW];
   bool small = true;
 #pragma unroll
   for (int q = 0; q < UPW; ++q) {
     qa[q] = __shfl_sync(FULL_MASK, a, q);
     qsz[q] = __shfl_sync(FULL_MASK, sz, q);
-    qslot[q] = __shfl_sync(FULL_MASK, slot, q);
-    small &= qsz[q] <= 32;
+    qlen[q] = __shfl_sync(FULL_MASK, glen, q);
+    small &= qsz[q] <= 32 && qlen[q] <= (uint32_t)PER;
   }
   if (small) {
-    // survivors move to the front, in order: all loads, then all stores
     int32_t x[UPW][D];
     uint32_t id[UPW];
-    bool keep[UPW];
 #pragma unroll
     for (int q = 0; q < UPW; ++q) {
-      keep[q] = lane < qsz[q] && !dead[(uint64_t)qa[q] + lane];
-      if (lane < qsz[q]) {
+      id[q] = 0;
+      if ((uint32_t)lane < qsz[q]) {
 #pragma unroll
         for (int j = 0; j < D; ++j) x[q][j] = A.c[(uint64_t)j * A.stride + qa[q] + lane];
         id[q] = A.id[(uint64_t)qa[q] + lane];
       }
     }
-    __syncwarp();
+    // lane q * PER + e holds batch point e of leaf q
+    const int mq = lane / PER, me = lane % PER;
+    const unsigned long long myst = __shfl_sync(FULL_MASK, gst, mq);
+    const uint32_t mylen = __shfl_sync(FULL_MASK, glen, mq);
+    int32_t fx[D];
+    uint32_t fid = 0xFFFFFFFFu;
+    if ((uint32_t)me < mylen) {
+      const uint64_t r = myst + (uint64_t)me;
+#pragma unroll
+      for (int j = 0; j < D; ++j) fx[j] = F.c[(uint64_t)j * F.stride + r];
+      fid = F.id[r];
+    }
 #pragma unroll
     for (int q = 0; q < UPW; ++q) {
-      const unsigned m = __ballot_sync(FULL_MASK, keep[q]);
-      if (keep[q]) {
-        const uint64_t o = (uint64_t)qa[q] + __popc(m & lanemask_lt());
+      bool hit = false;
+      for (int t = 0; t < (int)qlen[q]; ++t) {
+        const int src = q * PER + t;
+        bool same = __shfl_sync(FULL_MASK, fid, src) == id[q];
 #pragma unroll
-        for (int j = 0; j < D; ++j) A.c[(uint64_t)j * A.stride + o] = x[q][j];
-        A.id[o] = id[q];
+        for (int j = 0; j < D; ++j) same &= __shfl_sync(FULL_MASK, fx[j], src) == x[q][j];
+        hit |= same;
       }
-      if (lane == 0 && k0 + q < nn) nodes[qslot[q]].size = (uint32_t)__popc(m);
+      const bool in = (uint32_t)lane < qsz[q];
+      hit &= in;
+      gone += __popc(__ballot_sync(FULL_MASK, hit));
+      if constexpr (MARK) {
+        if (hit) dead[(uint64_t)qa[q] + lane] = 1;
+      } else {  // the whole leaf is in registers: survivors to the front, in order
+        const unsigned m = __ballot_sync(FULL_MASK, in && !hit);
+        if (in && !hit) {
+          const uint64_t o = (uint64_t)qa[q] + __popc(m & lanemask_lt());
+          if (o != (uint64_t)qa[q] + lane) {
+#pragma unroll
+            for (int j = 0; j < D; ++j) A.c[(uint64_t)j * A.stride + o] = x[q][j];
+            A.id[o] = id[q];
+          }
+        }
+        const uint32_t qslot = __shfl_sync(FULL_MASK, slot, q);
+        if (lane == 0 && qsz[q]) nodes[qslot].size = (uint32_t)__popc(m);
+      }
     }
-    return;
-  }
+  } else {
 #pragma unroll 1
-  for (int q = 0; q < UPW; ++q) {
-    if (k0 + q >= nn) break;
-    uint32_t out = 0;
-    for (uint32_t base = 0; base < qsz[q]; base += 32) {
-      const uint32_t i = base + lane;
-      const bool keep = i < qsz[q] && !dead[(uint64_t)qa[q] + i];
-      int32_t x[D];
-      uint32_t id = 0;
-      if (keep) {
+    for (int q = 0; q < UPW; ++q) {
+      if (k0 + q >= n) break;
+      const uint32_t qslot = __shfl_sync(FULL_MASK, slot, q);
+      const uint32_t qa_ = __shfl_sync(FULL_MASK, a, q), qsz_ = __shfl_sync(FULL_MASK, sz, q);
+      const uint32_t qlen_ = __shfl_sync(FULL_MASK, glen, q);
+      const unsigned long long qst = __shfl_sync(FULL_MASK, gst, q);
+      uint32_t out = 0;
+      for (uint32_t base = 0; base < qsz_; base += 32) {
+        const uint32_t i = base + lane;
+        bool hit = false;
+        int32_t x[D];
+        uint32_t id = 0;
+        if (i < qsz_) {
+          const uint64_t p = (uint64_t)qa_ + i;
 #pragma unroll
-        for (int j = 0; j < D; ++j) x[j] = A.c[(uint64_t)j * A.stride + qa[q] + i];
-        id = A.id[(uint64_t)qa[q] + i];
-      }
-      const unsigned m = __ballot_sync(FULL_MASK, keep);
-      __syncwarp();
-      if (keep) {
-        const uint64_t o = (uint64_t)qa[q] + out + __popc(m & lanemask_lt());
+          for (int j = 0; j < D; ++j) x[j] = A.c[(uint64_t)j * A.stride + p];
+          id = A.id[p];
+        }
+        // the routed batch points, 32 at a time, broadcast lane by lane
+        for (uint32_t b0 = 0; b0 < qlen_; b0 += 32) {
+          const uint32_t rb = b0 + lane;
+          int32_t fx[D];
+          uint32_t fid = 0xFFFFFFFFu;
+          if (rb < qlen_) {
+            const uint64_t r = qst + rb;
 #pragma unroll
-        for (int j = 0; j < D; ++j) A.c[(uint64_t)j * A.stride + o] = x[j];
-        A.id[o] = id;
+            for (int j = 0; j < D; ++j) fx[j] = F.c[(uint64_t)j * F.stride + r];
+            fid = F.id[r];
+          }
+          const int cnt = (int)min(32u, qlen_ - b0);
+          for (int t = 0; t < cnt; ++t) {
+            bool same = __shfl_sync(FULL_MASK, fid, t) == id;
+#pragma unroll
+            for (int j = 0; j < D; ++j) same &= __shfl_sync(FULL_MASK, fx[j], t) == x[j];
+            hit |= same;
+          }
+        }
+        hit &= i < qsz_;
+        gone += __popc(__ballot_sync(FULL_MASK, hit));
+        if constexpr (MARK) {
+          if (hit) dead[(uint64_t)qa_ + i] = 1;
+        } else {
+          const bool keep = i < qsz_ && !hit;
+          const unsigned m = __ballot_sync(FULL_MASK, keep);
+          __syncwarp();
+          if (keep) {
+            const uint64_t o = (uint64_t)qa_ + out + __popc(m & lanemask_lt());
+#pragma unroll
+            for (int j = 0; j < D; ++j) A.c[(uint64_t)j * A.stride + o] = x[j];
+            A.id[o] = id;
+          }
+          out += __popc(m);
+          __syncwarp();
+        }
       }
-      out += __popc(m);
-      __syncwarp();
+      if (!MARK && lane == 0) nodes[qslot].size = out;
     }
-    if (lane == 0) nodes[qslot[q]].size = out;
+  }
+  if (lane == 0) sum_sh[warp_id()] = gone;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t t = 0;
+    for (int w = 0; w < UPW_WARPS; ++w) t += sum_sh[w];
+    if (t) atomicAdd(total, t);
   }
 }
 
-// Arena positions of the rebuild items (exclusive scan of their sizes).
-__global__ void k_item_sizes(const RebuildItem* it, const uint32_t* n, uint32_t* sizes) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < *n) sizes[i] = it[i].size;
-}
-
-// An item of at most phi points is a leaf again (Build wraps it): its
-// segment is skipped by the rebuild, which then only visits the items that
-// split, and k_item_leaves writes its node once its points are in place.
-__global__ void k_item_pos(RebuildItem* it, const uint32_t* n, const uint32_t* off, uint64_t top, Seg* segs,
-                           uint32_t phi) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= *n) return;
-  const RebuildItem x = it[i];
-  const uint64_t pos = top + off[i];
-  it[i].pos = pos;
-  segs[i] = Seg{pos, x.size <= phi ? SEG_SKIP : x.size, x.depth, x.slot, IN_A};
+// The marks of a delete's rebuilt subtrees, cleared: one warp per leaf (its
+// node record, in the old subtree, is still there).
+__global__ void k_clear_dead(const LeafGroup* groups, const uint32_t* ngroups, const Node* nodes, uint8_t* dead) {
+  const uint32_t n = *ngroups;
+  for (uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < n; g += (gridDim.x * blockDim.x) >> 5) {
+    const Node nd = nodes[groups[g].slot];
+    for (uint32_t i = lane_id(); i < nd.size; i += 32) dead[(uint64_t)nd.a + i] = 0;
+  }
 }
 
 // The node of every item of at most phi points: a leaf over its new range.
@@ -889,14 +223,11 @@ struct Front {
   uint64_t off;
 };
 
-// Leaves of more than BIG_LEAF points are copied one block each.
-constexpr uint32_t BIG_LEAF = 1024;
-
 constexpr int FRONT_BATCH = 8;  // frontier levels launched per host check
 
 __global__ void k_front_init(const RebuildItem* it, const uint32_t* n, Front* f, uint32_t* nf) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool e = i < *n && it[i].old_live != 0;
+  const bool e = i < *n && !it[i].leaf && it[i].old_live != 0;
   const uint32_t c[1] = {e ? 1u : 0u};
   uint32_t* const ctrs[1] = {nf};
   uint32_t first[1];
@@ -909,13 +240,15 @@ __global__ void k_front_init(const RebuildItem* it, const uint32_t* n, Front* f,
 // reading any count in between; a level with an empty frontier does nothing.
 // An entry past a list's capacity is not written: it sets *ovf, and the
 // host redoes the flatten with larger lists.  The counts still include such
-// entries, so a level reads at most `cap` entries of its frontier (the
-// entries past it were never written; the attempt is redone anyway).
+// entries, so a level reads at most `cap` entries of its frontier, rounded down
+// to whole pairs: children are written in pairs from even positions, and a pair
+// that does not fit whole is not written (the attempt is redone anyway).  The
+// roots always fit with room to spare.
 __global__ void k_front_expand(const Front* f, const uint32_t* nf, Front* g, uint32_t* ng, Front* leaves,
                                uint32_t* nleaves, Front* bigleaves, uint32_t* nbig, const Node* nodes,
                                const uint8_t* ndim, const uint32_t* aux, int use_aux, uint32_t cap, uint32_t bcap,
                                uint32_t* ovf) {
-  const uint32_t n = min(*nf, cap);
+  const uint32_t n = min(*nf, cap & ~1u);
   for (uint32_t base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
     const uint32_t i = base + threadIdx.x;
     const bool have = i < n;
@@ -1022,51 +355,93 @@ __global__ void __launch_bounds__(UPW_WARPS * 32) k_copy_leaves(const Front* lv,
   }
 }
 
-// Insert: append each item's new batch points after its old ones (UPW
-// items per warp); items with more than NEW_BIG new points are left to
-// k_copy_new_flat.
+// Rebuild items, UPW per warp: the item's build segment; a leaf item's stored
+// points (an insert's items are mostly leaves) and the new points of an item
+// with at most NEW_BIG of them go to its arena range.  The larger ones are
+// left to k_copy_new_flat, the other old subtrees to the flatten.
+// An item of at most phi points is a leaf again (Build wraps it): its segment
+// is skipped by the rebuild, which then only visits the items that split, and
+// k_item_leaves writes its node once its points are in place.
 constexpr uint64_t NEW_BIG = 256;
 template <int D>
-__global__ void __launch_bounds__(UPW_WARPS * 32, (D <= 3 ? 8 : 1)) k_copy_new(const RebuildItem* items, const uint32_t* n, Pts F,
-                                                             Pts A) {
+__global__ void __launch_bounds__(UPW_WARPS * 32, (D <= 3 ? 6 : 1)) k_copy_items(const RebuildItem* items,
+                                                            const uint32_t* n, const Node* nodes, Pts F, Pts A,
+                                                            Seg* segs, uint32_t phi) {
   const uint32_t nn = *n;
   const uint32_t k0 = (blockIdx.x * UPW_WARPS + warp_id()) * UPW;
   if (k0 >= nn) return;
   const int lane = lane_id();
-  unsigned long long ws = 0, cnt = 0, dst0 = 0;
+  unsigned long long ws = 0, cnt = 0, pos = 0;
+  uint32_t a = 0, sz = 0, live = 0;
   if (lane < UPW && k0 + lane < nn) {
     const RebuildItem it = items[k0 + lane];
     ws = it.ws;
     cnt = it.we - it.ws;
-    dst0 = it.pos + it.old_live;
-  }
-  {
-    // common case: at most 32 / UPW new points per item, one per lane
-    constexpr int PER = 32 / UPW;
-    const int mq = lane / PER, me = lane % PER;
-    const unsigned long long mws = __shfl_sync(FULL_MASK, ws, mq), mcnt = __shfl_sync(FULL_MASK, cnt, mq);
-    const unsigned long long md = __shfl_sync(FULL_MASK, dst0, mq);
-    if (__all_sync(FULL_MASK, mcnt <= (unsigned long long)PER)) {
-      if ((unsigned long long)me < mcnt) {
-        const uint64_t src = mws + me, dst = md + me;
-        int32_t x[D];
-#pragma unroll
-        for (int j = 0; j < D; ++j) x[j] = F.c[(uint64_t)j * F.stride + src];
-        const uint32_t id = F.id[src];
-#pragma unroll
-        for (int j = 0; j < D; ++j) A.c[(uint64_t)j * A.stride + dst] = x[j];
-        A.id[dst] = id;
-      }
-      return;
+    pos = it.pos;
+    live = it.old_live;
+    if (it.leaf) {
+      const Node nd = nodes[it.slot];
+      a = nd.a;
+      sz = nd.size;
     }
+    segs[k0 + lane] = Seg{it.pos, it.size <= phi ? SEG_SKIP : it.size, it.depth, it.slot, IN_A};
+  }
+  // common case: leaves of at most 32 points, at most 32 / UPW new points per
+  // item, one per lane: every load before the first store
+  constexpr int PER = 32 / UPW;
+  const int mq = lane / PER, me = lane % PER;
+  const unsigned long long mws = __shfl_sync(FULL_MASK, ws, mq), mcnt = __shfl_sync(FULL_MASK, cnt, mq);
+  const unsigned long long md = __shfl_sync(FULL_MASK, pos, mq) + __shfl_sync(FULL_MASK, live, mq);
+  const bool few = __all_sync(FULL_MASK, mcnt <= (unsigned long long)PER);
+  if (few && __all_sync(FULL_MASK, sz <= 32)) {
+    int32_t x[UPW][D], fx[D];
+    uint32_t id[UPW], fid = 0;
+#pragma unroll
+    for (int q = 0; q < UPW; ++q) {
+      const uint32_t qa = __shfl_sync(FULL_MASK, a, q), qsz = __shfl_sync(FULL_MASK, sz, q);
+      if ((uint32_t)lane < qsz) {
+#pragma unroll
+        for (int j = 0; j < D; ++j) x[q][j] = A.c[(uint64_t)j * A.stride + qa + lane];
+        id[q] = A.id[(uint64_t)qa + lane];
+      }
+    }
+    if ((unsigned long long)me < mcnt) {
+#pragma unroll
+      for (int j = 0; j < D; ++j) fx[j] = F.c[(uint64_t)j * F.stride + mws + me];
+      fid = F.id[mws + me];
+    }
+#pragma unroll
+    for (int q = 0; q < UPW; ++q) {
+      const uint32_t qsz = __shfl_sync(FULL_MASK, sz, q);
+      const unsigned long long o = __shfl_sync(FULL_MASK, pos, q) + lane;
+      if ((uint32_t)lane < qsz) {
+#pragma unroll
+        for (int j = 0; j < D; ++j) A.c[(uint64_t)j * A.stride + o] = x[q][j];
+        A.id[o] = id[q];
+      }
+    }
+    if ((unsigned long long)me < mcnt) {
+#pragma unroll
+      for (int j = 0; j < D; ++j) A.c[(uint64_t)j * A.stride + md + me] = fx[j];
+      A.id[md + me] = fid;
+    }
+    return;
   }
 #pragma unroll 1
   for (int q = 0; q < UPW; ++q) {
     const unsigned long long qws = __shfl_sync(FULL_MASK, ws, q), qcnt = __shfl_sync(FULL_MASK, cnt, q);
-    const unsigned long long qd = __shfl_sync(FULL_MASK, dst0, q);
+    const unsigned long long qpos = __shfl_sync(FULL_MASK, pos, q);
+    const uint32_t qa = __shfl_sync(FULL_MASK, a, q), qsz = __shfl_sync(FULL_MASK, sz, q);
+    const uint32_t qlive = __shfl_sync(FULL_MASK, live, q);
+    for (uint32_t i = lane; i < qsz; i += 32) {
+      const uint64_t src = (uint64_t)qa + i, dst = qpos + i;
+#pragma unroll
+      for (int j = 0; j < D; ++j) A.c[(uint64_t)j * A.stride + dst] = A.c[(uint64_t)j * A.stride + src];
+      A.id[dst] = A.id[src];
+    }
     if (qcnt > NEW_BIG) continue;  // k_copy_new_flat copies these
     for (uint64_t i = lane; i < qcnt; i += 32) {
-      const uint64_t src = qws + i, dst = qd + i;
+      const uint64_t src = qws + i, dst = qpos + qlive + i;
 #pragma unroll
       for (int j = 0; j < D; ++j) A.c[(uint64_t)j * A.stride + dst] = F.c[(uint64_t)j * F.stride + src];
       A.id[dst] = F.id[src];
@@ -1084,7 +459,7 @@ __global__ void k_item_newcounts(const RebuildItem* it, const uint32_t* n, uint3
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < *n) {
     const uint64_t c = it[i].we - it[i].ws;
-    cnt[i] = c > NEW_BIG ? (uint32_t)c : 0u;  // the items k_copy_new leaves out
+    cnt[i] = c > NEW_BIG ? (uint32_t)c : 0u;  // the items k_copy_items leaves out
   }
 }
 
@@ -1172,14 +547,10 @@ static void launch_copy_big_leaves(const Front* lv, const uint32_t* n, uint32_t 
 }
 
 template <int D>
-static void launch_match(LeafGroup* g, const uint32_t* ng, uint32_t n, const Node* nodes, Pts A, Pts F,
-                         uint8_t* dead, uint32_t* aux, cudaStream_t s) {
-  PKD_LAUNCH(k_match<D><<<upw_blocks(n), UPW_WARPS * 32, 0, s>>>(g, ng, nodes, A, F, dead, aux));
-}
-template <int D>
-static void launch_compact(const LeafGroup* g, const uint32_t* list, const uint32_t* n, uint32_t nh, Node* nodes,
-                           Pts A, const uint8_t* dead, cudaStream_t s) {
-  PKD_LAUNCH(k_compact_leaves<D><<<upw_blocks(nh), UPW_WARPS * 32, 0, s>>>(g, list, n, nodes, A, dead));
+static void launch_delete(bool mark, const LeafGroup* g, const uint32_t* ng, uint32_t n, Node* nodes, Pts A, Pts F,
+                          uint8_t* dead, uint32_t* total, cudaStream_t s) {
+  if (mark) PKD_LAUNCH((k_delete_leaves<D, true><<<upw_blocks(n), UPW_WARPS * 32, 0, s>>>(g, ng, nodes, A, F, dead, total)));
+  else PKD_LAUNCH((k_delete_leaves<D, false><<<upw_blocks(n), UPW_WARPS * 32, 0, s>>>(g, ng, nodes, A, F, dead, total)));
 }
 template <int D>
 static void launch_copy_leaves(const Front* lv, const uint32_t* n, uint32_t nh, const RebuildItem* items,
@@ -1187,42 +558,45 @@ static void launch_copy_leaves(const Front* lv, const uint32_t* n, uint32_t nh, 
   PKD_LAUNCH(k_copy_leaves<D><<<upw_blocks(nh), UPW_WARPS * 32, 0, s>>>(lv, n, items, nodes, A, dead, use_dead));
 }
 template <int D>
-static void launch_copy_new(const RebuildItem* items, const uint32_t* n, uint32_t nh, Pts F, Pts A, cudaStream_t s) {
-  PKD_LAUNCH(k_copy_new<D><<<upw_blocks(nh), UPW_WARPS * 32, 0, s>>>(items, n, F, A));
+static void launch_copy_items(const RebuildItem* items, const uint32_t* n, uint32_t nh, const Node* nodes, Pts F, Pts A,
+                              Seg* segs, uint32_t phi, cudaStream_t s) {
+  PKD_LAUNCH(k_copy_items<D><<<upw_blocks(nh), UPW_WARPS * 32, 0, s>>>(items, n, nodes, F, A, segs, phi));
 }
 
-// The deferred size updates of the nodes that stay (k_decide), applied once
-// the update can no longer fail for lack of memory.
-__global__ void k_apply_sizes(const uint32_t* slots, const uint32_t* nsz, uint64_t n, Node* nodes) {
-  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n && nsz[i] != 0xFFFFFFFFu) nodes[slots[i]].size = nsz[i];
-}
-
-// Node records of the rebuild items' root slots, saved before the rebuild
-// writes them and put back when it fails.
-__global__ void k_save_roots(const RebuildItem* it, const uint32_t* n, const Node* nodes, const uint8_t* ndim,
-                             Node* bn, uint8_t* bd) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < *n) {
-    bn[i] = nodes[it[i].slot];
-    bd[i] = ndim[it[i].slot];
+// The items of a round that one team answers each; nmid and nsmall bound (or
+// are) their numbers.
+template <int D>
+static void launch_route(const RouteArgs& a, const Seg* mid, const uint32_t* d_nmid, uint32_t nmid, const Seg* small,
+                         const uint32_t* d_nsmall, uint32_t nsmall, cudaStream_t s) {
+  const size_t per = skel_bytes(a.HN, a.NB), warps = per * WARP_TEAMS;
+  if (warps > 48 * 1024) {
+    cudaFuncSetAttribute(k_route<D, MID_TEAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)per);
+    cudaFuncSetAttribute(k_route<D, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)warps);
   }
-}
-__global__ void k_restore_roots(const RebuildItem* it, const uint32_t* n, Node* nodes, uint8_t* ndim, const Node* bn,
-                                const uint8_t* bd) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < *n) {
-    nodes[it[i].slot] = bn[i];
-    ndim[it[i].slot] = bd[i];
+  if (nmid) PKD_LAUNCH((k_route<D, MID_TEAM><<<nmid, MID_TEAM, per, s>>>(a, mid, d_nmid)));
+  if (nsmall) {
+    const unsigned g = (nsmall + WARP_TEAMS - 1) / WARP_TEAMS;
+    PKD_LAUNCH((k_route<D, 32><<<g, 32 * WARP_TEAMS, warps, s>>>(a, small, d_nsmall)));
   }
 }
 
-__global__ void k_clear_aux(const uint32_t* slots, uint64_t n, uint32_t* aux) {
-  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) {
-    const uint32_t s = slots[i];
-    if (s != 0xFFFFFFFFu) aux[s] = 0;
-  }
+// The recorded sizes of the nodes that stay, applied once the update can no
+// longer fail for lack of memory.
+__global__ void k_apply_sizes(const uint2* stay, const uint32_t* n, uint32_t cap, Node* nodes) {
+  const uint32_t nn = min(*n, cap);
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += gridDim.x * blockDim.x)
+    nodes[stay[i].x].size = stay[i].y;
+}
+
+__global__ void k_clear_aux(const uint32_t* slots, const uint32_t* n, uint32_t cap, uint32_t* aux) {
+  const uint32_t nn = min(*n, cap);
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += gridDim.x * blockDim.x) aux[slots[i]] = 0;
+}
+
+// The counters of an update, zeroed, and its first round: one item, the root.
+__global__ void k_update_init(uint32_t* ctl, uint32_t words, Seg root, Seg* list, int which) {
+  for (uint32_t i = threadIdx.x; i < words; i += blockDim.x) ctl[i] = (int)i == which ? 1u : 0u;
+  if (threadIdx.x == 0) *list = root;
 }
 
 __global__ void k_stage(const int32_t* coords, const uint32_t* ids, uint64_t m, int d, Pts W) {
@@ -1293,48 +667,53 @@ static int ensure_capacity(TreeMem& t, uint64_t need, cudaStream_t s) {
   return PKD_OK;
 }
 
-static int ensure_delete_scratch(TreeMem& t, cudaStream_t s) {
+// The delete scratch: aux before the batch is routed, dead when a subtree is
+// rebuilt.
+static int ensure_aux(TreeMem& t, cudaStream_t s) {
+  if (t.aux) return PKD_OK;
   bool zero = false;
-  if (!t.dead) {
-    PKD_CUDA(big_alloc_zeroed((void**)&t.dead, t.cap, s, &zero));
-    if (!zero) PKD_TRY(dev_fill(t.dead, 0, t.cap, s));
-  }
-  if (!t.aux) {
-    PKD_CUDA(big_alloc_zeroed((void**)&t.aux, t.node_cap * 4, s, &zero));
-    if (!zero) PKD_TRY(dev_fill(t.aux, 0, t.node_cap * 4, s));
-    else stat_items("scratch_zeroed", t.node_cap * 4);
-  }
+  PKD_CUDA(big_alloc_zeroed((void**)&t.aux, t.node_cap * 4, s, &zero));
+  if (!zero) PKD_TRY(dev_fill(t.aux, 0, t.node_cap * 4, s));
+  else stat_items("scratch_zeroed", t.node_cap * 4);
+  return PKD_OK;
+}
+static int ensure_dead(TreeMem& t, cudaStream_t s) {
+  if (t.dead) return PKD_OK;
+  bool zero = false;
+  PKD_CUDA(big_alloc_zeroed((void**)&t.dead, t.cap, s, &zero));
+  if (!zero) PKD_TRY(dev_fill(t.dead, 0, t.cap, s));
   return PKD_OK;
 }
 
+// One round of a route: its lists of recorded sizes and of aux words.
 struct RouteRound {
-  Seg* items;
-  uint32_t n;
-  int2* skel;
-  uint32_t* slots;
-  uint32_t* fnd;
-  uint32_t* nsz;
-  uint32_t* link;
-  uint64_t* bstart;
-  uint32_t* blen;
-  uint32_t* iflag;
-  uint32_t* d_n;  // device copy of n
+  uint2* stay = nullptr;
+  uint32_t stay_cap = 0;
+  uint32_t* auxs = nullptr;
+  uint32_t aux_cap = 0;
+  const uint32_t* ctl = nullptr;  // the round's R_* counters
 };
+
+static unsigned list_blocks(uint64_t n) {
+  return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((n + 255) / 256, 152 * 8));
+}
 
 // The batch comes either point-major from the caller (coords, ids) or
 // already staged in structure-of-arrays form (`staged`, a buffer of at least
-// m positions that the route may overwrite).
+// m positions that the route may overwrite).  Returns after its work has
+// finished, with the tree's status read; *idflags (insert): the id table's
+// flags of the batch, nothing of the tree has changed when they are set.
 static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, const Pts* staged, uint64_t m,
-                      bool insert, uint64_t* n_changed, cudaStream_t s) {
+                      bool insert, uint64_t* n_changed, int* idflags, cudaStream_t s) {
   const Params& p = t.p;
   const int d = p.d, lam = p.lambda, NB = 1 << lam, HN = 2 << lam;
   const int TILE = std::min(std::max(knobs().tile, 256), 4096);
   Scratch sc{s, {}};
   trace_mark(s, insert ? "insert: enter" : "delete: enter");
-  if (!insert) PKD_TRY(ensure_delete_scratch(t, s));
+  if (!insert) PKD_TRY(ensure_aux(t, s));
   trace_mark(s, "upd: delete scratch");
 
-  // batch buffers: W0/W1 ping-pong for the sieve, F final positions
+  // batch buffers: W0/W1 ping-pong between the rounds, F final positions
   int32_t *wc[3] = {nullptr, nullptr, nullptr};
   uint32_t* wid[3] = {nullptr, nullptr, nullptr};
   for (int k = staged ? 1 : 0; k < 3; ++k) {
@@ -1345,405 +724,323 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
   Pts F{wc[2], wid[2], m};
   if (!staged) PKD_LAUNCH(k_stage<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(coords, ids, m, d, W[0]));
 
-  uint32_t* dctr;
-  PKD_TRY(sc.get(&dctr, 32));
-  PKD_TRY(dev_fill(dctr, 0, 32 * 4, s));
-  PinnedBlock hblk;  // 128 bytes of host counters
-  uint32_t* hctr = (uint32_t*)hblk.p;
-  if (!hctr) return PKD_ENOMEM;
-  uint32_t* d_ngroups = dctr + 4;
-  uint32_t* d_nitems = dctr + 5;
-  unsigned long long* d_total = (unsigned long long*)(dctr + 6);
-  uint32_t* d_ncompact = dctr + 8;
+  // A batch of at most MID_ITEM points needs no sieve: its rounds, at most
+  // the tree's height / lambda, are queued one after another on bounds of
+  // their lists' lengths, and the host reads the counters once at the end.
+  // A larger one reads them after every round, for the next round's sieve
+  // and list sizes (about 20 us each).
+  const bool queued = m <= MID_ITEM;
+  const uint32_t height = t.st_host->max_depth;  // an upper bound
+  const int max_rounds = (int)std::max<uint64_t>(1, ((uint64_t)height + lam - 1) / lam);
+  const uint32_t ctl_words = U_WORDS + (uint32_t)(max_rounds + 2) * R_WORDS;
+  uint32_t* ctl;
+  PKD_TRY(sc.get(&ctl, ctl_words));
+  PinnedBlock hblk;
+  uint32_t* hu = (uint32_t*)hblk.p;
+  if (!hu) return PKD_ENOMEM;
+  static_assert((U_WORDS + 2 * R_WORDS) * 4 <= PINNED_BLOCK, "counters");
+  auto rc = [&](int r) { return ctl + U_WORDS + (uint32_t)r * R_WORDS; };
 
-  // every routed point ends in exactly one leaf group: at most m groups
-  const uint32_t group_cap = (uint32_t)std::min<uint64_t>(m + 16, 0xFFFFFFF0ull);
-  LeafGroup* groups;
-  PKD_TRY(sc.get(&groups, group_cap));
-  RebuildItem* items_out;
-  const uint32_t items_cap = group_cap;  // at most one rebuild per routed point
-  PKD_TRY(sc.get(&items_out, items_cap));
-
-  UpdArgs ua{};
-  ua.p = p;
-  ua.lam = lam;
-  ua.NB = NB;
-  ua.HN = HN;
-  ua.TILE = TILE;
-  ua.insert = insert ? 1 : 0;
-  ua.nodes = t.nodes;
-  ua.ndim = t.ndim;
-  ua.groups = groups;
-  ua.ngroups = d_ngroups;
-  ua.group_cap = group_cap;
-  ua.items_out = items_out;
-  ua.nitems_out = d_nitems;
-  ua.items_total = d_total;
-  ua.items_max = dctr + 9;
-  ua.inner_total = (unsigned long long*)(dctr + 10);
-  ua.items_cap = items_cap;
-  ua.aux = t.aux;
-  ua.st = t.st;
+  // every routed point ends in one leaf group or rebuild item
+  const uint32_t group_cap = (uint32_t)m;
+  RouteArgs ra{};
+  ra.p = p;
+  ra.lam = lam;
+  ra.NB = NB;
+  ra.HN = HN;
+  ra.TILE = TILE;
+  ra.insert = insert ? 1 : 0;
+  ra.nodes = t.nodes;
+  ra.ndim = t.ndim;
+  ra.aux = t.aux;
+  ra.st = t.st;
+  ra.F = F;
+  ra.top = t.top;
+  ra.u = ctl;
+  ra.group_cap = ra.item_cap = group_cap;
+  PKD_TRY(sc.get(&ra.items, group_cap));
+  if (!insert) {
+    PKD_TRY(sc.get(&ra.gout, group_cap));
+    PKD_TRY(sc.get(&ra.gin, group_cap));
+  }
 
   // ---- route ----
   std::vector<RouteRound> rounds;
-  Seg root{0, (uint32_t)m, 0, t.root, IN_B};
-  Seg* cur;
-  Seg* cur_big;
-  uint32_t *cur_bigmap, *cur_small;
-  PKD_TRY(sc.get(&cur, 1));
-  PKD_TRY(sc.get(&cur_big, 1));
-  PKD_TRY(sc.get(&cur_bigmap, 1));
-  PKD_TRY(sc.get(&cur_small, 1));
-  uint32_t zero = 0;
-  PKD_TRY(dev_store(cur, &root, sizeof(Seg), s));
-  const bool root_big = m > SMALL_ITEM;
-  if (root_big) {
-    PKD_TRY(dev_store(cur_big, &root, sizeof(Seg), s));
-    PKD_TRY(dev_store(cur_bigmap, &zero, 4, s));
-  } else {
-    PKD_TRY(dev_store(cur_small, &zero, 4, s));
+  const Seg root{0, (uint32_t)m, 0, t.root, IN_B};
+  Seg* first;
+  PKD_TRY(sc.get(&first, 1));
+  uint32_t nbig = m > MID_ITEM, nmid = !nbig && m > SMALL_ITEM, nsmall = !nbig && !nmid;
+  uint32_t tiles = nbig ? (uint32_t)((m + TILE - 1) / TILE) : 0;
+  uint64_t big_pts = nbig ? m : 0;  // points the round's sieve kernels move
+  Seg *big = first, *mid = first, *small = first;
+  PKD_LAUNCH(k_update_init<<<1, 256, 0, s>>>(ctl, ctl_words, root, first,
+                                             U_WORDS + (nbig ? R_BIG : (nmid ? R_MID : R_SMALL))));
+  RouteRound all{};  // queued rounds share their lists
+  if (queued) {
+    // a point's path has at most `height` inner nodes
+    all.stay_cap = (uint32_t)(m * std::max<uint32_t>(height, 1));
+    PKD_TRY(sc.get(&all.stay, all.stay_cap));
+    if (!insert) {
+      all.aux_cap = (uint32_t)(m * (height + 1ull));
+      PKD_TRY(sc.get(&all.auxs, all.aux_cap));
+    }
+    all.ctl = rc(max_rounds + 1);
+    rounds.push_back(all);
   }
-  uint32_t ncur = 1, tiles = root_big ? (uint32_t)((m + TILE - 1) / TILE) : 0;
-  uint64_t big_pts = root_big ? m : 0;  // points the round's sieve kernels move
-  uint32_t nbig = root_big ? 1 : 0, nsmall = root_big ? 0 : 1;
-  int w = 0;
-  uint32_t groups_before = 0;
-  for (int r = 0; ncur > 0; ++r) {
-    if (r > 200) return PKD_EINTERNAL;
-    RouteRound R{};
-    R.items = cur;
-    R.n = ncur;
-    PKD_TRY(sc.get(&R.skel, (size_t)ncur * HN));
-    PKD_TRY(sc.get(&R.slots, (size_t)ncur * HN));
-    PKD_TRY(sc.get(&R.fnd, (size_t)ncur * HN));
-    PKD_TRY(sc.get(&R.nsz, (size_t)ncur * HN));
-    PKD_TRY(dev_fill(R.nsz, 0xFF, (size_t)ncur * HN * 4, s));
-    PKD_TRY(sc.get(&R.link, (size_t)ncur * NB));
-    PKD_TRY(sc.get(&R.bstart, (size_t)ncur * NB));
-    PKD_TRY(sc.get(&R.blen, (size_t)ncur * NB));
-    PKD_TRY(sc.get(&R.iflag, ncur));
-    PKD_TRY(sc.get(&R.d_n, 4));
-    uint32_t hn[4] = {ncur, nbig, nsmall, 0};
-    PKD_TRY(dev_fill(R.iflag, 0, (size_t)ncur * 4, s));
-    PKD_TRY(dev_store(R.d_n, hn, 16, s));
-    uint32_t* nbk;
-    PKD_TRY(sc.get(&nbk, ncur));
-    Seg *next, *next_big;
-    uint32_t *next_bigmap, *next_small;
-    PKD_TRY(sc.get(&next, (size_t)ncur * NB));
-    PKD_TRY(sc.get(&next_big, (size_t)ncur * NB));
-    PKD_TRY(sc.get(&next_bigmap, (size_t)ncur * NB));
-    PKD_TRY(sc.get(&next_small, (size_t)ncur * NB));
-    PKD_TRY(dev_fill(dctr, 0, 16, s));
-    PKD_TRY(dev_fill(dctr + 16, 0, 4, s));
-
-    ua.items = cur;
-    ua.nitems = R.d_n;
-    ua.skel = R.skel;
-    ua.slots = R.slots;
-    ua.nbk = nbk;
-    ua.bstart = R.bstart;
-    ua.blen = R.blen;
-    ua.link = R.link;
-    ua.fnd = R.fnd;
-    ua.iflag = R.iflag;
-    ua.next = next;
-    ua.next_ctr = dctr;
-    ua.next_big = next_big;
-    ua.next_bigmap = next_bigmap;
-    ua.next_small = next_small;
-    const unsigned g1 = item_blocks(ncur);
-    {
-      const size_t smb = (size_t)ITEM_WARPS * HN * (sizeof(int2) + sizeof(uint32_t));
-      static size_t set = 0;
-      if (smb > 48 * 1024 && set < smb) {
-        cudaFuncSetAttribute(k_fetch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
-        set = smb;
-      }
-      PKD_LAUNCH(k_fetch<<<g1, ITEM_WARPS * 32, smb, s>>>(ua));
-    }
-
-    RoundArgs ra{};
-    ra.wait_cycles = knobs().wait_cycles;
-    ra.p = p;
-    ra.lam = lam;
-    ra.NB = NB;
-    ra.HN = HN;
-    ra.TILE = TILE;
-    ra.src.soa = W[w];
-    ra.src.is_aos = 0;
-    ra.dst = W[w ^ 1];
-    ra.skel = R.skel;
-    ra.st = t.st;
-    if (nbig) {
-      // big items: tile histograms, bucket-major scan, scatter
-      uint32_t *tile0, *hist, *hscan, *partial;
-      uint64_t* excl;
-      PKD_TRY(sc.get(&tile0, nbig));
-      PKD_TRY(sc.get(&excl, nbig));
-      PKD_TRY(sc.get(&hist, (size_t)tiles * NB));
-      PKD_TRY(sc.get(&hscan, (size_t)tiles * NB));
-      const uint64_t nh = (uint64_t)tiles * NB;
-      PKD_TRY(sc.get(&partial, (nh + SCAN_TILE - 1) / SCAN_TILE + 1));
-      ra.big = cur_big;
-      ra.nbig = R.d_n + 1;
-      ra.skel_map = cur_bigmap;
-      ra.tile0 = tile0;
-      ra.excl = excl;
-      ra.hist = hist;
-      ra.hscan = hscan;
-      if (record_buckets(NB)) PKD_TRY(sc.get(&ra.bkt, (size_t)tiles * TILE));
-      PKD_LAUNCH(k_big_prefix<<<1, 1024, 0, s>>>(cur_big, R.d_n + 1, (uint32_t)TILE, tile0, excl));
-      PKD_DISPATCH_D(d, launch_count, ra, tiles, big_pts, "count_route", s);
-      device_excl_scan(hist, hscan, nh, partial, s);
-      PKD_LAUNCH(k_bucket_ranges<<<(unsigned)(((uint64_t)nbig * 32 + 127) / 128), 128, 0, s>>>(ra, R.bstart, R.blen,
-                                                                                               nbk));
-      PKD_DISPATCH_D(d, launch_scatter, ra, tiles, big_pts, "scatter_route", s);
-      PKD_LAUNCH(k_copy_round<<<tiles, 256, 0, s>>>(ra, F));
-    }
-    if (nsmall) {
-      PKD_DISPATCH_D(d, launch_route_small, ra, cur_small, R.d_n + 2, cur, nbk, R.bstart, R.blen, F, nsmall, s);
-    }
-    PKD_LAUNCH(k_route_emit<<<g1, ITEM_WARPS * 32, 0, s>>>(ua));
-    PKD_CUDA(cudaMemcpyAsync(hctr, dctr, 68, cudaMemcpyDeviceToHost, s));
-    PKD_CUDA(cudaStreamSynchronize(s));
-    const uint32_t nnext = hctr[0], ntiles = hctr[1], ngroups = hctr[4];
-    big_pts = hctr[16];
-    groups_before = ngroups;
-    rounds.push_back(R);
-    cur = next;
-    cur_big = next_big;
-    cur_bigmap = next_bigmap;
-    cur_small = next_small;
-    ncur = nnext;
-    tiles = ntiles;
-    nbig = hctr[2];
-    nsmall = hctr[3];
-    w ^= 1;
-  }
-  const uint32_t ngroups = groups_before;
-  trace_mark(s, "upd: route");
-
-  // From here on, every exit clears the delete marks this batch sets (the
-  // scratch must be zero for the next call).
+  // From here on, every exit clears the marks a delete sets (the scratch
+  // must be zero for the next call).
   struct ClearMarks {
     TreeMem& t;
     const std::vector<RouteRound>& rounds;
-    int HN;
     cudaStream_t s;
     bool on;
+    const LeafGroup* gin = nullptr;  // the groups whose points were marked
+    const uint32_t* ngin = nullptr;
+    uint32_t most = 0;
+    bool aux = true;  // the routed rounds may have set aux words
+    void clear() {
+      if (!on) return;
+      on = false;
+      if (gin) PKD_LAUNCH(k_clear_dead<<<list_blocks((uint64_t)most * 32), 256, 0, s>>>(gin, ngin, t.nodes, t.dead));
+      if (!aux) return;
+      for (const auto& R : rounds)
+        PKD_LAUNCH(k_clear_aux<<<list_blocks(R.aux_cap), 256, 0, s>>>(R.auxs, R.ctl + R_AUX, R.aux_cap, t.aux));
+    }
     ~ClearMarks() {
       if (!on) return;
-      const bool ok = dev_fill(t.dead, 0, t.cap, s) == PKD_OK;
-      for (const auto& R : rounds)
-        PKD_LAUNCH(k_clear_aux<<<(unsigned)(((uint64_t)R.n * HN + 255) / 256), 256, 0, s>>>(R.slots, (uint64_t)R.n * HN,
-                                                                                           t.aux));
-      // (a leaf group's slot is a heap bucket of its round, cleared above)
-      if (ok && cudaPeekAtLastError() == cudaSuccess) t.scratch_dirty = false;
+      clear();
+      if (cudaPeekAtLastError() == cudaSuccess) t.scratch_dirty = false;
     }
-  } clear_marks{t, rounds, HN, s, !insert};
+  } marks{t, rounds, s, !insert};
   if (!insert) t.scratch_dirty = true;
 
-  // ---- match (delete) ----
-  if (!insert && ngroups)
-    PKD_DISPATCH_D(d, launch_match, groups, d_ngroups, ngroups, t.nodes, t.A, F, t.dead, t.aux, s);
-
-  // ---- count, bottom-up ----
-  for (int r = (int)rounds.size() - 1; r >= 0; --r) {
-    RouteRound& R = rounds[r];
-    ua.items = R.items;
-    ua.nitems = R.d_n;
-    ua.skel = R.skel;
-    ua.slots = R.slots;
-    ua.link = R.link;
-    ua.fnd = R.fnd;
-    ua.next_fnd = (r + 1 < (int)rounds.size()) ? rounds[r + 1].fnd : nullptr;
-    ua.next_HN = HN;
-    {
-      const size_t smb = (size_t)ITEM_WARPS * HN * 2 * sizeof(uint32_t);
-      static size_t set = 0;
-      if (smb > 48 * 1024 && set < smb) {
-        cudaFuncSetAttribute(k_aggregate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
-        set = smb;
+  auto read_flags = [&]() {  // the tree's status, with the batch's id flags
+    PKD_CUDA(cudaMemcpyAsync(t.st_host, t.st, sizeof(DevStatus), cudaMemcpyDeviceToHost, s));
+    PKD_CUDA(cudaStreamSynchronize(s));
+    if (idflags) *idflags = t.st_host->idflags;
+    return status_code(t.st_host->err, t.st_host->detail);
+  };
+  int w = 0, r = 0;
+  for (;; ++r) {
+    const uint64_t nitems = (uint64_t)nbig + nmid + nsmall;  // or a bound
+    if (queued ? r == max_rounds : nitems == 0) break;
+    if (r > max_rounds) return PKD_EINTERNAL;
+    ra.src = W[w];
+    ra.dst = W[w ^ 1];
+    ra.next = rc(r + 1);
+    ra.last = queued && r + 1 == max_rounds;
+    ra.cur = queued ? rc(max_rounds + 1) : rc(r);
+    if (queued) {
+      ra.stay = all.stay;
+      ra.stay_cap = all.stay_cap;
+      ra.auxs = all.auxs;
+      ra.aux_cap = all.aux_cap;
+    } else {
+      RouteRound R{};
+      R.stay_cap = (uint32_t)std::min<uint64_t>(m * (uint64_t)lam, nitems * (uint64_t)(NB - 1));
+      PKD_TRY(sc.get(&R.stay, R.stay_cap));
+      if (!insert) {
+        R.aux_cap = (uint32_t)std::min<uint64_t>(m * (uint64_t)(lam + 1), nitems * (uint64_t)(HN - 1));
+        PKD_TRY(sc.get(&R.auxs, R.aux_cap));
       }
-      PKD_LAUNCH(k_aggregate<<<item_blocks(R.n), ITEM_WARPS * 32, smb, s>>>(ua));
+      R.ctl = rc(r);
+      ra.stay = R.stay;
+      ra.stay_cap = R.stay_cap;
+      ra.auxs = R.auxs;
+      ra.aux_cap = R.aux_cap;
+      rounds.push_back(R);
     }
-  }
-  uint32_t total_changed = 0;
-  PKD_CUDA(cudaMemcpyAsync(&total_changed, rounds[0].fnd + 1, 4, cudaMemcpyDeviceToHost, s));
-  uint32_t* compact;
-  PKD_TRY(sc.get(&compact, std::max<uint32_t>(ngroups, 1)));
-
-  // ---- decide, top-down (sizes of the nodes that stay are only recorded) ----
-  for (size_t r = 0; r < rounds.size(); ++r) {
-    RouteRound& R = rounds[r];
-    ua.items = R.items;
-    ua.nitems = R.d_n;
-    ua.skel = R.skel;
-    ua.slots = R.slots;
-    ua.link = R.link;
-    ua.fnd = R.fnd;
-    ua.nsz = R.nsz;
-    ua.bstart = R.bstart;
-    ua.blen = R.blen;
-    ua.iflag = R.iflag;
-    ua.next_iflag = (r + 1 < rounds.size()) ? rounds[r + 1].iflag : nullptr;
-    {
-      const size_t smb = (size_t)ITEM_WARPS * HN * (sizeof(int2) + 3 * sizeof(uint32_t));
-      static size_t set = 0;
-      if (smb > 48 * 1024 && set < smb) {
-        cudaFuncSetAttribute(k_decide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
-        set = smb;
-      }
-      PKD_LAUNCH(k_decide<<<item_blocks(R.n), ITEM_WARPS * 32, smb, s>>>(ua));
+    ra.small = ra.mid = ra.big = nullptr;
+    ra.small_cap = ra.mid_cap = ra.big_cap = 0;
+    if (!ra.last) {  // every item has NB external nodes and a point at least
+      ra.small_cap = (uint32_t)std::min<uint64_t>(m, nitems * NB);
+      ra.mid_cap = (uint32_t)std::min<uint64_t>(ra.small_cap, m / (SMALL_ITEM + 1));
+      ra.big_cap = queued ? 0 : (uint32_t)std::min<uint64_t>(ra.small_cap, m / (MID_ITEM + 1));
+      PKD_TRY(sc.get(&ra.small, ra.small_cap));
+      PKD_TRY(sc.get(&ra.mid, ra.mid_cap));
+      if (ra.big_cap) PKD_TRY(sc.get(&ra.big, ra.big_cap));
     }
+    if (nbig) {
+      // big items: fetch, tile histograms, bucket-major scan, emit, scatter
+      RoundArgs sa{};
+      uint32_t *slots, *sizes, *hist, *hscan, *partial;
+      const uint64_t nh = (uint64_t)tiles * NB;
+      PKD_TRY(sc.get(&sa.skel, (size_t)nbig * HN));
+      PKD_TRY(sc.get(&slots, (size_t)nbig * HN));
+      PKD_TRY(sc.get(&sizes, (size_t)nbig * HN));
+      PKD_TRY(sc.get(&sa.tile0, nbig));
+      PKD_TRY(sc.get(&sa.excl, nbig));
+      PKD_TRY(sc.get(&hist, nh));
+      PKD_TRY(sc.get(&hscan, nh));
+      PKD_TRY(sc.get(&partial, (nh + SCAN_TILE - 1) / SCAN_TILE + 1));
+      if (record_buckets(NB)) PKD_TRY(sc.get(&sa.bkt, (size_t)tiles * TILE));
+      ra.copy_cap = (uint32_t)(tiles + (uint64_t)nbig * NB);
+      PKD_TRY(sc.get(&ra.copy, ra.copy_cap));
+      sa.wait_cycles = knobs().wait_cycles;
+      sa.p = p;
+      sa.lam = lam;
+      sa.NB = NB;
+      sa.HN = HN;
+      sa.TILE = TILE;
+      sa.src.soa = W[w];
+      sa.dst = W[w ^ 1];
+      sa.st = t.st;
+      sa.big = big;
+      sa.nbig = rc(r) + R_BIG;
+      sa.hist = hist;
+      sa.hscan = hscan;
+      const size_t per = skel_bytes(HN, NB);
+      if (per > 48 * 1024) return PKD_EINTERNAL;  // (45 KB at lambda = 10)
+      PKD_LAUNCH(k_big_fetch<<<nbig, BIG_TEAM, per, s>>>(ra, big, sa.skel, slots, sizes));
+      PKD_LAUNCH(k_big_prefix<<<1, 1024, 0, s>>>(big, sa.nbig, (uint32_t)TILE, sa.tile0, sa.excl));
+      PKD_DISPATCH_D(d, launch_count, sa, tiles, big_pts, "count_route", s);
+      device_excl_scan(hist, hscan, nh, partial, s);
+      PKD_LAUNCH(k_big_emit<<<nbig, BIG_TEAM, per, s>>>(ra, sa, slots, sizes));
+      PKD_DISPATCH_D(d, launch_scatter, sa, tiles, big_pts, "scatter_route", s);
+      PKD_LAUNCH(k_copy_ended<<<std::min<uint32_t>(ra.copy_cap, 152 * 8), 256, 0, s>>>(ra, rc(r) + R_COPY));
+    }
+    PKD_DISPATCH_D(d, launch_route, ra, mid, rc(r) + R_MID, nmid, small, rc(r) + R_SMALL, nsmall, s);
+    if (queued) {
+      nmid = ra.mid_cap;
+      nsmall = ra.small_cap;
+    } else {
+      PKD_CUDA(cudaMemcpyAsync(hu + U_WORDS, rc(r), 2 * R_WORDS * 4, cudaMemcpyDeviceToHost, s));
+      PKD_TRY(read_flags());
+      if (idflags && *idflags) return PKD_OK;
+      const uint32_t* nx = hu + U_WORDS + R_WORDS;
+      nbig = nx[R_BIG];
+      nmid = nx[R_MID];
+      nsmall = nx[R_SMALL];
+      tiles = nx[R_TILES];
+      big_pts = nx[R_BIGPTS];
+    }
+    big = ra.big;
+    mid = ra.mid;
+    small = ra.small;
+    w ^= 1;
   }
-  trace_mark(s, "upd: match+count+decide");
-  if (ngroups) PKD_LAUNCH(k_leaf_items<<<(ngroups + 255) / 256, 256, 0, s>>>(ua, groups, d_ngroups, compact, d_ncompact));
-  PKD_CUDA(cudaMemcpyAsync(hctr, dctr, 48, cudaMemcpyDeviceToHost, s));
-  PKD_CUDA(cudaStreamSynchronize(s));
-  const uint32_t nitems = hctr[5];
-  const uint64_t total = *(unsigned long long*)(hctr + 6);
-  const uint32_t ncompact = hctr[8];
-  const uint64_t inner_total = *(unsigned long long*)(hctr + 10);
+  PKD_CUDA(cudaMemcpyAsync(hu, ctl, U_WORDS * 4, cudaMemcpyDeviceToHost, s));
+  PKD_TRY(read_flags());
+  if (idflags && *idflags) return PKD_OK;
+  const uint32_t nitems = hu[U_ITEMS], ninner = hu[U_INNER], ngout = hu[U_GOUT], ngin = hu[U_GIN];
+  const uint64_t total = *(unsigned long long*)(hu + U_TOTAL);
+  const uint64_t inner_total = *(unsigned long long*)(hu + U_INNER_PTS);
+  marks.aux = ninner != 0;
+  const uint32_t* d_nitems = ctl + U_ITEMS;
+  const RebuildItem* items = ra.items;
   stat_items(insert ? "rebuilt_insert" : "rebuilt_delete", total);
-  trace_mark(s, "upd: leaf items");
+  trace_mark(s, "upd: route");
 
   // ---- rebuild ----
   // Nothing the tree shows has changed so far: the new sizes are recorded,
-  // the leaves to compact are listed.  Every allocation of the rebuild comes
-  // first; the new subtrees are built in fresh arena positions (past top);
-  // the rebuild items' root records are saved and put back if the rebuild
-  // fails, so PKD_ENOMEM leaves the tree as it was.
+  // the leaves to compact are listed.  The new subtrees are built in fresh
+  // arena positions (past top), and every allocation, the build's included,
+  // comes before the first write to a node, so PKD_ENOMEM leaves the tree as
+  // it was.
   if (nitems) {
     PKD_TRY(ensure_capacity(t, total, s));
     trace_mark(s, "upd: ensure capacity");
-    uint32_t *isz, *ioff, *ipart, *saved_next;
-    PKD_TRY(sc.get(&isz, nitems));
-    PKD_TRY(sc.get(&ioff, nitems));
-    PKD_TRY(sc.get(&ipart, ((uint64_t)nitems + SCAN_TILE - 1) / SCAN_TILE + 1));
+    if (ngin) {  // a delete's marks in the subtrees that are rebuilt
+      PKD_TRY(ensure_dead(t, s));
+      PKD_DISPATCH_D(d, launch_delete, true, ra.gin, ctl + U_GIN, ngin, t.nodes, t.A, F, t.dead, ctl + U_FOUND, s);
+      marks.gin = ra.gin;
+      marks.ngin = ctl + U_GIN;
+      marks.most = ngin;
+    }
     Seg* segs;
     PKD_TRY(sc.get(&segs, nitems));
-    Node* saved_nodes;
-    uint8_t* saved_dims;
-    PKD_TRY(sc.get(&saved_nodes, nitems));
-    PKD_TRY(sc.get(&saved_dims, nitems));
-    PKD_TRY(sc.get(&saved_next, 1));
-    // Capacity of the flatten's lists: every node of the old subtrees
-    // appears once: a leaf item is one node, an interior item of P stored
-    // points has at most 2P - 1 nodes unless deletes left empty leaves in it.
-    // The first attempt is sized by that (an insert's items are mostly
-    // leaves); when a level overflows it, the flatten is redone with four
-    // entries per stored point of the tree.
-    const uint64_t big_fcap = 4 * ((uint64_t)t.size + (uint64_t)nitems) + 1024;
-    uint64_t fcap = 2 * inner_total + (uint64_t)nitems + 1024;
-    if (knobs().front_cap > 0) fcap = (uint64_t)knobs().front_cap;
-    fcap = std::max<uint64_t>(std::min(fcap, big_fcap), (uint64_t)nitems + 1024);  // the roots always fit
-    Front *fa = nullptr, *fb = nullptr, *leaves = nullptr, *bigleaves = nullptr;
-    uint32_t *ncnt = nullptr, *noff = nullptr, *npart = nullptr;
-    if (insert) {
+    const unsigned gi = (nitems + 127) / 128;
+    PKD_DISPATCH_D(d, launch_copy_items, items, d_nitems, nitems, t.nodes, F, t.A, segs, (uint32_t)p.phi, s);
+    if (hu[U_MAXNEW] > NEW_BIG) {
+      uint32_t *ncnt, *noff, *npart;
       PKD_TRY(sc.get(&ncnt, nitems));
       PKD_TRY(sc.get(&noff, nitems));
       PKD_TRY(sc.get(&npart, ((uint64_t)nitems + SCAN_TILE - 1) / SCAN_TILE + 1));
+      PKD_LAUNCH(k_item_newcounts<<<gi, 128, 0, s>>>(items, d_nitems, ncnt));
+      device_excl_scan(ncnt, noff, nitems, npart, s);
+      PKD_DISPATCH_D(d, launch_copy_new_flat, items, d_nitems, noff, ncnt, m, F, t.A, s);
     }
-    const unsigned gi = (nitems + 127) / 128;
-    PKD_LAUNCH(k_item_sizes<<<gi, 128, 0, s>>>(items_out, d_nitems, isz));
-    device_excl_scan(isz, ioff, nitems, ipart, s);
-    PKD_LAUNCH(k_item_pos<<<gi, 128, 0, s>>>(items_out, d_nitems, ioff, t.top, segs, (uint32_t)p.phi));
-    // flatten the old subtrees breadth first (capacity: every node of the
-    // old subtrees appears once).  The levels run in batches whose counts
-    // stay on the device; the host reads the frontier once per batch: one
-    // level first (an insert's items are mostly leaves), then FRONT_BATCH
-    // levels at a time (a rebuilt interior subtree is many levels deep).
-    {
-      uint32_t* fc = dctr + 12;  // [0] frontier, [1] overflow, [2] leaves, [3] big leaves
-      uint32_t* lc;              // the frontier of every level of a batch
+    if (ninner) {
+      // Flatten the old subtrees that are not single leaves, breadth first.
+      // Capacity of the lists: every node of the old subtrees appears once: a
+      // subtree of P stored points has at most 2P - 1 nodes unless deletes
+      // left empty leaves in it.  When a level overflows that, the flatten is
+      // redone with four entries per stored point of the tree.  The levels run
+      // in batches whose counts stay on the device; the host reads the
+      // frontier once per batch (a rebuilt subtree is many levels deep).
+      const uint64_t big_fcap = 4 * ((uint64_t)t.size + (uint64_t)nitems) + 1024;
+      uint64_t fcap = 2 * inner_total + (uint64_t)ninner + 1024;
+      if (knobs().front_cap > 0) fcap = (uint64_t)knobs().front_cap;
+      fcap = std::max<uint64_t>(std::min(fcap, big_fcap), (uint64_t)ninner + 1024);  // the roots always fit
+      Front *fa = nullptr, *fb = nullptr, *leaves = nullptr, *bigleaves = nullptr;
+      uint32_t* fc;  // [0] frontier, [1] overflow, [2] leaves, [3] big leaves
+      uint32_t* lc;  // the frontier of every level of a batch
+      PKD_TRY(sc.get(&fc, 4));
       PKD_TRY(sc.get(&lc, FRONT_BATCH + 1));
       const unsigned gexp = (unsigned)sm_count() * 8;
-      for (int attempt = 0;; ++attempt) {
+      uint32_t* hf = hu + U_WORDS;
+      for (;;) {
         const uint32_t fcap32 = (uint32_t)std::min<uint64_t>(fcap, 0xFFFFFFF0ull);
-        const uint32_t bcap32 = (uint32_t)std::min<uint64_t>(fcap / BIG_LEAF + 16, 0xFFFFFFF0ull);
+        const uint32_t bcap32 = (uint32_t)std::min<uint64_t>(fcap / BIG_LEAF + 16 + ninner, 0xFFFFFFF0ull);
         PKD_TRY(sc.get(&fa, fcap32));
         PKD_TRY(sc.get(&fb, fcap32));
         PKD_TRY(sc.get(&leaves, fcap32));
         PKD_TRY(sc.get(&bigleaves, bcap32));
         PKD_TRY(dev_fill(fc, 0, 16, s));
-        PKD_LAUNCH(k_front_init<<<gi, 128, 0, s>>>(items_out, d_nitems, fa, fc));
+        PKD_LAUNCH(k_front_init<<<gi, 128, 0, s>>>(items, d_nitems, fa, fc));
         int levels = 0;
-        for (int batch = 1;; batch = FRONT_BATCH) {
+        do {
           if (levels > 100000) return PKD_EINTERNAL;
-          PKD_TRY(dev_fill(lc + 1, 0, (size_t)batch * 4, s));
+          PKD_TRY(dev_fill(lc + 1, 0, (size_t)FRONT_BATCH * 4, s));
           PKD_TRY(dev_copy_words(lc, fc, 1, s));
-          for (int k = 0; k < batch; ++k) {
+          for (int k = 0; k < FRONT_BATCH; ++k) {
             PKD_LAUNCH(k_front_expand<<<gexp, 128, 0, s>>>(fa, lc + k, fb, lc + k + 1, leaves, fc + 2, bigleaves,
                                                             fc + 3, t.nodes, t.ndim, t.aux, insert ? 0 : 1, fcap32,
                                                             bcap32, fc + 1));
             std::swap(fa, fb);
           }
-          levels += batch;
-          PKD_TRY(dev_copy_words(fc, lc + batch, 1, s));
-          PKD_CUDA(cudaMemcpyAsync(hctr + 12, fc, 16, cudaMemcpyDeviceToHost, s));
+          levels += FRONT_BATCH;
+          PKD_TRY(dev_copy_words(fc, lc + FRONT_BATCH, 1, s));
+          PKD_CUDA(cudaMemcpyAsync(hf, fc, 16, cudaMemcpyDeviceToHost, s));
           PKD_CUDA(cudaStreamSynchronize(s));
-          if (hctr[12] == 0 || hctr[13] != 0) break;
-        }
-        if (hctr[13] == 0) break;
+        } while (hf[0] != 0 && hf[1] == 0);
+        if (hf[1] == 0) break;
         // a list overflowed: nothing the tree shows has changed yet
         if (fcap >= big_fcap) return PKD_EINTERNAL;
         stat_items("front_retries", 1);
         fcap = big_fcap;
       }
-      const uint32_t nleaves = hctr[14], nbigleaves = hctr[15];
-      if (nleaves)
-        PKD_DISPATCH_D(d, launch_copy_leaves, leaves, fc + 2, nleaves, items_out, t.nodes, t.A, t.dead,
-                       insert ? 0 : 1, s);
-      if (nbigleaves)
-        PKD_DISPATCH_D(d, launch_copy_big_leaves, bigleaves, fc + 3, nbigleaves, items_out, t.nodes, t.A, t.dead,
-                       insert ? 0 : 1, s);
-    }
-    if (insert) {
-      PKD_DISPATCH_D(d, launch_copy_new, items_out, d_nitems, nitems, F, t.A, s);
-      PKD_LAUNCH(k_item_newcounts<<<gi, 128, 0, s>>>(items_out, d_nitems, ncnt));
-      device_excl_scan(ncnt, noff, nitems, npart, s);
-      PKD_DISPATCH_D(d, launch_copy_new_flat, items_out, d_nitems, noff, ncnt, m, F, t.A, s);
+      if (hf[2])
+        PKD_DISPATCH_D(d, launch_copy_leaves, leaves, fc + 2, hf[2], items, t.nodes, t.A, t.dead, ngin ? 1 : 0, s);
+      if (hf[3])
+        PKD_DISPATCH_D(d, launch_copy_big_leaves, bigleaves, fc + 3, hf[3], items, t.nodes, t.A, t.dead, ngin ? 1 : 0,
+                       s);
     }
     trace_mark(s, "upd: flatten + gather");
-    PKD_LAUNCH(k_save_roots<<<gi, 128, 0, s>>>(items_out, d_nitems, t.nodes, t.ndim, saved_nodes, saved_dims));
-    PKD_TRY(dev_copy_words(saved_next, t.shared_next, 1, s));
     BuildJob job;
     job.base = t.top;
     job.extent = std::max<uint64_t>(total, 1);
     job.dsegs = segs;
     job.dsegs_n = nitems;
-    job.max_len = hctr[9];
-    const int eb = run_build(t, job, s);
-    if (eb != PKD_OK) {
-      PKD_LAUNCH(k_restore_roots<<<gi, 128, 0, s>>>(items_out, d_nitems, t.nodes, t.ndim, saved_nodes, saved_dims));
-      dev_copy_words(t.shared_next, saved_next, 1, s);
-      return eb;
-    }
-    PKD_LAUNCH(k_item_leaves<<<gi, 128, 0, s>>>(items_out, d_nitems, t.nodes, t.ndim, (uint32_t)p.phi));
+    job.max_len = hu[U_MAX];
+    PKD_TRY(run_build(t, job, s));
+    PKD_LAUNCH(k_item_leaves<<<gi, 128, 0, s>>>(items, d_nitems, t.nodes, t.ndim, (uint32_t)p.phi));
     trace_mark(s, "upd: rebuild");
   }
 
   // ---- the visible changes: nothing below allocates ----
-  if (ncompact)  // delete: the reached leaves lose their deleted points
-    PKD_DISPATCH_D(d, launch_compact, groups, compact, d_ncompact, ncompact, t.nodes, t.A, t.dead, s);
+  if (ngout)  // delete: the reached leaves lose their deleted points
+    PKD_DISPATCH_D(d, launch_delete, false, ra.gout, ctl + U_GOUT, ngout, t.nodes, t.A, F, nullptr, ctl + U_FOUND, s);
   for (const auto& R : rounds)
-    PKD_LAUNCH(k_apply_sizes<<<(unsigned)(((uint64_t)R.n * HN + 255) / 256), 256, 0, s>>>(R.slots, R.nsz,
-                                                                                         (uint64_t)R.n * HN, t.nodes));
+    PKD_LAUNCH(k_apply_sizes<<<list_blocks(R.stay_cap), 256, 0, s>>>(R.stay, R.ctl + R_STAY, R.stay_cap, t.nodes));
   t.top += total;
-  clear_marks.on = false;
-  if (!insert) {
-    PKD_TRY(dev_fill(t.dead, 0, t.cap, s));
-    for (auto& R : rounds)
-      PKD_LAUNCH(k_clear_aux<<<(unsigned)(((uint64_t)R.n * HN + 255) / 256), 256, 0, s>>>(R.slots, (uint64_t)R.n * HN, t.aux));
-  }
-  PKD_CUDA(cudaStreamSynchronize(s));
+  marks.clear();
+  PKD_CUDA(cudaMemcpyAsync(hu, ctl, U_WORDS * 4, cudaMemcpyDeviceToHost, s));
+  const int e = read_flags();  // waits for everything
   if (!insert && cudaPeekAtLastError() == cudaSuccess) t.scratch_dirty = false;  // every mark is cleared
   trace_mark(s, "upd: cleanup");
-  if (n_changed) *n_changed = total_changed;
-  return PKD_OK;
+  if (n_changed) *n_changed = insert ? m : hu[U_FOUND];
+  return e;
 }
 
 }  // namespace pkd
@@ -1760,23 +1057,26 @@ int pkd_batch_insert(pkd_tree* tc, const int32_t* coords, const uint32_t* ids, u
   if (t.size + m >= (1ull << 31)) return PKD_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
   TreeTouch touch{&t, s};
-  bool ok;
-  PKD_TRY_(validate_coords(coords, m * (uint64_t)t.p.d, s, &ok));
-  if (!ok) return PKD_EINVAL;
-  PKD_TRY_(check_status(t, s));
+  {
+    QueryCheck check(t, s);
+    PKD_TRY_(check.begin(coords, m * (uint64_t)t.p.d, nullptr, 0));
+    PKD_TRY_(check.end());
+  }
   // the batch's ids take their slots first: a stored or repeated id rejects
-  // the whole batch before the tree changes
+  // the whole batch before the tree changes (the flags are read with the
+  // route's counters)
   PKD_TRY_(ids_reserve(t, m, s));
   uint64_t* slots = nullptr;
   PKD_TRY_(dalloc(&slots, m, s));
   ids_claim(t, coords, ids, m, slots, s);
   t.ids.used += m;
   int fl = 0;
-  int e = read_idflags(t, s, &fl);
-  if (e == PKD_OK && fl) e = (fl & IDF_FULL) ? PKD_EINTERNAL : PKD_EINVAL;
-  uint64_t changed = 0;
-  if (e == PKD_OK) e = run_update(t, coords, ids, nullptr, m, true, &changed, s);
-  if (e == PKD_OK) e = check_status(t, s);
+  int e = run_update(t, coords, ids, nullptr, m, true, nullptr, &fl, s);
+  if (e != PKD_OK || fl) {  // the flags, read and cleared: a bad batch is told as such
+    const int ec = read_idflags(t, s, &fl);
+    if (fl && (e == PKD_OK || e == PKD_ENOMEM)) e = (fl & IDF_FULL) ? PKD_EINTERNAL : PKD_EINVAL;
+    if (ec != PKD_OK) e = ec;
+  }
   if (e == PKD_OK) {
     t.size += m;
     t.ids.live += m;
@@ -1797,7 +1097,6 @@ int pkd_batch_delete(pkd_tree* tc, const uint32_t* ids, uint64_t m, uint64_t* n_
   if (m >= (1ull << 31)) return PKD_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
   TreeTouch touch{&t, s};
-  PKD_TRY_(check_status(t, s));
   // ids -> coordinates: every LIVE id of the batch is taken once (repeats and
   // unknown or deleted ids are skipped) and staged for the sieve
   Scratch sc{s, {}};
@@ -1817,6 +1116,7 @@ int pkd_batch_delete(pkd_tree* tc, const uint32_t* ids, uint64_t m, uint64_t* n_
   PKD_CUDA(cudaMemcpyAsync(hb.p, cnt, 4, cudaMemcpyDeviceToHost, s));
   int fl = 0;
   PKD_TRY(read_idflags(t, s, &fl));  // synchronises s
+  PKD_TRY(status_code(t.st_host->err, t.st_host->detail));
   const uint32_t taken = *(const uint32_t*)hb.p;
   if (fl) {
     ids_restore(t, wslots, taken, s);
@@ -1825,8 +1125,7 @@ int pkd_batch_delete(pkd_tree* tc, const uint32_t* ids, uint64_t m, uint64_t* n_
   stat_items("delete_gather", taken);
   if (taken == 0) return PKD_OK;
   uint64_t removed = 0;
-  int e = run_update(t, nullptr, nullptr, &W, taken, false, &removed, s);
-  if (e == PKD_OK) e = check_status(t, s);
+  int e = run_update(t, nullptr, nullptr, &W, taken, false, &removed, nullptr, s);
   if (e == PKD_OK && removed != taken) {
     fprintf(stderr, "pkd: delete removed %llu points for %u live ids\n", (unsigned long long)removed, taken);
     e = PKD_EINTERNAL;
