@@ -25,6 +25,12 @@
 // sieve for every item above SMALL_ITEM) were bound by the latency of their
 // dependent loads, and a batch of a thousand points took 17 launches and a
 // host read per round.
+//
+// What bounds it: the chain of lambda dependent node loads of an item, hidden
+// by 32 warps per SM (64 registers), and the instructions around them.  The
+// last round of 1e7 random points in 1e8 (262144 items of 38 points): 0.64 ms;
+// the round before (4096 items of 2441): 0.35 ms.  Four passes: 0.9-1.2 ms and
+// 0.5 ms with the sieve.
 #pragma once
 
 #include "sieve_tma.cuh"
@@ -37,15 +43,15 @@ struct LeafGroup {
   uint64_t start;  // the first of them (position in F)
 };
 
-struct RebuildItem {
+struct __align__(16) RebuildItem {  // (arena and batch positions are below 2^31)
   uint32_t slot;
   uint32_t depth;
   uint32_t size;      // points after the update
   uint32_t old_live;  // stored points that remain
-  uint64_t ws, we;    // batch points (insert) in F
-  uint64_t pos;       // arena position assigned
+  uint32_t pos;       // arena position assigned
+  uint32_t ws;        // the first of its batch points (insert) in F
+  uint32_t nw;        // their number
   uint32_t leaf;      // 1: the old subtree is a leaf of at most BIG_LEAF points
-  uint32_t pad;
 };
 
 // Leaves of more than BIG_LEAF points are copied one block each.
@@ -55,14 +61,16 @@ constexpr uint32_t SMALL_ITEM = 256;  // one warp, 8 points a lane
 constexpr uint32_t MID_ITEM = 4096;   // one CTA of MID_TEAM threads, 16 points each
 constexpr int MID_TEAM = 256, BIG_TEAM = 128, WARP_TEAMS = 4;
 constexpr uint32_t ITEM_FLAG = 0x80000000u;  // in a Seg's depth: inside a rebuilt subtree
-constexpr uint32_t CONT_FLAG = 0x80000000u;  // in a count: the node's points go on
+constexpr int CONT_FLAG = 0x100;             // in an external entry's x: its points go on
 
 // Counters of an update (U_*) and of a round (R_*), 32-bit words on the device.
 enum : int {
-  U_ITEMS = 0, U_INNER = 1, U_TOTAL = 2 /* u64 */, U_INNER_PTS = 4 /* u64 */, U_MAX = 6, U_MAXNEW = 7,
+  U_INNER = 0, U_TOTAL = 2 /* u64: items << 32 | their points */, U_ITEMS = 3, U_INNER_PTS = 4 /* u64 */, U_MAX = 6, U_MAXNEW = 7,
   U_GOUT = 8, U_GIN = 9, U_FOUND = 10, U_WORDS = 16
 };
 enum : int { R_BIG = 0, R_MID = 1, R_SMALL = 2, R_TILES = 3, R_BIGPTS = 4, R_STAY = 5, R_AUX = 6, R_COPY = 7, R_WORDS = 8 };
+// The blocks of counters lie 128 bytes apart: atomics on one line serialise.
+constexpr uint32_t CTL_STRIDE = 32;
 
 struct RouteArgs {
   Params p;
@@ -97,20 +105,18 @@ struct Skel {
   int2* sk;         // split (internal) or split dimension (external), meta
   uint32_t* sl;     // node slot
   uint32_t* sz;     // node size
-  uint32_t* f;      // batch points below
   uint32_t* st;     // batch points before the position
   uint32_t* under;  // bits: inside a subtree that is rebuilt
 };
 __host__ __device__ inline size_t skel_bytes(int HN, int NB) {
-  return (size_t)HN * 20 + (size_t)NB * 4 + (size_t)(HN < 128 ? 4 : HN / 32) * 4;
+  return (size_t)HN * 16 + (size_t)NB * 4 + (size_t)(HN < 128 ? 4 : HN / 32) * 4;
 }
 __device__ __forceinline__ Skel skel_at(unsigned char* p, int HN, int NB) {
   Skel S;
   S.sk = (int2*)p;
   S.sl = (uint32_t*)(S.sk + HN);
   S.sz = S.sl + HN;
-  S.f = S.sz + HN;
-  S.st = S.f + HN;
+  S.st = S.sz + HN;
   S.under = S.st + NB;
   return S;
 }
@@ -129,6 +135,13 @@ __device__ __forceinline__ int heap_level(int v) { return 31 - __clz(v); }
 __device__ __forceinline__ int heap_pos(int v, int lam) {
   const int j = heap_level(v);
   return (v - (1 << j)) << (lam - j);
+}
+
+// Batch points below heap entry v of an item of `len` points: the starts of the
+// positions below it are consecutive.
+__device__ __forceinline__ uint32_t heap_count(const Skel& S, int v, int lam, uint32_t len) {
+  const int lo = heap_pos(v, lam), hi = lo + (1 << (lam - heap_level(v)));
+  return (hi == (1 << lam) ? len : S.st[hi]) - S.st[lo];
 }
 
 // Nodes of one skeleton level: every defined heap entry is loaded; one that
@@ -160,10 +173,7 @@ __device__ __forceinline__ bool skel_level(const RouteArgs& a, const Skel& S, in
 
 template <int T>
 __device__ __forceinline__ void skel_clear(const RouteArgs& a, const Skel& S) {
-  for (int v = team_rank<T>(); v < a.HN; v += T) {
-    S.sk[v] = make_int2(0, sk_meta(SK_NONE, 0, 0));
-    S.f[v] = 0;
-  }
+  for (int v = team_rank<T>(); v < a.HN; v += T) S.sk[v] = make_int2(0, sk_meta(SK_NONE, 0, 0));
   for (int b = team_rank<T>(); b < a.NB; b += T) S.st[b] = 0;
   for (int w = team_rank<T>(); w < max(4, a.HN / 32); w += T) S.under[w] = 0;
 }
@@ -172,262 +182,266 @@ __device__ __forceinline__ void skel_clear(const RouteArgs& a, const Skel& S) {
 // needed any more).
 enum : int { ACT_NONE = 0, ACT_STAY = 1, ACT_AUX = 2, ACT_REBUILD = 3 };
 
-// With the points of every external entry in f and the positions' starts in
-// st: counts bottom-up, the balance test top-down, and everything the item
-// emits.  On return f[v] of an external entry has CONT_FLAG when its points
-// go on to another round.
+// With the positions' starts in st: the balance test of every internal entry,
+// and everything the item emits.  On return the x of an external entry has
+// CONT_FLAG when its points go on to another round.
 template <int T>
-__device__ __forceinline__ void route_tail(const RouteArgs& a, const Skel& S, const Seg& it, bool is_big) {
+__device__ __forceinline__ void route_tail(const RouteArgs& a, const Skel& S, const Seg& it, uint2& seen,
+                                           bool is_big) {
   const int tid = team_rank<T>();
   const bool ins = a.insert != 0;
   const uint32_t depth0 = it.depth & ~ITEM_FLAG;
-  for (int j = a.lam - 1; j >= 0; --j) {
-    for (int v = (1 << j) + tid; v < (2 << j); v += T)
-      if (sk_state(S.sk[v].y) == SK_INTERNAL) S.f[v] = S.f[2 * v] + S.f[2 * v + 1];
-    team_sync<T>();
-  }
-  if (tid == 0 && (it.depth & ITEM_FLAG)) S.under[0] |= 2u;
-  team_sync<T>();
-  for (int j = 0; j < a.lam; ++j) {
-    for (int v = (1 << j) + tid; v < (2 << j); v += T) {
-      if (sk_state(S.sk[v].y) != SK_INTERNAL) continue;
-      const uint32_t c = S.f[v];
-      int act = ACT_NONE;
-      if (c) {
-        const int c0 = 2 * v;  // the children share a word of `under`
-        if ((S.under[v >> 5] >> (v & 31)) & 1u) {
-          act = ins ? ACT_NONE : ACT_AUX;
-          atomicOr(&S.under[c0 >> 5], 3u << (c0 & 31));
-        } else {
-          const uint32_t N = ins ? S.sz[v] + c : S.sz[v] - c;
-          const uint32_t L = ins ? S.sz[c0] + S.f[c0] : S.sz[c0] - S.f[c0];
-          if (N > 0 && is_balanced(L, N, a.p.alpha_num, a.p.alpha_den)) {
-            act = ACT_STAY;
-          } else {
-            act = ACT_REBUILD;
-            atomicOr(&S.under[c0 >> 5], 3u << (c0 & 31));
-          }
-        }
-      }
-      S.sk[v].x = act;
+  // all tests at once: a rebuilt node (rare) covers the ones below it afterwards
+  bool fix = (it.depth & ITEM_FLAG) != 0;
+  for (int v = 1 + tid; v < a.NB; v += T) {
+    if (sk_state(S.sk[v].y) != SK_INTERNAL) continue;
+    const uint32_t c = heap_count(S, v, a.lam, it.len);
+    int act = ACT_NONE;
+    if (c) {
+      const uint32_t lc = heap_count(S, 2 * v, a.lam, it.len);
+      const uint32_t N = ins ? S.sz[v] + c : S.sz[v] - c;
+      const uint32_t L = ins ? S.sz[2 * v] + lc : S.sz[2 * v] - lc;
+      act = N > 0 && is_balanced(L, N, a.p.alpha_num, a.p.alpha_den) ? ACT_STAY : ACT_REBUILD;
+      fix |= act == ACT_REBUILD;
     }
-    team_sync<T>();
+    S.sk[v].x = act;
   }
-  // Emission, a warp at a time over 32 * PER heap entries: one atomic per
-  // counter for all of them, on different lanes so that they overlap.
-  constexpr int PER = 4;
+  if constexpr (T == 32) {
+    fix = __any_sync(FULL_MASK, fix);
+    __syncwarp();
+  } else {
+    fix = __syncthreads_or(fix);
+  }
+  if (fix) {
+    if (tid == 0 && (it.depth & ITEM_FLAG)) S.under[0] |= 2u;
+    team_sync<T>();
+    for (int j = 0; j < a.lam; ++j) {
+      for (int v = (1 << j) + tid; v < (2 << j); v += T) {
+        if (sk_state(S.sk[v].y) != SK_INTERNAL || S.sk[v].x == ACT_NONE) continue;
+        const bool und = (S.under[v >> 5] >> (v & 31)) & 1u;
+        if (und) S.sk[v].x = ins ? ACT_NONE : ACT_AUX;
+        if (und || S.sk[v].x == ACT_REBUILD) atomicOr(&S.under[(2 * v) >> 5], 3u << ((2 * v) & 31));
+      }
+      team_sync<T>();
+    }
+  }
+  // Emission, a warp at a time over its share of the heap, in two passes: the
+  // totals, one atomic per counter for all of them (on different lanes, so that
+  // they overlap), then the entries.  Appending through one counter serialises
+  // at its address (about 1.3 ns each): with an update of every counter per 64
+  // heap entries the last round of a 1e7-point insert took 1.35 ms, now 0.64.
   const int lane = lane_id();
-  const int w = T == 32 ? 0 : warp_id();
+  const int step = 32 * (T / 32), vw = T == 32 ? 0 : 32 * warp_id();
   const unsigned lt = lanemask_lt();
-  for (int v0 = 32 * PER * w; v0 < a.HN; v0 += 32 * PER * (T / 32)) {
-    uint32_t len[PER], size[PER];
-    // lists: 0 rebuild items, 1 small, 2 mid, 3 big, 4 gout, 5 gin, 6 stay, 7 aux
-    int kind[PER];
-    bool inner[PER], aux[PER];
-    uint32_t nsz = 0, imax = 0, nmax = 0, tiles = 0, bpts = 0, ninner = 0;
-    unsigned long long ipts = 0;
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-      const int v = v0 + 32 * u + lane;
-      kind[u] = -1;
-      len[u] = size[u] = 0;
-      inner[u] = aux[u] = false;
-      if (v < 1 || v >= a.HN) continue;
-      const int2 e = S.sk[v];
-      const int st = sk_state(e.y);
-      if (st == SK_NONE) continue;
-      len[u] = S.f[v];
-      if (len[u] == 0) continue;
-      const uint32_t old = S.sz[v];
-      if (st == SK_INTERNAL) {
-        if (e.x == ACT_REBUILD) {
-          kind[u] = 0;
-          size[u] = ins ? old + len[u] : old - len[u];
-          inner[u] = true;
-          ipts += old;
-        } else if (e.x == ACT_STAY) {
-          kind[u] = 6;
-          size[u] = ins ? old + len[u] : old - len[u];
-        } else if (e.x == ACT_AUX) {
-          aux[u] = true;
-        }
-        continue;
+  // What heap entry v emits: a list (kind), its points, a size.
+  //   0 rebuild items, 1 small, 2 mid, 3 big, 4 gout, 5 gin, 6 stay
+  struct Out {
+    int kind;
+    bool inner, aux;
+    uint32_t len, size;
+  };
+  auto what = [&](int v) {
+    Out o{-1, false, false, 0, 0};
+    if (v < 1 || v >= a.HN) return o;
+    const int2 e = S.sk[v];
+    const int st = sk_state(e.y);
+    if (st == SK_NONE || (st == SK_INTERNAL && e.x == ACT_NONE)) return o;
+    o.len = heap_count(S, v, a.lam, it.len);
+    if (o.len == 0) return o;
+    const uint32_t old = S.sz[v];
+    if (st == SK_INTERNAL) {
+      if (e.x == ACT_AUX) {
+        o.aux = true;
+      } else {
+        o.kind = e.x == ACT_STAY ? 6 : 0;
+        o.size = ins ? old + o.len : old - o.len;
+        o.inner = true;
       }
-      const bool und = (S.under[v >> 5] >> (v & 31)) & 1u;
-      if (ins && und) continue;  // the rebuilt subtree takes the range as it is
-      if (e.x == PKD_LEAF) {
-        if (ins) {
-          kind[u] = 0;
-          size[u] = old + len[u];
-          inner[u] = old > BIG_LEAF;
-        } else {
-          kind[u] = und ? 5 : 4;
-          aux[u] = und;
-        }
-        continue;
-      }
-      kind[u] = len[u] > MID_ITEM ? 3 : (len[u] > SMALL_ITEM ? 2 : 1);
-      S.f[v] = len[u] | CONT_FLAG;
-      if (kind[u] == 3) {
-        tiles += (len[u] + a.TILE - 1) / a.TILE;
-        bpts += len[u];
-      }
+      return o;
     }
-    uint32_t tot[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) tot[k] = 0;
-    bool anything = false;
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-      if (kind[u] == 0) {
-        nsz += size[u];
-        imax = max(imax, size[u]);
-        nmax = max(nmax, ins ? len[u] : 0u);
-        ninner += inner[u];
+    const bool und = (S.under[v >> 5] >> (v & 31)) & 1u;
+    if (ins && und) return o;  // the rebuilt subtree takes the range as it is
+    if (e.x == PKD_LEAF) {
+      if (ins) {
+        o.kind = 0;
+        o.size = old + o.len;
+        o.inner = old > BIG_LEAF;
+      } else {
+        o.kind = und ? 5 : 4;
+        o.aux = und;
       }
-      anything |= kind[u] >= 0 || aux[u] || (is_big && len[u]);
+    } else {
+      o.kind = o.len > MID_ITEM ? 3 : (o.len > SMALL_ITEM ? 2 : 1);
     }
-    if (!__any_sync(FULL_MASK, anything)) continue;
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-#pragma unroll
-      for (int k = 0; k < 7; ++k) tot[k] += __popc(__ballot_sync(FULL_MASK, kind[u] == k));
-      tot[7] += __popc(__ballot_sync(FULL_MASK, aux[u]));
+    return o;
+  };
+  uint32_t nsz = 0, imax = 0, nmax = 0, tiles = 0, bpts = 0, ninner = 0;
+  unsigned long long ipts = 0, cnt = 0;  // cnt: a byte per list, 7: aux words
+  for (int v0 = vw; v0 < a.HN; v0 += step) {
+    const Out o = what(v0 + lane);
+    if (o.kind >= 0) cnt += 1ull << (8 * o.kind);
+    if (o.aux) cnt += 1ull << 56;
+    if (o.kind == 0) {
+      nsz += o.size;
+      imax = max(imax, o.size);
+      if (ins) nmax = max(nmax, o.len);
+      ninner += o.inner;
+      if (sk_state(S.sk[v0 + lane].y) == SK_INTERNAL) ipts += S.sz[v0 + lane];
+    } else if (o.kind == 3) {
+      tiles += (o.len + a.TILE - 1) / a.TILE;
+      bpts += o.len;
     }
-    uint32_t incl = 0, first = 0;
-    unsigned long long pos0 = 0;
-    if (tot[0]) {
-      incl = (uint32_t)warp_incl_scan((int)nsz);
-      imax = __reduce_max_sync(FULL_MASK, imax);
-      nmax = __reduce_max_sync(FULL_MASK, nmax);
-      ninner = __reduce_add_sync(FULL_MASK, ninner);
+  }
+  unsigned present = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if ((cnt >> (8 * k)) & 0xFFu) present |= 1u << k;
+  present = __reduce_or_sync(FULL_MASK, present);
+  uint32_t amount = 0;  // lane k: entries of list k
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    if (!((present >> k) & 1u)) continue;  // warp-uniform
+    const uint32_t t = __reduce_add_sync(FULL_MASK, (uint32_t)(cnt >> (8 * k)) & 0xFFu);
+    if (lane == k) amount = t;
+  }
+  uint32_t first = 0, pos32 = 0;
+  if (present & 1u) {
+    nsz = __reduce_add_sync(FULL_MASK, nsz);
+    imax = __reduce_max_sync(FULL_MASK, imax);
+    nmax = __reduce_max_sync(FULL_MASK, nmax);
+    ninner = __reduce_add_sync(FULL_MASK, ninner);
+    if (ninner) {
       for (int o = 16; o; o >>= 1) ipts += __shfl_xor_sync(FULL_MASK, ipts, o);
-      const uint32_t all = __shfl_sync(FULL_MASK, incl, 31);
-      if (lane == 8) pos0 = atomicAdd((unsigned long long*)(a.u + U_TOTAL), (unsigned long long)all);
-      if (lane == 9 && ipts) atomicAdd((unsigned long long*)(a.u + U_INNER_PTS), ipts);
-      if (lane == 10) atomicMax(a.u + U_MAX, imax);
-      if (lane == 11 && nmax) atomicMax(a.u + U_MAXNEW, nmax);
-      if (lane == 12 && ninner) atomicAdd(a.u + U_INNER, ninner);
+      if (lane == 9) atomicAdd((unsigned long long*)(a.u + U_INNER_PTS), ipts);
+      if (lane == 10) atomicAdd(a.u + U_INNER, ninner);
     }
-    if (tot[3]) {
-      tiles = __reduce_add_sync(FULL_MASK, tiles);
-      bpts = __reduce_add_sync(FULL_MASK, bpts);
-      if (lane == 13) atomicAdd(a.next + R_TILES, tiles);
-      if (lane == 14) atomicAdd(a.next + R_BIGPTS, bpts);
+    // the maxima seldom grow: only what this warp has not sent yet
+    if (imax > seen.x) {
+      seen.x = imax;
+      if (lane == 11) atomicMax(a.u + U_MAX, imax);
     }
-    {
-      uint32_t n = 0;
-      uint32_t* c = nullptr;
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (lane == k) n = tot[k];
-      switch (lane) {
-        case 0: c = a.u + U_ITEMS; break;
-        case 1: c = a.next + R_SMALL; break;
-        case 2: c = a.next + R_MID; break;
-        case 3: c = a.next + R_BIG; break;
-        case 4: c = a.u + U_GOUT; break;
-        case 5: c = a.u + U_GIN; break;
-        case 6: c = a.cur + R_STAY; break;
-        case 7: c = a.cur + R_AUX; break;
-        default: break;
-      }
-      if (n) first = atomicAdd(c, n);
-      if (n) {  // the lists hold every entry by construction
-        const uint32_t cap = lane == 0 ? a.item_cap : lane == 1 ? a.small_cap : lane == 2 ? a.mid_cap
-                             : lane == 3 ? a.big_cap : lane <= 5 ? a.group_cap : lane == 6 ? a.stay_cap : a.aux_cap;
-        if (first + n > cap || first + n < first) {
-          set_error(a.st, DERR_CAPACITY, 800 + lane);
-          first = 0xFFFFFFFFu;
-        }
-        if (a.last && lane >= 1 && lane <= 3) {
-          set_error(a.st, DERR_STATE, 820 + lane);
-          first = 0xFFFFFFFFu;
-        }
-      }
+    if (nmax > seen.y) {
+      seen.y = nmax;
+      if (lane == 12) atomicMax(a.u + U_MAXNEW, nmax);
     }
-    uint32_t at[8];
+  }
+  if (present & 8u) {
+    tiles = __reduce_add_sync(FULL_MASK, tiles);
+    bpts = __reduce_add_sync(FULL_MASK, bpts);
+    if (lane == 13) atomicAdd(a.next + R_TILES, tiles);
+    if (lane == 14) atomicAdd(a.next + R_BIGPTS, bpts);
+  }
+  if (amount) {  // the lists hold every entry by construction
+    uint32_t* c = nullptr;
+    uint32_t cap = 0;
+    switch (lane) {
+      case 0: cap = a.item_cap; break;
+      case 1: c = a.next + R_SMALL, cap = a.small_cap; break;
+      case 2: c = a.next + R_MID, cap = a.mid_cap; break;
+      case 3: c = a.next + R_BIG, cap = a.big_cap; break;
+      case 4: c = a.u + U_GOUT, cap = a.group_cap; break;
+      case 5: c = a.u + U_GIN, cap = a.group_cap; break;
+      case 6: c = a.cur + R_STAY, cap = a.stay_cap; break;
+      default: c = a.cur + R_AUX, cap = a.aux_cap; break;
+    }
+    if (lane == 0) {  // items (high word) and their arena positions (fewer than 2^31) in one
+      const unsigned long long r =
+          atomicAdd((unsigned long long*)(a.u + U_TOTAL), ((unsigned long long)amount << 32) | nsz);
+      first = (uint32_t)(r >> 32);
+      pos32 = (uint32_t)r;
+    } else {
+      first = atomicAdd(c, amount);
+    }
+    if (first + amount > cap || first + amount < first) {
+      set_error(a.st, DERR_CAPACITY, 800 + lane);
+      first = 0xFFFFFFFFu;
+    }
+    if (a.last && lane >= 1 && lane <= 3) {
+      set_error(a.st, DERR_STATE, 820 + lane);
+      first = 0xFFFFFFFFu;
+    }
+  }
+  uint32_t at[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) at[k] = __shfl_sync(FULL_MASK, first, k);
-    uint64_t pos = a.top + __shfl_sync(FULL_MASK, pos0, 8) + incl - nsz;
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-      const int v = v0 + 32 * u + lane;
+  for (int k = 0; k < 8; ++k) at[k] = __shfl_sync(FULL_MASK, first, k);
+  uint64_t pos = a.top + __shfl_sync(FULL_MASK, pos32, 0);
+  if (present || is_big)
+    for (int v0 = vw; v0 < a.HN; v0 += step) {
+      const int v = v0 + lane;
+      const Out o = what(v);
+      if (!__any_sync(FULL_MASK, o.len != 0)) continue;
+      const uint64_t b0 = o.len ? it.start + S.st[heap_pos(v, a.lam)] : 0;
+      const uint32_t slot = o.len ? S.sl[v] : 0, dep = depth0 + (uint32_t)heap_level(max(v, 1));
 #pragma unroll
       for (int k = 0; k < 7; ++k) {
-        if (tot[k] == 0 || at[k] == 0xFFFFFFFFu) continue;  // warp-uniform
-        const unsigned bits = __ballot_sync(FULL_MASK, kind[u] == k);
-        if (kind[u] == k) {
-          const uint32_t o = at[k] + __popc(bits & lt);
-          const uint64_t b0 = it.start + S.st[heap_pos(v, a.lam)];
-          const uint32_t dep = depth0 + (uint32_t)heap_level(v), slot = S.sl[v];
-          if (k == 0) {
-            a.items[o] = RebuildItem{slot, dep, size[u], ins ? S.sz[v] : size[u], b0, b0 + (ins ? len[u] : 0u), pos,
-                                     inner[u] ? 0u : 1u, 0u};
-            pos += size[u];
-          } else if (k <= 3) {
+        if (!((present >> k) & 1u) || at[k] == 0xFFFFFFFFu) continue;  // warp-uniform
+        const unsigned bits = __ballot_sync(FULL_MASK, o.kind == k);
+        const uint32_t i = at[k] + __popc(bits & lt);
+        at[k] += __popc(bits);
+        if (k == 0) {
+          if (!bits) continue;
+          const uint32_t mine = o.kind == 0 ? o.size : 0u;
+          const uint32_t incl = (uint32_t)warp_incl_scan((int)mine);
+          if (o.kind == 0)
+            a.items[i] = RebuildItem{slot, dep, o.size, ins ? S.sz[v] : o.size, (uint32_t)(pos + incl - mine),
+                                     (uint32_t)b0, ins ? o.len : 0u, o.inner ? 0u : 1u};
+          pos += __shfl_sync(FULL_MASK, incl, 31);
+        } else if (o.kind == k) {
+          if (k <= 3) {
             const bool und = (S.under[v >> 5] >> (v & 31)) & 1u;
-            (k == 1 ? a.small : k == 2 ? a.mid : a.big)[o] = Seg{b0, len[u], dep | (und ? ITEM_FLAG : 0u), slot, IN_B};
+            (k == 1 ? a.small : k == 2 ? a.mid : a.big)[i] = Seg{b0, o.len, dep | (und ? ITEM_FLAG : 0u), slot, IN_B};
+            S.sk[v].x |= CONT_FLAG;
           } else if (k <= 5) {
-            (k == 4 ? a.gout : a.gin)[o] = LeafGroup{slot, len[u], b0};
+            (k == 4 ? a.gout : a.gin)[i] = LeafGroup{slot, o.len, b0};
           } else {
-            a.stay[o] = make_uint2(slot, size[u]);
+            a.stay[i] = make_uint2(slot, o.size);
           }
         }
-        at[k] += __popc(bits);
       }
-      if (tot[7] && at[7] != 0xFFFFFFFFu) {
-        const unsigned bits = __ballot_sync(FULL_MASK, aux[u]);
-        if (aux[u]) {
-          a.auxs[at[7] + __popc(bits & lt)] = S.sl[v];
-          a.aux[S.sl[v]] = len[u];
+      if ((present >> 7 & 1u) && at[7] != 0xFFFFFFFFu) {
+        const unsigned bits = __ballot_sync(FULL_MASK, o.aux);
+        if (o.aux) {
+          a.auxs[at[7] + __popc(bits & lt)] = slot;
+          a.aux[slot] = o.len;
         }
         at[7] += __popc(bits);
       }
       // the sieve moved every point of a big item to the other buffer: the
       // ranges that end here are copied to F afterwards, TILE points at a time
-      if (is_big && v >= 1 && v < a.HN && len[u] && sk_state(S.sk[v].y) == SK_BUCKET && !(S.f[v] & CONT_FLAG)) {
-        const uint32_t nc = (len[u] + a.TILE - 1) / a.TILE;
-        const uint32_t o = atomicAdd(a.cur + R_COPY, nc);
-        const uint32_t b0 = (uint32_t)it.start + S.st[heap_pos(v, a.lam)];
-        if (o + nc > a.copy_cap) set_error(a.st, DERR_CAPACITY, 810);
+      if (is_big && o.len && sk_state(S.sk[v].y) == SK_BUCKET && !(S.sk[v].x & CONT_FLAG)) {
+        const uint32_t nc = (o.len + a.TILE - 1) / a.TILE;
+        const uint32_t i = atomicAdd(a.cur + R_COPY, nc);
+        if (i + nc > a.copy_cap) set_error(a.st, DERR_CAPACITY, 810);
         else
           for (uint32_t k = 0; k < nc; ++k)
-            a.copy[o + k] = make_uint2(b0 + k * a.TILE, min((uint32_t)a.TILE, len[u] - k * a.TILE));
+            a.copy[i + k] = make_uint2((uint32_t)b0 + k * a.TILE, min((uint32_t)a.TILE, o.len - k * a.TILE));
       }
     }
-  }
   team_sync<T>();
 }
 
 template <int D, int T>
-__global__ void __launch_bounds__(T == 32 ? 32 * WARP_TEAMS : T, T == 32 ? 5 : 2) k_route(RouteArgs a, const Seg* list,
+__global__ void __launch_bounds__(T == 32 ? 32 * WARP_TEAMS : T, T == 32 ? 8 : 4) k_route(RouteArgs a, const Seg* list,
                                                                          const uint32_t* n) {
   constexpr int PER = (int)(T == 32 ? SMALL_ITEM : MID_ITEM) / T;
   constexpr int TEAMS = T == 32 ? WARP_TEAMS : 1;
-  constexpr bool REGS = T == 32 && D <= 3;  // the points' coordinates stay in registers
   extern __shared__ __align__(16) unsigned char route_sm[];
   if (pkd_failed_block(a.st)) return;
   const int tid = team_rank<T>(), team = T == 32 ? warp_id() : 0;
   const Skel S = skel_at(route_sm + (size_t)team * skel_bytes(a.HN, a.NB), a.HN, a.NB);
   const uint32_t nn = *n;
+  uint2 seen = make_uint2(0, 0);  // (reading the counters would queue behind the atomics on their line)
   for (uint32_t i = blockIdx.x * TEAMS + team; i < nn; i += gridDim.x * TEAMS) {
     const Seg it = list[i];
     const int len = (int)it.len;
     skel_clear<T>(a, S);
-    int32_t x[PER][REGS ? D : 1];
-    uint32_t hr[PER];  // heap index, then also the rank within the external entry << 12
+    // Heap index of every point, then also its rank within the external entry
+    // << 12.  The coordinates are read again where they are needed (from L1 or
+    // L2): held in registers they made the warps' kernel spill at 3-D, with the
+    // same time.
+    uint32_t hr[PER];
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-      hr[q] = 0;
-      if (q * T + tid < len) {
-        hr[q] = 1;
-        if constexpr (REGS) {
-#pragma unroll
-          for (int j = 0; j < D; ++j) x[q][j] = a.src.c[(uint64_t)j * a.src.stride + it.start + q * T + tid];
-        }
-      }
-    }
+    for (int q = 0; q < PER; ++q) hr[q] = q * T + tid < len ? 1 : 0;
     team_sync<T>();
     if (tid == 0) {
       S.sl[1] = it.root;
@@ -451,16 +465,7 @@ __global__ void __launch_bounds__(T == 32 ? 32 * WARP_TEAMS : T, T == 32 ? 5 : 2
         if (!h) continue;
         const int2 e = S.sk[h];
         if (sk_state(e.y) != SK_INTERNAL) continue;
-        const int dm = sk_dim(e.y);
-        int32_t xv;
-        if constexpr (REGS) {
-          xv = x[q][0];
-#pragma unroll
-          for (int k = 1; k < D; ++k)
-            if (dm == k) xv = x[q][k];
-        } else {
-          xv = a.src.c[(uint64_t)dm * a.src.stride + it.start + q * T + tid];
-        }
+        const int32_t xv = a.src.c[(uint64_t)sk_dim(e.y) * a.src.stride + it.start + q * T + tid];
         const int c = 2 * h + (xv >= e.x);
         hr[q] = (uint32_t)c;
         S.sk[c].x = 1;
@@ -470,11 +475,8 @@ __global__ void __launch_bounds__(T == 32 ? 32 * WARP_TEAMS : T, T == 32 ? 5 : 2
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
       if (q * T >= len) break;
-      if (hr[q]) hr[q] |= atomicAdd(&S.f[hr[q]], 1u) << 12;
+      if (hr[q]) hr[q] |= atomicAdd(&S.st[heap_pos((int)hr[q], a.lam)], 1u) << 12;
     }
-    team_sync<T>();
-    for (int v = 1 + tid; v < a.HN; v += T)
-      if (sk_state(S.sk[v].y) == SK_BUCKET && S.f[v]) S.st[heap_pos(v, a.lam)] = S.f[v];
     team_sync<T>();
     if (tid < 32) {  // starts: exclusive scan of the positions' counts
       unsigned carry = 0;
@@ -488,7 +490,7 @@ __global__ void __launch_bounds__(T == 32 ? 32 * WARP_TEAMS : T, T == 32 ? 5 : 2
       }
     }
     team_sync<T>();
-    route_tail<T>(a, S, it, false);
+    route_tail<T>(a, S, it, seen, false);
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
       if (q * T >= len) break;
@@ -496,14 +498,9 @@ __global__ void __launch_bounds__(T == 32 ? 32 * WARP_TEAMS : T, T == 32 ? 5 : 2
       const int v = (int)(hr[q] & 0xFFFu);
       const uint64_t g = it.start + q * T + tid;
       const uint64_t o = it.start + S.st[heap_pos(v, a.lam)] + (hr[q] >> 12);
-      const Pts& P = (S.f[v] & CONT_FLAG) ? a.dst : a.F;
+      const Pts& P = (S.sk[v].x & CONT_FLAG) ? a.dst : a.F;
 #pragma unroll
-      for (int j = 0; j < D; ++j) {
-        int32_t xv;
-        if constexpr (REGS) xv = x[q][j];
-        else xv = a.src.c[(uint64_t)j * a.src.stride + g];
-        P.c[(uint64_t)j * P.stride + o] = xv;
-      }
+      for (int j = 0; j < D; ++j) P.c[(uint64_t)j * P.stride + o] = a.src.c[(uint64_t)j * a.src.stride + g];
       P.id[o] = a.src.id[g];
     }
     team_sync<T>();
@@ -554,13 +551,8 @@ static __global__ void __launch_bounds__(BIG_TEAM) k_big_emit(RouteArgs a, Round
   const uint32_t base = r.hscan[hb];
   for (int b = threadIdx.x; b < a.NB; b += BIG_TEAM) S.st[b] = r.hscan[hb + (uint64_t)b * nt] - base;
   __syncthreads();
-  for (int v = 1 + threadIdx.x; v < a.HN; v += BIG_TEAM)
-    if (sk_state(S.sk[v].y) == SK_BUCKET) {
-      const int b = heap_pos(v, a.lam);
-      S.f[v] = (b + 1 < a.NB ? S.st[b + 1] : it.len) - S.st[b];
-    }
-  __syncthreads();
-  route_tail<BIG_TEAM>(a, S, it, true);
+  uint2 seen = make_uint2(0, 0);
+  route_tail<BIG_TEAM>(a, S, it, seen, true);
 }
 
 // The ranges of the big items that ended, from the sieve's destination to F.

@@ -211,7 +211,7 @@ __global__ void k_item_leaves(const RebuildItem* it, const uint32_t* n, Node* no
   if (i >= *n) return;
   const RebuildItem x = it[i];
   if (x.size > phi) return;
-  nodes[x.slot] = Node{0, x.size, (uint32_t)x.pos, 0};
+  nodes[x.slot] = Node{0, x.size, x.pos, 0};
   ndim[x.slot] = PKD_LEAF;
 }
 
@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(UPW_WARPS * 32) k_copy_leaves(const Front* lv,
     const Node nd = nodes[e.slot];
     a = nd.a;
     sz = nd.size;
-    d0 = items[e.item].pos + e.off;
+    d0 = (uint64_t)items[e.item].pos + e.off;
   }
   uint32_t qa[UPW], qsz[UPW];
   unsigned long long qd[UPW];
@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(UPW_WARPS * 32, (D <= 3 ? 6 : 1)) k_copy_items
   if (lane < UPW && k0 + lane < nn) {
     const RebuildItem it = items[k0 + lane];
     ws = it.ws;
-    cnt = it.we - it.ws;
+    cnt = it.nw;
     pos = it.pos;
     live = it.old_live;
     if (it.leaf) {
@@ -458,8 +458,8 @@ __global__ void __launch_bounds__(UPW_WARPS * 32, (D <= 3 ? 6 : 1)) k_copy_items
 __global__ void k_item_newcounts(const RebuildItem* it, const uint32_t* n, uint32_t* cnt) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < *n) {
-    const uint64_t c = it[i].we - it[i].ws;
-    cnt[i] = c > NEW_BIG ? (uint32_t)c : 0u;  // the items k_copy_items leaves out
+    const uint32_t c = it[i].nw;
+    cnt[i] = c > NEW_BIG ? c : 0u;  // the items k_copy_items leaves out
   }
 }
 
@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(256) k_copy_new_flat(const RebuildItem* items,
     }
     const RebuildItem it = items[lo];
     const uint64_t k = j - off[lo];
-    const uint64_t src = it.ws + k, dst = it.pos + it.old_live + k;
+    const uint64_t src = it.ws + k, dst = (uint64_t)it.pos + it.old_live + k;
 #pragma unroll
     for (int q = 0; q < D; ++q) A.c[(uint64_t)q * A.stride + dst] = F.c[(uint64_t)q * F.stride + src];
     A.id[dst] = F.id[src];
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(256) k_copy_big_leaves(const Front* lv, const 
   for (uint32_t k = blockIdx.x; k < nn; k += gridDim.x) {
     const Front e = lv[k];
     const Node nd = nodes[e.slot];
-    const uint64_t d0 = items[e.item].pos + e.off;
+    const uint64_t d0 = (uint64_t)items[e.item].pos + e.off;
     uint64_t out = 0;
     for (uint32_t base = 0; base < nd.size; base += 256) {
       const uint32_t i = base + threadIdx.x;
@@ -575,7 +575,8 @@ static void launch_route(const RouteArgs& a, const Seg* mid, const uint32_t* d_n
   }
   if (nmid) PKD_LAUNCH((k_route<D, MID_TEAM><<<nmid, MID_TEAM, per, s>>>(a, mid, d_nmid)));
   if (nsmall) {
-    const unsigned g = (nsmall + WARP_TEAMS - 1) / WARP_TEAMS;
+    // persistent warps: each remembers the largest sizes that it has sent
+    const unsigned g = std::min<unsigned>((nsmall + WARP_TEAMS - 1) / WARP_TEAMS, (unsigned)sm_count() * 8);
     PKD_LAUNCH((k_route<D, 32><<<g, 32 * WARP_TEAMS, warps, s>>>(a, small, d_nsmall)));
   }
 }
@@ -732,14 +733,14 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
   const bool queued = m <= MID_ITEM;
   const uint32_t height = t.st_host->max_depth;  // an upper bound
   const int max_rounds = (int)std::max<uint64_t>(1, ((uint64_t)height + lam - 1) / lam);
-  const uint32_t ctl_words = U_WORDS + (uint32_t)(max_rounds + 2) * R_WORDS;
+  const uint32_t ctl_words = (uint32_t)(max_rounds + 3) * CTL_STRIDE;
   uint32_t* ctl;
   PKD_TRY(sc.get(&ctl, ctl_words));
   PinnedBlock hblk;
   uint32_t* hu = (uint32_t*)hblk.p;
   if (!hu) return PKD_ENOMEM;
-  static_assert((U_WORDS + 2 * R_WORDS) * 4 <= PINNED_BLOCK, "counters");
-  auto rc = [&](int r) { return ctl + U_WORDS + (uint32_t)r * R_WORDS; };
+  static_assert((U_WORDS + R_WORDS) * 4 <= PINNED_BLOCK, "counters");
+  auto rc = [&](int r) { return ctl + (uint32_t)(r + 1) * CTL_STRIDE; };
 
   // every routed point ends in one leaf group or rebuild item
   const uint32_t group_cap = (uint32_t)m;
@@ -774,7 +775,7 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
   uint64_t big_pts = nbig ? m : 0;  // points the round's sieve kernels move
   Seg *big = first, *mid = first, *small = first;
   PKD_LAUNCH(k_update_init<<<1, 256, 0, s>>>(ctl, ctl_words, root, first,
-                                             U_WORDS + (nbig ? R_BIG : (nmid ? R_MID : R_SMALL))));
+                                             (int)CTL_STRIDE + (nbig ? R_BIG : (nmid ? R_MID : R_SMALL))));
   RouteRound all{};  // queued rounds share their lists
   if (queued) {
     // a point's path has at most `height` inner nodes
@@ -890,7 +891,7 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
       sa.hist = hist;
       sa.hscan = hscan;
       const size_t per = skel_bytes(HN, NB);
-      if (per > 48 * 1024) return PKD_EINTERNAL;  // (45 KB at lambda = 10)
+      if (per > 48 * 1024) return PKD_EINTERNAL;  // (37 KB at lambda = 10)
       PKD_LAUNCH(k_big_fetch<<<nbig, BIG_TEAM, per, s>>>(ra, big, sa.skel, slots, sizes));
       PKD_LAUNCH(k_big_prefix<<<1, 1024, 0, s>>>(big, sa.nbig, (uint32_t)TILE, sa.tile0, sa.excl));
       PKD_DISPATCH_D(d, launch_count, sa, tiles, big_pts, "count_route", s);
@@ -904,10 +905,10 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
       nmid = ra.mid_cap;
       nsmall = ra.small_cap;
     } else {
-      PKD_CUDA(cudaMemcpyAsync(hu + U_WORDS, rc(r), 2 * R_WORDS * 4, cudaMemcpyDeviceToHost, s));
+      PKD_CUDA(cudaMemcpyAsync(hu + U_WORDS, rc(r + 1), R_WORDS * 4, cudaMemcpyDeviceToHost, s));
       PKD_TRY(read_flags());
       if (idflags && *idflags) return PKD_OK;
-      const uint32_t* nx = hu + U_WORDS + R_WORDS;
+      const uint32_t* nx = hu + U_WORDS;
       nbig = nx[R_BIG];
       nmid = nx[R_MID];
       nsmall = nx[R_SMALL];
@@ -923,7 +924,7 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
   PKD_TRY(read_flags());
   if (idflags && *idflags) return PKD_OK;
   const uint32_t nitems = hu[U_ITEMS], ninner = hu[U_INNER], ngout = hu[U_GOUT], ngin = hu[U_GIN];
-  const uint64_t total = *(unsigned long long*)(hu + U_TOTAL);
+  const uint64_t total = hu[U_TOTAL];
   const uint64_t inner_total = *(unsigned long long*)(hu + U_INNER_PTS);
   marks.aux = ninner != 0;
   const uint32_t* d_nitems = ctl + U_ITEMS;
