@@ -222,9 +222,11 @@ __device__ void presort_dim(const SCtx<D>& cx, int k, int vmin, int vmax, int n,
 
 // Faster presort for the common case: one most-significant-digit counting
 // pass over MSD_BINS bins of the top varying bits (plain shared-memory
-// atomics, no ranking), then every bin, now a contiguous run of the list, is
-// sorted by (coordinate, point index) by one thread.  The order is the same
-// as the stable LSD sort's.  Returns false, before writing the list, when a
+// atomics, no ranking) into the spare list, then every point counts the points
+// of its bin that come before it by (coordinate, point index): its place in
+// the sorted list.  (Sorting each bin by one thread, eight bins a thread, cost
+// about three times the instructions: most bins hold a point or none, and a
+// warp waits for its fullest.)  The order is the same as the stable LSD sort's.  Returns false, before writing the list, when a
 // bin holds more than MSD_MAX_BUCKET points (clustered coordinates); the
 // caller then sorts that dimension with presort_dim.
 constexpr int MSD_BITS = 12;
@@ -274,25 +276,25 @@ __device__ bool presort_dim_msd(const SCtx<D>& cx, int k, int vmin, int vmax, in
     run += c[q];
   }
   __syncthreads();
+  uint16_t* binned = cx.list(D);
   for (int i = tid; i < n; i += SS_THREADS)
-    target[atomicAdd(&hist[((unsigned)Xk[i] - (unsigned)vmin) >> shift], 1u)] = (uint16_t)i;
+    binned[atomicAdd(&hist[((unsigned)Xk[i] - (unsigned)vmin) >> shift], 1u)] = (uint16_t)i;
   __syncthreads();
-  // hist[b] is now the end of bin b; sort each bin by (coordinate, index)
-  for (int b = tid; b < MSD_BINS; b += SS_THREADS) {
+  // hist[b] is now the end of bin b
+  for (int i = tid; i < n; i += SS_THREADS) {
+    const int v = binned[i];
+    const int32_t kv = Xk[v];
+    const unsigned b = ((unsigned)kv - (unsigned)vmin) >> shift;
     const int e = (int)hist[b], st = b ? (int)hist[b - 1] : 0;
-    for (int i = st + 1; i < e; ++i) {
-      const int v = target[i];
-      const int32_t kv = Xk[v];
-      int j = i - 1;
-      while (j >= st) {
-        const int u = target[j];
+    int r = st;
+    if (e - st > 1) {
+      for (int j = st; j < e; ++j) {
+        const int u = binned[j];
         const int32_t ku = Xk[u];
-        if (ku < kv || (ku == kv && u < v)) break;
-        target[j + 1] = (uint16_t)u;
-        --j;
+        r += ku < kv || (ku == kv && u < v);
       }
-      target[j + 1] = (uint16_t)v;
     }
+    target[r] = (uint16_t)v;
   }
   __syncthreads();
   return true;
@@ -597,6 +599,62 @@ __device__ uint32_t spartition(const Team& tm, const SCtx<D>& cx, uint32_t map, 
   }
   const int per = ((n + nw * 32 - 1) / (nw * 32)) * 32;
   const int wlo = min(hi, lo + w * per), whi = min(hi, wlo + per);
+  if constexpr (D == 2 || D == 3) {
+    // Runs of at most 32 * G entries a warp: every list is read once, kept in
+    // registers over the one barrier that the counts need, and written (a list
+    // takes the buffer that the one before it has left).  The form below reads
+    // each list twice and needs a barrier per list.
+    constexpr int G = 8, M = D - 1;
+    if (per <= 32 * G) {
+      uint32_t pk[M][G / 2];  // two entries a word
+      unsigned fl[M];         // bit u: entry u goes left
+#pragma unroll
+      for (int q = 0; q < M; ++q) {
+        const uint16_t* src = cx.list(mget(map, q + (q >= dim)));
+        int cl = 0;
+        fl[q] = 0;
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+          if ((u & 1) == 0) pk[q][u / 2] = 0;
+          if (wlo + u * 32 < whi) {  // warp-uniform
+            const int i = wlo + u * 32 + lane;
+            const unsigned p = i < whi ? src[i] : 0u;
+            const bool left = i < whi && Xd[p] < x;
+            pk[q][u / 2] |= p << (16 * (u & 1));
+            fl[q] |= (unsigned)left << u;
+            cl += __popc(__ballot_sync(FULL_MASK, left));
+          }
+        }
+        if (lane == 0) tm.red[w * SS_RED + q] = cl;
+      }
+      tm.sync();
+#pragma unroll
+      for (int q = 0; q < M; ++q) {
+        const int before = warp_sum(lane < w ? tm.red[lane * SS_RED + q] : 0);
+        int lb = lo + before, rb = lo + L + (wlo - lo - before);
+        uint16_t* dst = cx.list(spare);
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+          const int rem = whi - (wlo + u * 32);
+          if (rem > 0) {
+            const unsigned vm = rem >= 32 ? FULL_MASK : ((1u << rem) - 1u);
+            const bool left = (fl[q] >> u) & 1u;
+            const unsigned bl = __ballot_sync(FULL_MASK, left), br = vm & ~bl;
+            const uint16_t p = (uint16_t)(pk[q][u / 2] >> (16 * (u & 1)));
+            if (left) dst[lb + __popc(bl & lanemask_lt())] = p;
+            else if (lane < rem) dst[rb + __popc(br & lanemask_lt())] = p;
+            lb += __popc(bl);
+            rb += __popc(br);
+          }
+        }
+        const int k = q + (q >= dim), freed = mget(map, k);
+        map = mset(map, k, spare);
+        spare = freed;
+      }
+      tm.sync();
+      return map;
+    }
+  }
 #pragma unroll
   for (int k = 0; k < D; ++k) {
     if (k == dim) continue;
