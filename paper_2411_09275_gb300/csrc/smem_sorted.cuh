@@ -678,9 +678,23 @@ __device__ uint32_t spartition(const Team& tm, const SCtx<D>& cx, uint32_t map, 
   return map;
 }
 
-// Process one node; returns the number of children written to ch (0 or 2).
+// The children of a split node: positions [lo, lo + L) and [lo + L, hi), slots
+// sl and sl + 1.  (Two task records instead were an array in local memory.)
+struct SKids {
+  int L;
+  uint32_t sl, map;
+  int SL, SR;  // sampled points of each
+  uint8_t j;
+};
+__device__ __forceinline__ STask skid(const STask& tk, const SKids& c, bool right) {
+  const uint16_t mid = (uint16_t)(tk.lo + c.L);
+  return STask{right ? mid : tk.lo, right ? tk.hi : mid, (uint16_t)(right ? c.SR : c.SL), c.j, 0, tk.t + 1,
+               c.sl + (right ? 1u : 0u), c.map, 0};
+}
+
+// Process one node; whether it has children to process (in ch).
 template <int D>
-__device__ int snode(const Team& tm, const SCtx<D>& cx, STask tk, STask* ch) {
+__device__ bool snode(const Team& tm, const SCtx<D>& cx, STask tk, SKids& ch) {
   for (;;) {
     const int lo = tk.lo, hi = tk.hi, n = hi - lo;
     int dim = 0, x = 0, L = 0, SL = 0;
@@ -689,7 +703,7 @@ __device__ int snode(const Team& tm, const SCtx<D>& cx, STask tk, STask* ch) {
       // Build(P, t): leaf wrap, heavy leaf, then sample and skeleton root.
       if (n <= cx.p.phi) {
         semit_leaf<D>(tm, cx, tk);
-        return 0;
+        return false;
       }
       int wd = -1;
       long long ext = 0;
@@ -704,7 +718,7 @@ __device__ int snode(const Team& tm, const SCtx<D>& cx, STask tk, STask* ch) {
       }
       if (wd < 0) {
         semit_leaf<D>(tm, cx, tk);
-        return 0;
+        return false;
       }
       // fewer than 2*sigma_os points cannot reach the split threshold
       int ns = 0;
@@ -743,7 +757,7 @@ __device__ int snode(const Team& tm, const SCtx<D>& cx, STask tk, STask* ch) {
     }
     if (L <= 0 || L >= n) {
       if (tm.leader()) set_error(cx.st, DERR_STATE, 300 + L);
-      return 0;
+      return false;
     }
     // both children wrap into leaves (at most phi points each, and neither
     // is a skeleton node that its sample would split further): their points
@@ -758,7 +772,7 @@ __device__ int snode(const Team& tm, const SCtx<D>& cx, STask tk, STask* ch) {
     b = tm.bcast(b);
     if (b + 2 > cx.slot_limit) {
       if (tm.leader()) set_error(cx.st, DERR_SLOT, b);
-      return 0;
+      return false;
     }
     const uint32_t sl = cx.slot_base + (uint32_t)b, sr = sl + 1;
     if (tm.leader()) {
@@ -779,13 +793,12 @@ __device__ int snode(const Team& tm, const SCtx<D>& cx, STask tk, STask* ch) {
         cx.ndim[sr] = PKD_LEAF;
         atomicMax(&cx.ctl->maxd, tk.t + 1);
       }
-      return 0;
+      return false;
     }
     const uint8_t nj = on_sample ? (uint8_t)(tk.j + 1) : (uint8_t)0;
     const int SR = on_sample ? tk.ns - SL : 0;
-    ch[0] = STask{(uint16_t)lo, (uint16_t)(lo + L), (uint16_t)(on_sample ? SL : 0), nj, 0, tk.t + 1, sl, cmap, 0};
-    ch[1] = STask{(uint16_t)(lo + L), (uint16_t)hi, (uint16_t)SR, nj, 0, tk.t + 1, sr, cmap, 0};
-    return 2;
+    ch = SKids{L, sl, cmap, on_sample ? SL : 0, SR, nj};
+    return true;
   }
 }
 
@@ -794,24 +807,22 @@ template <int D>
 __device__ void swarp_run(const Team& wt, const SCtx<D>& cx, STask tk, STask* stk, int sp0) {
   int sp = sp0;
   for (int iter = 1;; ++iter) {
-    STask ch[2];
-    const int nch = snode<D>(wt, cx, tk, ch);
+    SKids ch;
+    const bool kids = snode<D>(wt, cx, tk, ch);
     if ((iter & 63) == 0) {  // another CTA's failure ends this one early
       const int err = *(volatile int*)&cx.st->err;
       if (__shfl_sync(FULL_MASK, err, 0)) return;  // warp-uniform exit
     }
-    if (nch == 2) {
-      const int s0 = ch[0].hi - ch[0].lo, s1 = ch[1].hi - ch[1].lo;
-      const STask big = s0 >= s1 ? ch[0] : ch[1];
-      const STask small = s0 >= s1 ? ch[1] : ch[0];
+    if (kids) {
+      const bool left_big = 2 * ch.L >= tk.hi - tk.lo;
       if (sp >= SS_STK) {
         if (lane_id() == 0) set_error(cx.st, DERR_STACK, sp);
         return;
       }
-      if (lane_id() == 0) stk[sp] = big;
+      if (lane_id() == 0) stk[sp] = skid(tk, ch, !left_big);
       __syncwarp();
       ++sp;
-      tk = small;
+      tk = skid(tk, ch, left_big);
     } else {
       if (sp == 0) return;
       --sp;
@@ -831,30 +842,29 @@ __device__ void srun_tasks(const SCtx<D>& cx, STask root, int* sred, STask* wsta
   bool have_task = true;
   while (nw > 1) {
     const Team tm{f, nw, team_barrier(f, nw, SS_NW), nullptr, sred + f * SS_RED};
-    STask ch[2];
-    const int nch = snode<D>(tm, cx, tk, ch);
-    if (nch == 0) {
+    SKids ch;
+    if (!snode<D>(tm, cx, tk, ch)) {
       have_task = false;
       break;
     }
-    const int s0 = ch[0].hi - ch[0].lo, s1 = ch[1].hi - ch[1].lo;
-    const int big = s0 >= s1 ? 0 : 1;
+    const int s0 = ch.L, s1 = tk.hi - tk.lo - ch.L;
+    const bool right_big = s1 > s0;
     const int small_n = min(s0, s1);
     tm.sync();
     const bool defer = small_n <= DEFER_MAX && small_n * 8 <= max(s0, s1) && cx.ctl->wsp[f] < SS_STK;
     tm.sync();
     if (defer) {
       if (tm.leader()) {
-        wstack[f * SS_STK + cx.ctl->wsp[f]] = ch[big ^ 1];
+        wstack[f * SS_STK + cx.ctl->wsp[f]] = skid(tk, ch, !right_big);
         cx.ctl->wsp[f] += 1;
       }
       tm.sync();
-      tk = ch[big];
+      tk = skid(tk, ch, right_big);
       continue;
     }
     const int half = nw / 2;
     const bool second = w >= f + half;
-    tk = second ? ch[1] : ch[0];
+    tk = skid(tk, ch, second);
     if (second) f += half;
     nw = half;
   }
