@@ -5,9 +5,9 @@
 //           becomes LIVE; an id found LIVE (stored, or taken by another point
 //           of the same batch) raises IDF_BAD_ID.  A rejected batch gives its
 //           claimed slots back as DEAD (unclaim), so the stored set is
-//           unchanged.  A build with ids 0..n-1 stores its keys without
-//           compare-and-swap: the table is empty and those ids have distinct
-//           home slots.
+//           unchanged.
+//  dense    build with ids 0..n-1: those ids have distinct home slots, so every
+//           slot of the new table is written once, with its id or as empty.
 //  take     delete: every id found LIVE becomes DEAD (one winner per id, so
 //           repeats count once), and its coordinates and id are appended to
 //           the batch buffer that the delete sieves; unknown and DEAD ids are
@@ -33,8 +33,7 @@ unsigned id_blocks(uint64_t n) {
 
 // CLAIM_PER ids per thread: their first probe loads, then their
 // compare-and-swaps, are all issued before any is waited for (random
-// accesses into a table far larger than L2).  The dense build path (ids
-// 0..m-1 into an empty table) stores its keys directly.
+// accesses into a table far larger than L2).
 constexpr int CLAIM_PER = 4;
 
 __device__ __forceinline__ void claim_store(const int32_t* coords, uint64_t i, int d, const IdTable& T, uint64_t got,
@@ -50,14 +49,6 @@ __device__ __forceinline__ void claim_store(const int32_t* coords, uint64_t i, i
 __global__ void __launch_bounds__(ID_THREADS) k_ids_claim(const int32_t* coords, const uint32_t* ids, uint64_t m,
                                                           int d, IdTable T, uint64_t* slots, DevStatus* st) {
   const uint64_t mask = T.cap - 1;
-  if (!ids) {  // ids 0..m-1 into an empty table: distinct home slots
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
-      const uint64_t got = id_home((uint32_t)i, T.lgc);
-      T.key[got] = id_key((uint32_t)i, coords[i * (uint64_t)d], ID_LIVE);
-      claim_store(coords, i, d, T, got, slots);
-    }
-    return;
-  }
   const uint64_t span = (uint64_t)ID_THREADS * CLAIM_PER;
   for (uint64_t b0 = (uint64_t)blockIdx.x * span; b0 < m; b0 += (uint64_t)gridDim.x * span) {
     uint32_t id[CLAIM_PER];
@@ -112,6 +103,59 @@ __global__ void __launch_bounds__(ID_THREADS) k_ids_claim(const int32_t* coords,
     }
     if (bad) atomicOr(&st->idflags, bad);
   }
+}
+
+// A new table of ids 0..m-1 (m <= cap), every slot written once: the home
+// slots of chunks of 32 ids are a permutation, so each chunk of slots knows
+// its ids (minv: the inverse of the home slot's multiplier modulo 2^lgc).  A
+// warp takes DENSE_PER chunks at a time, every load before the first store,
+// all of them coalesced.  Bound by HBM: 2^28 slots for 1e8 3-D points are 4.1 GB;
+// filling the keys first and storing the ids in a second pass moved 4.9 GB, in
+// 0.33 + 0.70 ms, most of the second after the base cases that it should
+// overlap.  DENSE_CTAS per SM leave room for the largest base case's CTA, which
+// starts at the same time: the step of 1e8 points takes 22.1 ms with them, 22.4
+// with four per SM, 22.3 with one, 22.7 with the two passes.
+constexpr int DENSE_PER = 2, DENSE_CTAS = 2;
+template <int D>
+__global__ void __launch_bounds__(ID_THREADS, D <= 4 ? 6 : 2) k_ids_dense(const int32_t* coords, uint64_t m, IdTable T, uint32_t minv) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t chunks = T.cap >> 5, cmask = chunks - 1;
+  const uint64_t nw = (uint64_t)gridDim.x * (ID_THREADS / 32);
+  for (uint64_t c0 = (uint64_t)blockIdx.x * (ID_THREADS / 32) + (threadIdx.x >> 5); c0 < chunks; c0 += nw * DENSE_PER) {
+    int32_t x[DENSE_PER][D];
+    uint64_t id[DENSE_PER];
+#pragma unroll
+    for (int u = 0; u < DENSE_PER; ++u) {
+      const uint64_t c = c0 + nw * u;
+      id[u] = ((uint64_t)((uint32_t)c * minv) & cmask) << 5 | lane;
+#pragma unroll
+      for (int j = 0; j < D; ++j) x[u][j] = c < chunks && id[u] < m ? coords[id[u] * D + j] : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < DENSE_PER; ++u) {
+      const uint64_t c = c0 + nw * u;
+      if (c >= chunks) break;
+      const uint64_t s = (c << 5) | lane;
+      T.key[s] = id[u] < m ? id_key((uint32_t)id[u], x[u][0], ID_LIVE) : ID_EMPTY;
+      if (id[u] < m) {
+        if constexpr (D == 3) {
+          *(int2*)(T.xs + 2 * s) = make_int2(x[u][1], x[u][2]);
+        } else {
+#pragma unroll
+          for (int j = 1; j < D; ++j) T.xs[s * (uint64_t)T.cw + (j - 1)] = x[u][j];
+        }
+      }
+    }
+  }
+}
+template <int D>
+static void launch_dense(const int32_t* coords, uint64_t m, const IdTable& T, uint32_t minv, cudaStream_t s) {
+  const uint64_t warps = ((T.cap >> 5) + DENSE_PER - 1) / DENSE_PER;
+  const unsigned g = (unsigned)std::min<uint64_t>((warps + ID_THREADS / 32 - 1) / (ID_THREADS / 32), 152 * DENSE_CTAS);
+  // an SM set up for this kernel's own shared memory (none) would have to drain
+  // before the base case could start on it
+  cudaFuncSetAttribute(k_ids_dense<D>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  PKD_LAUNCH(k_ids_dense<D><<<std::max(g, 1u), ID_THREADS, 0, s>>>(coords, m, T, minv));
 }
 
 __global__ void __launch_bounds__(ID_THREADS) k_ids_restate(const uint64_t* slots, uint64_t m, IdTable T,
@@ -233,7 +277,7 @@ uint64_t ids_cap_for(uint64_t n) {
   return c;
 }
 
-int ids_alloc(IdTable& T, int d, uint64_t cap, cudaStream_t s) {
+int ids_alloc(IdTable& T, int d, uint64_t cap, bool fill, cudaStream_t s) {
   T = IdTable{};
   if (cap > (1ull << 32)) return PKD_ENOMEM;
   T.cap = cap;
@@ -251,7 +295,7 @@ int ids_alloc(IdTable& T, int d, uint64_t cap, cudaStream_t s) {
     ids_release(T, s);
     return e == cudaErrorMemoryAllocation ? PKD_ENOMEM : PKD_ECUDA;
   }
-  PKD_TRY(dev_fill(T.key, 0xFF, (size_t)cap * 8, s));
+  if (fill) PKD_TRY(dev_fill(T.key, 0xFF, (size_t)cap * 8, s));
   return PKD_OK;
 }
 
@@ -263,13 +307,22 @@ void ids_release(IdTable& T, cudaStream_t s) {
   T = IdTable{};
 }
 
-int ids_create(TreeMem& t, uint64_t n, cudaStream_t s) { return ids_alloc(t.ids, t.p.d, ids_cap_for(n), s); }
+int ids_create(TreeMem& t, uint64_t n, cudaStream_t s) { return ids_alloc(t.ids, t.p.d, ids_cap_for(n), true, s); }
+
+int ids_create_dense(TreeMem& t, const int32_t* coords, uint64_t n, cudaStream_t s) {
+  PKD_TRY(ids_alloc(t.ids, t.p.d, ids_cap_for(n), n == 0, s));
+  if (n == 0) return PKD_OK;
+  uint32_t minv = 1;  // of the odd multiplier, by Newton's iteration modulo 2^32
+  for (int k = 0; k < 5; ++k) minv *= 2u - ID_MULT * minv;
+  PKD_DISPATCH_D(t.p.d, launch_dense, coords, n, t.ids, minv, s);
+  return PKD_OK;
+}
 
 int ids_reserve(TreeMem& t, uint64_t extra, cudaStream_t s) {
   IdTable& T = t.ids;
   if (T.used + extra <= T.cap / 4 * 3) return PKD_OK;
   IdTable B;
-  PKD_TRY(ids_alloc(B, t.p.d, ids_cap_for(T.live + extra), s));
+  PKD_TRY(ids_alloc(B, t.p.d, ids_cap_for(T.live + extra), true, s));
   PKD_LAUNCH(k_ids_rehash<<<id_blocks(T.cap), ID_THREADS, 0, s>>>(T, B, t.p.d, t.st));
   int fl = 0;
   int e = read_idflags(t, s, &fl);
@@ -296,7 +349,7 @@ int read_idflags(TreeMem& t, cudaStream_t s, int* flags) {
 void ids_claim(TreeMem& t, const int32_t* coords, const uint32_t* ids, uint64_t m, uint64_t* slots,
                cudaStream_t s) {
   if (m == 0) return;
-  const uint64_t per = ids ? CLAIM_PER : 1;
+  const uint64_t per = CLAIM_PER;
   // timed for inserts only: a build's fill runs beside its base cases on a
   // second stream, so its span is not the kernel's own time
   KTimer kt;

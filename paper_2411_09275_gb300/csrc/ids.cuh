@@ -31,6 +31,7 @@ constexpr unsigned long long ID_EMPTY = ~0ull;
 constexpr uint32_t ID_LIVE = 0, ID_DEAD = 1;
 constexpr uint32_t ID_RESERVED = 0xFFFFFFFFu;  // k-NN padding; never a point's id
 constexpr uint64_t ID_NO_SLOT = ~0ull;
+constexpr uint32_t ID_MULT = 0x9E3779B1u;  // odd
 
 // Flag bits the table kernels raise (DevStatus::idflags).
 constexpr int IDF_BAD_ID = 1;  // a repeated, stored or reserved id in a claim
@@ -49,7 +50,7 @@ struct IdTable {
 __host__ __device__ __forceinline__ uint64_t id_home(uint32_t id, int lgc) {
   const uint32_t c = id >> 5;
   const uint32_t f = lgc > 0 ? (c ^ (c >> lgc)) : 0u;
-  const uint64_t chunk = (uint64_t)(f * 0x9E3779B1u) & ((1ull << lgc) - 1ull);
+  const uint64_t chunk = (uint64_t)(f * ID_MULT) & ((1ull << lgc) - 1ull);
   return (chunk << 5) | (id & 31u);
 }
 

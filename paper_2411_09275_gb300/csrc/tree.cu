@@ -631,8 +631,12 @@ int pkd_build(const int32_t* coords, const uint32_t* ids, uint64_t n, const pkd_
       start = ev[0];
     }
     cudaStreamWaitEvent(s2, start, 0);
-    eid = ids_create(tt->m, n, s2);
-    if (eid == PKD_OK) ids_claim(tt->m, coords, ids, n, nullptr, s2);
+    if (!ids) {
+      eid = ids_create_dense(tt->m, coords, n, s2);
+    } else {
+      eid = ids_create(tt->m, n, s2);
+      if (eid == PKD_OK) ids_claim(tt->m, coords, ids, n, nullptr, s2);
+    }
     cudaEventRecord(ev[1], s2);
   };
   BuildJob job;

@@ -41,11 +41,11 @@ int export_from(const HostTree& h, uint32_t root, uint64_t top, uint64_t size, u
 
 // Id table (ids.cu; layout in ids.cuh).
 //  ids_create   an empty table for n ids with room to grow
+//  ids_create_dense  a table that holds ids 0..n-1 with these coordinates
 //  ids_reserve  room for `extra` more claims (rehashes into a larger table)
 //  ids_claim    launch: points take their ids' slots (LIVE); slots[i] gets
 //               the claimed slot or ID_NO_SLOT (slots may be NULL); a bad id
-//               raises IDF_BAD_ID in the status word; ids NULL (0..m-1) only
-//               into a new, empty table
+//               raises IDF_BAD_ID in the status word
 //  ids_unclaim  launch: claimed slots go back to DEAD (a rejected batch)
 //  ids_take     launch: LIVE ids become DEAD and their (coords, id) are
 //               appended to W (count is the device append counter), the slot
@@ -53,6 +53,7 @@ int export_from(const HostTree& h, uint32_t root, uint64_t top, uint64_t size, u
 //  ids_restore  launch: taken slots become LIVE again (a failed delete)
 //  read_idflags synchronises `s`, returns and clears the flags
 int ids_create(TreeMem& t, uint64_t n, cudaStream_t s);
+int ids_create_dense(TreeMem& t, const int32_t* coords, uint64_t n, cudaStream_t s);
 int ids_reserve(TreeMem& t, uint64_t extra, cudaStream_t s);
 void ids_release(IdTable& T, cudaStream_t s);
 void ids_claim(TreeMem& t, const int32_t* coords, const uint32_t* ids, uint64_t m, uint64_t* slots, cudaStream_t s);

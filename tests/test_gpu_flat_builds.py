@@ -45,6 +45,28 @@ for d, kind in ((1, "uniform"), (2, "varden"), (3, "uniform"), (3, "dups"), (5, 
         U.assert_exports_equal(t.export(), o.export())
         assert graphs() == g0, (d, n)
         t.close()
+# ids 0..n-1 (their table is written slot by slot): every id is found again, at
+# the sizes where the table has one chunk, a few, and just fits
+for d in (1, 2, 3, 4, 6, 8):
+    for n in (1, 31, 32, 33, 614, 615, 5000):
+        X = I.uniform(n, d, n + d)
+        p = pkd.Params(d=d)
+        t, o = pkd.Tree(to_dev(X), None, p), O.OracleTree(X, None, oparams(p))
+        for bad in (0, n - 1):
+            try:
+                t.insert(to_dev(X[:1]), ids_dev(np.array([bad], np.uint32)))
+                raise AssertionError("a stored id was inserted")
+            except pkd.PkdError:
+                pass
+        gone = np.arange(n + 5, dtype=np.uint32)[::2].copy()
+        assert t.delete(ids_dev(gone)) == o.delete(gone)
+        U.assert_exports_equal(t.export(), o.export())
+        back = gone[gone < n][::3].copy()
+        t.insert(to_dev(X[back]), ids_dev(back))
+        o.insert(X[back], back)
+        rest = np.arange(n, dtype=np.uint32)
+        assert t.delete(ids_dev(rest)) == o.delete(rest) and t.size == 0
+        t.close()
 g0 = graphs()
 X = I.uniform(100000, 3, 5)
 p = pkd.Params(d=3)
