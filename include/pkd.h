@@ -295,7 +295,9 @@ const char* pkd_strerror(int code);
  *                Until it is set, builds run as with 1, except that one whose
  *                subproblems are known to fit shared memory (a single tree of
  *                at most base_cap points, an update's rebuild of small
- *                subtrees) has no rounds and launches its base cases directly
+ *                subtrees) has no rounds and launches its base cases directly,
+ *                and that the larger rebuilds inside updates run as with 0
+ *                unless the same arguments (arena positions) come again
  *   "front_cap"  > 0: first capacity (entries) of the lists with which an
  *                update flattens the subtrees it rebuilds (testing; 0, the
  *                default, sizes them by the points of those subtrees).  A

@@ -1464,7 +1464,10 @@ struct GraphEntry {
   BaseShape shapes[MAX_SHAPES];
   uint64_t used = 0;
 };
-constexpr int GRAPH_CACHE = 16;
+// (A few trees built and updated in turn, on memory that the pool hands out in
+// different places, already cycle through more than 16 graphs: with 16 a step of
+// 1e7 clustered points recorded three graphs a pass, 7.0 against 6.1 ms.)
+constexpr int GRAPH_CACHE = 64;
 static std::vector<GraphEntry> g_graphs;   // guarded by flow_mutex()
 static std::vector<GraphEntry> g_retired;  // evicted, maybe still running
 static uint64_t g_graph_clock = 0;
@@ -1495,6 +1498,20 @@ static GraphEntry* graph_find(const std::vector<uint64_t>& key) {
       return &e;
     }
   return nullptr;
+}
+
+// Whether a key was looked for before (the last GRAPH_SEEN that were not in
+// the cache, by hash; guarded by flow_mutex() like the cache).
+constexpr size_t GRAPH_SEEN = 128;
+static bool graph_seen(const std::vector<uint64_t>& key) {
+  static std::vector<uint64_t> seen;
+  static size_t next = 0;
+  uint64_t h = 0;
+  for (uint64_t v : key) h = finalize64(h ^ v) + K_DEPTH;
+  if (std::find(seen.begin(), seen.end(), h) != seen.end()) return true;
+  if (seen.size() < GRAPH_SEEN) seen.push_back(h);
+  else seen[next++ % GRAPH_SEEN] = h;
+  return false;
 }
 
 static GraphEntry* graph_slot() {
@@ -2026,11 +2043,16 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
   };
 
   PKD_LAUNCH(k_ctl_init<<<1, 64, 0, s>>>(dctr, (uint32_t)nroots));
-  if (!graph) {
+  auto host_rounds = [&]() {
     PKD_TRY(classify(f));
-    PKD_TRY(flow_while(f, C_GO, round));
-    // the counts come back once more: every list gets its exact grid
-    PKD_TRY(flow_read(f));
+    // the first round is certain when a segment is known to exceed one CTA;
+    // the last read brings the base lists' lengths, for their exact grids
+    if (job.max_len <= cap || ktiming_enabled()) PKD_TRY(flow_read(f));
+    else hctr[C_GO] = 1;
+    while (hctr[C_GO]) {
+      PKD_TRY(round(f));
+      PKD_TRY(flow_read(f));
+    }
     if (job.before_base) job.before_base(nullptr);
     auto host_blocks = [&](int w, uint32_t per, uint32_t mx) {
       const uint32_t c = (uint32_t)std::min<uint64_t>(hctr[w], base_cap_segs);
@@ -2039,6 +2061,11 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
     };
     auto none = [](cudaStream_t, int, uint32_t, uint32_t) { return PKD_OK; };
     PKD_TRY(base_stage(sa, L, dctr, hctr, d, nsm, s, aux_stream(), host_blocks, none));
+    PKD_CUDA(cudaGetLastError());
+    return PKD_OK;
+  };
+  if (!graph) {
+    PKD_TRY(host_rounds());
   } else {
     // One graph: WHILE(another round) { ... WHILE(another skeleton level)
     // { ... } ... IF(exact levels) { ... } ... }, then the base cases as
@@ -2089,6 +2116,11 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
       PKD_CUDA(cudaGetLastError());
       return PKD_OK;
     }
+    // The rebuild of an update seldom meets its arguments again (its arena
+    // positions are new), and recording, instantiating and destroying a graph
+    // takes about 0.6 ms of host time, the host's reads of a rebuild's one or
+    // two rounds 0.1: only a repeated one is recorded.
+    if (knobs().graph_rounds < 0 && job.dsegs && !graph_seen(key)) return host_rounds();
 
     int nshape = 0;
     cudaGraphNode_t shape_nodes[MAX_SHAPES] = {};

@@ -73,6 +73,15 @@ p = pkd.Params(d=3)
 t = pkd.Tree(to_dev(X), None, p)
 assert graphs() == g0 + 1
 U.assert_exports_equal(t.export(), O.OracleTree(X, None, oparams(p)).export())
+# more build shapes than the graph cache holds: evicted graphs and fresh ones
+pkd.pkd_set_option("base_cap", 256)
+p = pkd.Params(d=2, phi=8, lam=3, sigma_log2=2, sigma_os=4)
+for i in range(80):
+    X = make_points("uniform", 3000 + 17 * (i % 75), 2, i)
+    t = pkd.Tree(to_dev(X), None, p)
+    if i % 8 == 0 or i > 74:
+        U.assert_exports_equal(t.export(), O.OracleTree(X, None, oparams(p)).export())
+    t.close()
 print("RESULT ok")
 '''
 
