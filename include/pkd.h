@@ -20,9 +20,10 @@
  *    exact levels run from one CUDA graph launch whose conditional nodes
  *    test counts the kernels leave in device memory, so the host does not
  *    wait between rounds (option "graph_rounds").  The rebuilds inside a
- *    batch update run the same way; the update's own routing rounds read
- *    their counts on the host.  Queries are asynchronous: their outputs are
- *    valid once `stream` has been synchronised.
+ *    batch update run the same way or are sequenced by the host; the routing
+ *    rounds of a batch of more than 4096 points read their counts on the
+ *    host, a smaller one's are queued together.  Queries are asynchronous:
+ *    their outputs are valid once `stream` has been synchronised.
  *  - A pkd_tree is not thread-safe: one call at a time per tree, except
  *    that queries on an unchanging tree may overlap.
  *  - Return value 0 (PKD_OK) or one of the error codes below; device-side
@@ -138,11 +139,9 @@ int pkd_knn(const pkd_tree* tree, const int32_t* queries, uint64_t q, int k, uin
  *   - calls whose device work overlaps (other streams, other host threads)
  *     race on the scratch; calls one after another on one stream do not;
  *   - the first call on a device is its set-up: it resolves the scratch
- *     address and runs every search kernel variant (all d, both k ranges)
- *     once on an empty query set, so that the kernels are loaded and the
- *     driver's local-memory reservation is sized for the largest of them
- *     (about 10 KB per resident thread at d = 8, k > 16); make that call
- *     before any region in which the caller may not allocate.  Later calls
+ *     address and runs every search kernel variant (all d, every k range)
+ *     once on an empty query set, so that the kernels are loaded and any
+ *     local memory they use is reserved; make that call before any region in which the caller may not allocate.  Later calls
  *     allocate nothing on the host or the device.
  * The call synchronises `stream` once (after the coordinate check) and
  * returns with the search queued on it; out_ids is valid once `stream` has
@@ -157,8 +156,8 @@ int pkd_knn_ids_noalloc(const pkd_tree* tree, const int32_t* queries, uint64_t q
                         uint32_t* out_ids, void* stream);
 
 /* Search depth (pkd_knn, pkd_range_count, pkd_range_report): each query's
- * depth-first stack holds up to height + 1 entries.  Below height 126 they
- * live in registers and local memory; a deeper tree (possible only after
+ * depth-first stack holds up to height + 1 entries (a box's a few hundred
+ * more).  Below height 126 they live in shared memory; a deeper tree (possible only after
  * long runs of one-sided updates with alpha near 1/2, where no interior node
  * is rebuilt) is searched with stacks in a scratch buffer of the library's
  * pool, at most 1 GiB, a chunk of queries at a time. */
@@ -292,12 +291,12 @@ const char* pkd_strerror(int code);
  *                are persistent launches over device-side lists; 0: the same
  *                kernels with the host reading the counts after every step
  *                (one stream synchronisation per round and skeleton level).
- *                Until it is set, builds run as with 1, except that one whose
- *                subproblems are known to fit shared memory (a single tree of
- *                at most base_cap points, an update's rebuild of small
- *                subtrees) has no rounds and launches its base cases directly,
- *                and that the larger rebuilds inside updates run as with 0
- *                unless the same arguments (arena positions) come again
+ *                Until it is set, builds run as with 1, except that a single
+ *                tree of at most base_cap points, which has no rounds, launches
+ *                its base cases directly.  With 1 or unset, the rebuilds
+ *                inside updates do the same when their subtrees fit shared
+ *                memory, and otherwise run as with 0 unless the same arguments
+ *                (arena positions) come again
  *   "front_cap"  > 0: first capacity (entries) of the lists with which an
  *                update flattens the subtrees it rebuilds (testing; 0, the
  *                default, sizes them by the points of those subtrees).  A

@@ -1730,6 +1730,10 @@ static int build_flat(TreeMem& t, const BuildJob& job, Scratch& sc) {
     PKD_TRY(dev_store(roots, job.segs.data(), nroots * sizeof(Seg), s));
   }
   BaseLists L = base_limits(d);
+  // Few enough segments above the small slice for one CTA each, all at once: a
+  // CTA finishes 500 points in a quarter of the time that a warp takes (131 us),
+  // and there are no others to fill the chip with.
+  if (job.extent / (L.tcap + 1) < 2 * (uint64_t)nsm) L.wcap = std::min(L.wcap, L.tcap);
   PKD_TRY(L.alloc(sc, job.extent, nroots));
   RoundDyn* dyn;
   PKD_TRY(sc.get(&dyn, 1));
@@ -1792,7 +1796,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
   const uint64_t base = job.base, extent = std::max<uint64_t>(job.extent, 1);
   const int nsm = num_sms();
   Scratch sc{s, {}};
-  if (job.max_len && job.max_len <= cap && knobs().graph_rounds != 1) return build_flat(t, job, sc);
+  if (job.max_len && job.max_len <= cap && (knobs().graph_rounds != 1 || job.dsegs)) return build_flat(t, job, sc);
 
   // scratch point buffer B and two sample buffers over [base, base + extent)
   int32_t *bc, *s0c, *s1c;
@@ -2120,7 +2124,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
     // positions are new), and recording, instantiating and destroying a graph
     // takes about 0.6 ms of host time, the host's reads of a rebuild's one or
     // two rounds 0.1: only a repeated one is recorded.
-    if (knobs().graph_rounds < 0 && job.dsegs && !graph_seen(key)) return host_rounds();
+    if (job.dsegs && !graph_seen(key)) return host_rounds();
 
     int nshape = 0;
     cudaGraphNode_t shape_nodes[MAX_SHAPES] = {};

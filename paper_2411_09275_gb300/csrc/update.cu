@@ -282,6 +282,62 @@ __global__ void k_front_expand(const Front* f, const uint32_t* nf, Front* g, uin
   }
 }
 
+// The whole flatten of a small update in one block: the roots, then level after
+// level, the lists' lengths in shared memory (a rebuilt subtree of a few hundred
+// points has four levels; as launches, the roots, a batch of levels and their
+// counters took 14 of 4 us each).  Returns after FRONT_LEVELS levels at most,
+// with what is left of the frontier in f and its length in fc[0].
+constexpr uint64_t FRONT_SMALL_POINTS = 8192, FRONT_SMALL_ITEMS = 16384;
+constexpr int FRONT_LEVELS = 128;  // even: f holds the frontier at the end
+__global__ void __launch_bounds__(512) k_front_small(const RebuildItem* it, const uint32_t* n, Front* f, Front* g,
+                                                     uint32_t* fc, Front* leaves, Front* bigleaves, const Node* nodes,
+                                                     const uint8_t* ndim, const uint32_t* aux, int use_aux,
+                                                     uint32_t cap, uint32_t bcap) {
+  __shared__ uint32_t nf[2], nl, nb, ovf;
+  if (threadIdx.x == 0) nf[0] = nf[1] = nl = nb = ovf = 0;
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < *n; i += blockDim.x)
+    if (!it[i].leaf && it[i].old_live != 0) f[atomicAdd(&nf[0], 1u)] = Front{it[i].slot, i, 0};  // the roots fit
+  __syncthreads();
+  int lev = 0;
+  for (; lev < FRONT_LEVELS; ++lev) {
+    const uint32_t c = min(nf[lev & 1], cap & ~1u);
+    if (c == 0 || ovf) break;  // uniform: nothing changes them before the barrier below
+    __syncthreads();
+    if (threadIdx.x == 0) nf[(lev + 1) & 1] = 0;
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < c; i += blockDim.x) {
+      const Front e = f[i];
+      const Node nd = nodes[e.slot];
+      if (ndim[e.slot] == PKD_LEAF) {
+        const bool big = nd.size > BIG_LEAF;
+        const uint32_t k = atomicAdd(big ? &nb : &nl, 1u);
+        if (k < (big ? bcap : cap)) (big ? bigleaves : leaves)[k] = e;
+        else ovf = 1;
+        continue;
+      }
+      const uint32_t llive = nodes[nd.a].size - (use_aux ? aux[nd.a] : 0u);
+      const uint32_t k = atomicAdd(&nf[(lev + 1) & 1], 2u);
+      if (k + 2 > cap) {
+        ovf = 1;
+        continue;
+      }
+      g[k] = Front{nd.a, e.item, e.off};
+      g[k + 1] = Front{nd.b, e.item, e.off + llive};
+    }
+    __syncthreads();
+    Front* t = f;
+    f = g;
+    g = t;
+  }
+  if (threadIdx.x == 0) {
+    fc[0] = lev == FRONT_LEVELS ? nf[0] : 0u;
+    fc[1] = ovf;
+    fc[2] = nl;
+    fc[3] = nb;
+  }
+}
+
 // Flattened leaves, UPW per warp: copy their live points to the item's range.
 template <int D>
 __global__ void __launch_bounds__(UPW_WARPS * 32) k_copy_leaves(const Front* lv, const uint32_t* n,
@@ -987,10 +1043,20 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
         PKD_TRY(sc.get(&fb, fcap32));
         PKD_TRY(sc.get(&leaves, fcap32));
         PKD_TRY(sc.get(&bigleaves, bcap32));
-        PKD_TRY(dev_fill(fc, 0, 16, s));
-        PKD_LAUNCH(k_front_init<<<gi, 128, 0, s>>>(items, d_nitems, fa, fc));
         int levels = 0;
-        do {
+        if (inner_total <= FRONT_SMALL_POINTS && nitems <= FRONT_SMALL_ITEMS) {
+          PKD_LAUNCH(k_front_small<<<1, 512, 0, s>>>(items, d_nitems, fa, fb, fc, leaves, bigleaves, t.nodes, t.ndim,
+                                                     t.aux, insert ? 0 : 1, fcap32, bcap32));
+          levels = FRONT_LEVELS;
+          PKD_CUDA(cudaMemcpyAsync(hf, fc, 16, cudaMemcpyDeviceToHost, s));
+          PKD_CUDA(cudaStreamSynchronize(s));
+        } else {
+          PKD_TRY(dev_fill(fc, 0, 16, s));
+          PKD_LAUNCH(k_front_init<<<gi, 128, 0, s>>>(items, d_nitems, fa, fc));
+          hf[0] = 1;
+          hf[1] = 0;
+        }
+        while (hf[0] != 0 && hf[1] == 0) {
           if (levels > 100000) return PKD_EINTERNAL;
           PKD_TRY(dev_fill(lc + 1, 0, (size_t)FRONT_BATCH * 4, s));
           PKD_TRY(dev_copy_words(lc, fc, 1, s));
@@ -1004,7 +1070,7 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
           PKD_TRY(dev_copy_words(fc, lc + FRONT_BATCH, 1, s));
           PKD_CUDA(cudaMemcpyAsync(hf, fc, 16, cudaMemcpyDeviceToHost, s));
           PKD_CUDA(cudaStreamSynchronize(s));
-        } while (hf[0] != 0 && hf[1] == 0);
+        }
         if (hf[1] == 0) break;
         // a list overflowed: nothing the tree shows has changed yet
         if (fcap >= big_fcap) return PKD_EINTERNAL;

@@ -101,3 +101,31 @@ def test_rejected_and_empty_batches():
         assert t.delete(ids_dev(np.concatenate([yid, yid[:3]]))) == o.delete(np.concatenate([yid, yid[:3]])) == m
         _same(t, o)
     t.close()
+
+
+@pytest.mark.parametrize("n", [700, 6000])
+def test_small_flatten_overflow_is_redone(n):
+    # a subtree of up to 8192 points is flattened by one block.  At alpha = 0 the
+    # insert rebuilds the root: 6000 points in leaves of at most 2 overflow the
+    # smallest lists (1024 entries above the roots'), which are then redone larger
+    from paper_2411_09275_gb300 import pkd as P
+    from tests.gpuutil import knobs
+
+    pkd, t, o, X = _pair("uniform", n, 3, 97, phi=2, lam=3, sigma_log2=2, sigma_os=4, alpha_num=0)
+    Y = I.uniform(n // 2, 3, 98)
+    Y[:, 0] //= 64
+    yid = np.arange(n, n + n // 2, dtype=np.uint32)
+    P.pkd_kernel_timing(True)
+    try:
+        with knobs(front_cap=64):
+            t.insert(to_dev(Y), ids_dev(yid))
+            retries = P.pkd_kernel_stats("front_retries")[0]
+            o.insert(Y, yid)
+            _same(t, o)
+            gone = yid[: n // 3]
+            assert t.delete(ids_dev(gone)) == o.delete(gone)
+            _same(t, o)
+    finally:
+        P.pkd_kernel_timing(False)
+    assert retries == (1 if n == 6000 else 0)
+    t.close()
