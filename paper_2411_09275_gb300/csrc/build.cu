@@ -182,17 +182,18 @@ __global__ void __launch_bounds__(SM_THREADS, 1) k_smem_build(SmemArgs a) {
 // and for two (half the shared memory and at most 64 registers a thread);
 // the segment lists of the two launches are separated when the segments are
 // classified.
-template <int D>
+template <int D, int NW>
 __device__ __forceinline__ void smem_sorted_one(const SmemArgs& a, uint32_t sid) {
+  constexpr int NT = NW * 32;
   extern __shared__ __align__(16) uint8_t sm[];
   const Seg seg = a.segs[sid];
   const int cap = a.cap, tid = threadIdx.x;
-  const SortedLayout Lo = sorted_layout(cap, D);
+  const SortedLayout Lo = sorted_layout(cap, D, NW);
   int32_t* X = (int32_t*)(sm + Lo.X);
   uint32_t* ID = (uint32_t*)(sm + Lo.ID);
   int* sred = (int*)(sm + Lo.red);
   STask* wstack = (STask*)(sm + Lo.stack);
-  SmemCtl* ctl = (SmemCtl*)(sm + Lo.ctl);
+  SortedCtl* ctl = (SortedCtl*)(sm + Lo.ctl);
   if (seg.len > (uint32_t)cap) {
     if (tid == 0) set_error(a.st, DERR_CAPACITY, 400000 + (int)sid);
     return;
@@ -213,7 +214,7 @@ __device__ __forceinline__ void smem_sorted_one(const SmemArgs& a, uint32_t sid)
     ctl->next_slot = 0;
     ctl->maxd = 0;
   }
-  if (tid < SS_NW) ctl->wsp[tid] = 0;
+  if (tid < NW) ctl->wsp[tid] = 0;
   __syncthreads();
   int lmn[D], lmx[D];
 #pragma unroll
@@ -232,12 +233,12 @@ __device__ __forceinline__ void smem_sorted_one(const SmemArgs& a, uint32_t sid)
     src_c[j] = aos ? a.in_coords + seg.start * (uint64_t)D + j : S.c + (uint64_t)j * S.stride + seg.start;
   const uint32_t* src_id = aos ? (a.in_ids ? a.in_ids + seg.start : nullptr) : S.id + seg.start;
   const int cstep = aos ? D : 1;
-  for (int i0 = tid; i0 < n; i0 += LU * SS_THREADS) {
+  for (int i0 = tid; i0 < n; i0 += LU * NT) {
     int32_t v[LU][D];
     uint32_t id[LU];
 #pragma unroll
     for (int u = 0; u < LU; ++u) {
-      const int i = i0 + u * SS_THREADS;
+      const int i = i0 + u * NT;
       if (i < n) {
 #pragma unroll
         for (int j = 0; j < D; ++j) v[u][j] = src_c[j][i * cstep];
@@ -246,7 +247,7 @@ __device__ __forceinline__ void smem_sorted_one(const SmemArgs& a, uint32_t sid)
     }
 #pragma unroll
     for (int u = 0; u < LU; ++u) {
-      const int i = i0 + u * SS_THREADS;
+      const int i = i0 + u * NT;
       if (i < n) {
 #pragma unroll
         for (int j = 0; j < D; ++j) {
@@ -296,12 +297,12 @@ __device__ __forceinline__ void smem_sorted_one(const SmemArgs& a, uint32_t sid)
   unsigned* hist = (unsigned*)wstack;  // the task stacks are not in use yet
 #pragma unroll 1
   for (int k = 0; k < D; ++k)
-    if (!presort_dim_msd<D>(cx, k, vmn[k], vmx[k], n, hist, sred + 2 * D))
-      presort_dim<D>(cx, k, vmn[k], vmx[k], n, hist, sred + 2 * D);
+    if (!presort_dim_msd<D, NW>(cx, k, vmn[k], vmx[k], n, hist, sred + 2 * D))
+      presort_dim<D, NW>(cx, k, vmn[k], vmx[k], n, hist, sred + 2 * D);
   uint32_t map = 0;
 #pragma unroll
   for (int k = 0; k < D; ++k) map |= (uint32_t)k << (4 * k);
-  srun_tasks<D>(cx, STask{0, (uint16_t)n, 0, 0, 0, seg.depth, seg.root, map, 0}, sred, wstack);
+  srun_tasks<D, NW>(cx, STask{0, (uint16_t)n, 0, 0, 0, seg.depth, seg.root, map, 0}, sred, wstack);
   __syncthreads();
   // every leaf left its points' indices in list 0: write the subproblem out
   // in leaf order, coalesced
@@ -311,7 +312,7 @@ __device__ __forceinline__ void smem_sorted_one(const SmemArgs& a, uint32_t sid)
 #pragma unroll
     for (int j = 0; j < D; ++j) oc[j] = a.A.c + (uint64_t)j * a.A.stride + seg.start;
     uint32_t* oid = a.A.id + seg.start;
-    for (int i = tid; i < n; i += SS_THREADS) {
+    for (int i = tid; i < n; i += NT) {
       const int p = P[i];
       if (p >= n) continue;  // only after a recorded error, when leaves are missing
 #pragma unroll
@@ -324,9 +325,9 @@ __device__ __forceinline__ void smem_sorted_one(const SmemArgs& a, uint32_t sid)
 
 // One CTA per entry of the list (a persistent loop around this body costs
 // registers the two-CTAs-per-SM form does not have: it would spill).
-template <int D, int MINB>
-__global__ void __launch_bounds__(SS_THREADS, MINB) k_smem_sorted(SmemArgs a) {
-  if (blockIdx.x < list_len(a.nsegs, a.list_cap)) smem_sorted_one<D>(a, blockIdx.x);
+template <int D, int MINB, int NW = SS_NW>
+__global__ void __launch_bounds__(NW * 32, MINB) k_smem_sorted(SmemArgs a) {
+  if (blockIdx.x < list_len(a.nsegs, a.list_cap)) smem_sorted_one<D, NW>(a, blockIdx.x);
 }
 
 template <int D>
@@ -472,15 +473,32 @@ static void launch_smem_build(const SmemArgs& a, uint32_t nblocks, size_t smb, c
   launch_with_smem(k_smem_build<D>, &set, nblocks, SM_THREADS, smb, s, a);
 }
 
+static int smem_optin();
+
+// One CTA per SM: 32 warps where 64 registers a thread do not spill (d <= 5)
+// and their stacks and counters fit beside the points (always at the derived
+// capacity; a larger one that the caller sets may need the 16), unless other
+// work shares the SMs: 32 warps hold all of an SM's registers, so a CTA waits
+// for the id table's CTAs to leave.  512 trees of 1e3 to 1e6 points (no id
+// tables): 10.58 -> 10.24 ms; a step of 1e8 points beside their table: 22.13
+// with 16 warps, 22.95 with 32.
 template <int D>
-static void launch_smem_sorted(const SmemArgs& a, uint32_t nblocks, size_t smb, cudaStream_t s) {
+static void launch_smem_sorted(const SmemArgs& a, uint32_t nblocks, bool shared, cudaStream_t s) {
+  if constexpr (D <= 5) {
+    const size_t wide = sorted_layout(a.cap, D, SS_WIDE).total;
+    if (!shared && wide <= (size_t)smem_optin()) {
+      static int set = 0;
+      launch_with_smem(k_smem_sorted<D, 1, SS_WIDE>, &set, nblocks, SS_WIDE * 32, wide, s, a);
+      return;
+    }
+  }
   static int set = 0;
-  launch_with_smem(k_smem_sorted<D, 1>, &set, nblocks, SS_THREADS, smb, s, a);
+  launch_with_smem(k_smem_sorted<D, 1>, &set, nblocks, SS_NW * 32, sorted_layout(a.cap, D).total, s, a);
 }
 template <int D>
 static void launch_smem_sorted2(const SmemArgs& a, uint32_t nblocks, size_t smb, cudaStream_t s) {
   static int set = 0;
-  launch_with_smem(k_smem_sorted<D, 2>, &set, nblocks, SS_THREADS, smb, s, a);
+  launch_with_smem(k_smem_sorted<D, 2>, &set, nblocks, SS_NW * 32, smb, s, a);
 }
 
 // A second stream of the current device, created on first use.
@@ -1600,6 +1618,7 @@ struct BaseLists {
   Seg *one, *two, *warp, *tiny;
   uint32_t n_one, n_two, n_warp, n_tiny;  // entries they can hold
   uint32_t cap, cap2, wcap, tcap;
+  bool shared;  // other work runs beside the base cases
 
   // Room for at most `segs` segments of `extent` points together: a list of
   // segments longer than x points has at most extent / (x + 1) of them.
@@ -1616,8 +1635,9 @@ struct BaseLists {
   }
 };
 
-static BaseLists base_limits(int d) {
+static BaseLists base_limits(int d, const BuildJob& job) {
   BaseLists L{};
+  L.shared = (bool)job.before_base;
   L.cap = (uint32_t)base_cap_for(d);
   L.wcap = (uint32_t)warp_cap_for(d);
   L.tcap = 128;
@@ -1668,7 +1688,7 @@ static int base_stage(const SmemArgs& sa, const BaseLists& L, const uint32_t* dc
       PKD_CUDA(cudaEventCreateWithFlags(&join, cudaEventDisableTiming));
       PKD_CUDA(cudaEventRecord(fork, q));
       PKD_CUDA(cudaStreamWaitEvent(aux, fork, 0));
-      PKD_DISPATCH_D(d, launch_smem_sorted, s1, b1, sorted_layout((int)L.cap, d).total, aux);
+      PKD_DISPATCH_D(d, launch_smem_sorted, s1, b1, L.shared, aux);
       PKD_TRY(recorded(aux, C_NBBASE, 1u, 0u));
     }
     SmemArgs s2 = sa;
@@ -1729,7 +1749,7 @@ static int build_flat(TreeMem& t, const BuildJob& job, Scratch& sc) {
     PKD_TRY(sc.get(&roots, std::max<uint64_t>(nroots, 1)));
     PKD_TRY(dev_store(roots, job.segs.data(), nroots * sizeof(Seg), s));
   }
-  BaseLists L = base_limits(d);
+  BaseLists L = base_limits(d, job);
   // Few enough segments above the small slice for one CTA each, all at once: a
   // CTA finishes 500 points in a quarter of the time that a warp takes (131 us),
   // and there are no others to fill the chip with.
@@ -1828,7 +1848,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
   }
   // every base segment is a root or a non-empty bucket: at most extent + roots
   const uint64_t base_cap_segs = extent + nroots + 16;
-  BaseLists L = base_limits(d);
+  BaseLists L = base_limits(d, job);
   PKD_TRY(L.alloc(sc, extent, base_cap_segs));
 
   // worst-case round buffers
@@ -2101,7 +2121,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
       put((uint64_t)p.d), put((uint64_t)p.phi), put((uint64_t)p.lambda), put((uint64_t)p.sigma_log2);
       put((uint64_t)p.sigma_os), put((uint64_t)p.count_mode), put((uint64_t)p.alpha_num), put((uint64_t)p.alpha_den);
       put(p.seed);
-      put((uint64_t)TILE), put(cap), put((uint64_t)scap), put(L.cap2), put(L.wcap), put((uint64_t)nsm);
+      put((uint64_t)TILE), put(cap), put((uint64_t)scap), put(L.cap2), put(L.wcap), put((uint64_t)L.shared), put((uint64_t)nsm);
       put((uint64_t)knobs().sieve_kernel), put((uint64_t)knobs().base_kernel), put((uint64_t)knobs().wait_cycles);
       put((uint64_t)record_buckets(NB));
     }

@@ -25,7 +25,7 @@
 // so their buffers never collide.
 //
 // Scheduling is the team scheme of the radix-select frame: the root is
-// processed by all 16 warps, teams halve at every split (tiny children are
+// processed by all 16 (or 32) warps, teams halve at every split (tiny children are
 // deferred to the first warp's stack), single warps finish their subtrees
 // depth first, always continuing with the smaller child.
 #pragma once
@@ -34,8 +34,11 @@
 
 namespace pkd {
 
+// Warps of a CTA: 16, or 32 (SS_WIDE) where one CTA has the SM to itself: the
+// node steps wait on shared memory and barriers, and 32 warps with 64
+// registers hide more of it, as two CTAs of 16 do.
 constexpr int SS_NW = 16;
-constexpr int SS_THREADS = SS_NW * 32;
+constexpr int SS_WIDE = 32;
 constexpr int SS_RED = 2 * PKD_DMAX + 8;  // reduction ints per warp
 constexpr int SS_STK = 32;                // deferred tasks per warp
 
@@ -49,13 +52,19 @@ struct STask {
 };
 static_assert(sizeof(STask) == 24, "STask layout");
 
+struct SortedCtl {
+  int next_slot;
+  unsigned maxd;     // deepest leaf written by this CTA
+  int wsp[SS_WIDE];  // per-warp stack depth
+};
+
 struct SortedLayout {
   size_t X, ID, lists, flag, red, stack, ctl, total;
 };
 
 // Shared memory of one CTA holding up to `cap` points of d dimensions.  The
-// radix counters of the presort (16 warps x 256 u32) share the task stacks.
-__host__ __device__ inline SortedLayout sorted_layout(int cap, int d) {
+// radix counters of the presort (256 u32 a warp) share the task stacks.
+__host__ __device__ inline SortedLayout sorted_layout(int cap, int d, int nw = SS_NW) {
   SortedLayout L;
   size_t o = 0;
   L.X = o;
@@ -67,12 +76,12 @@ __host__ __device__ inline SortedLayout sorted_layout(int cap, int d) {
   L.flag = o;
   o = align_up(o + (size_t)cap, 16);
   L.red = o;
-  o = align_up(o + (size_t)SS_NW * SS_RED * 4, 16);
+  o = align_up(o + (size_t)nw * SS_RED * 4, 16);
   L.stack = o;
-  const size_t stk = (size_t)SS_NW * SS_STK * sizeof(STask), hist = (size_t)SS_NW * 256 * 4;
+  const size_t stk = (size_t)nw * SS_STK * sizeof(STask), hist = (size_t)nw * 256 * 4;
   o = align_up(o + (stk > hist ? stk : hist), 16);
   L.ctl = o;
-  o = align_up(o + sizeof(SmemCtl), 16);
+  o = align_up(o + sizeof(SortedCtl), 16);
   L.total = o;
   return L;
 }
@@ -97,7 +106,7 @@ struct SCtx {
   uint8_t* flag;
   uint16_t* lists;  // [D + 1][cap]
   int cap;
-  SmemCtl* ctl;
+  SortedCtl* ctl;
   Pts out;
   uint64_t start;
   uint32_t slot_base;
@@ -118,10 +127,11 @@ struct SCtx {
 // ---------------------------------------------------------------------------
 constexpr int SS_BATCH = 4;
 
+template <int NW>
 __device__ __forceinline__ void radix_pass(const int32_t* Xj, unsigned vmin, int shift, const uint16_t* src,
                                            uint16_t* dst, int n, unsigned* hist, int* tmp) {
   const int w = warp_id(), lane = lane_id(), tid = threadIdx.x;
-  const int per = ((n + SS_THREADS - 1) / SS_THREADS) * 32;
+  const int per = ((n + NW * 32 - 1) / (NW * 32)) * 32;
   const int wlo = min(n, w * per), whi = min(n, wlo + per);
   const int ng = (whi - wlo + 31) >> 5;
   unsigned* H = hist + w * 256;
@@ -144,23 +154,29 @@ __device__ __forceinline__ void radix_pass(const int32_t* Xj, unsigned vmin, int
     }
   }
   __syncthreads();
-  // exclusive offsets per (digit, warp), digit-major: lanes 2i and 2i+1 of
-  // warp w own digit 16w + i, each summing the counters of 8 warps
+  // exclusive offsets per (digit, warp), digit-major: LPD neighbouring lanes
+  // own a digit, each summing the counters of 8 warps
   {
-    const int dgt = tid >> 1, h = tid & 1;
+    constexpr int LPD = NW / 8;
+    const int dgt = tid / LPD, h = tid % LPD;
     unsigned part = 0;
 #pragma unroll
-    for (int v = 0; v < SS_NW / 2; ++v) part += hist[(h * (SS_NW / 2) + v) * 256 + dgt];
-    const unsigned other = __shfl_xor_sync(FULL_MASK, part, 1);
-    const unsigned tot = part + other;
+    for (int v = 0; v < 8; ++v) part += hist[(h * 8 + v) * 256 + dgt];
+    unsigned tot = part, before = 0;  // of the digit; in its lanes before this one
+#pragma unroll
+    for (int o = 1; o < LPD; o <<= 1) {
+      const unsigned other = __shfl_xor_sync(FULL_MASK, tot, o);
+      if (h & o) before += other;
+      tot += other;
+    }
     const unsigned inc = (unsigned)warp_incl_scan(h == 0 ? (int)tot : 0);
     if (lane == 31) tmp[w] = (int)inc;
     __syncthreads();
-    unsigned run = inc - tot + (h ? other : 0u);
+    unsigned run = inc - tot + before;
     for (int v = 0; v < w; ++v) run += (unsigned)tmp[v];
 #pragma unroll
-    for (int v = 0; v < SS_NW / 2; ++v) {
-      unsigned* c = &hist[(h * (SS_NW / 2) + v) * 256 + dgt];
+    for (int v = 0; v < 8; ++v) {
+      unsigned* c = &hist[(h * 8 + v) * 256 + dgt];
       const unsigned cnt = *c;
       *c = run;
       run += cnt;
@@ -197,7 +213,7 @@ __device__ __forceinline__ void radix_pass(const int32_t* Xj, unsigned vmin, int
 
 // Sort dimension k of the n loaded points into buffer k (buffer D is the
 // ping-pong partner).  vmin/vmax bound the coordinates.
-template <int D>
+template <int D, int NW>
 __device__ void presort_dim(const SCtx<D>& cx, int k, int vmin, int vmax, int n, unsigned* hist, int* tmp) {
   const int32_t* Xk = cx.X + k * cx.cap;
   uint16_t* target = cx.list(k);
@@ -206,7 +222,7 @@ __device__ void presort_dim(const SCtx<D>& cx, int k, int vmin, int vmax, int n,
   const int bits = range ? 32 - __clz(range) : 0;
   const int passes = (bits + 7) / 8;
   if (passes == 0) {
-    for (int i = threadIdx.x; i < n; i += SS_THREADS) target[i] = (uint16_t)i;
+    for (int i = threadIdx.x; i < n; i += NW * 32) target[i] = (uint16_t)i;
     __syncthreads();
     return;
   }
@@ -214,7 +230,7 @@ __device__ void presort_dim(const SCtx<D>& cx, int k, int vmin, int vmax, int n,
   uint16_t* out = (passes & 1) ? target : partner;
   const uint16_t* in = nullptr;
   for (int ps = 0; ps < passes; ++ps) {
-    radix_pass(Xk, (unsigned)vmin, 8 * ps, in, out, n, hist, tmp);
+    radix_pass<NW>(Xk, (unsigned)vmin, 8 * ps, in, out, n, hist, tmp);
     in = out;
     out = (out == target) ? partner : target;
   }
@@ -232,11 +248,11 @@ __device__ void presort_dim(const SCtx<D>& cx, int k, int vmin, int vmax, int n,
 constexpr int MSD_BITS = 12;
 constexpr int MSD_BINS = 1 << MSD_BITS;  // 4096 counters fill the 16 KB radix region
 constexpr int MSD_MAX_BUCKET = 64;
-constexpr int MSD_PER = MSD_BINS / SS_THREADS;  // bins per thread
 
-template <int D>
+template <int D, int NW>
 __device__ bool presort_dim_msd(const SCtx<D>& cx, int k, int vmin, int vmax, int n, unsigned* hist, int* tmp) {
-  static_assert(MSD_PER * SS_THREADS == MSD_BINS && MSD_BINS <= SS_NW * 256, "bins per thread, radix region");
+  constexpr int NT = NW * 32, MSD_PER = MSD_BINS / NT;  // bins per thread
+  static_assert(MSD_PER * NT == MSD_BINS && MSD_BINS <= NW * 256, "bins per thread, radix region");
   const int32_t* Xk = cx.X + k * cx.cap;
   uint16_t* target = cx.list(k);
   const unsigned range = (unsigned)vmax - (unsigned)vmin;
@@ -244,9 +260,9 @@ __device__ bool presort_dim_msd(const SCtx<D>& cx, int k, int vmin, int vmax, in
   const int shift = max(0, bits - MSD_BITS);
   const int tid = threadIdx.x, lane = lane_id(), w = warp_id();
 #pragma unroll
-  for (int q = 0; q < MSD_PER; ++q) hist[q * SS_THREADS + tid] = 0;
+  for (int q = 0; q < MSD_PER; ++q) hist[q * NT + tid] = 0;
   __syncthreads();
-  for (int i = tid; i < n; i += SS_THREADS) atomicAdd(&hist[((unsigned)Xk[i] - (unsigned)vmin) >> shift], 1u);
+  for (int i = tid; i < n; i += NT) atomicAdd(&hist[((unsigned)Xk[i] - (unsigned)vmin) >> shift], 1u);
   __syncthreads();
   // bin starts: thread t owns bins [MSD_PER t, MSD_PER (t + 1))
   unsigned c[MSD_PER], sum = 0, mx = 0;
@@ -259,12 +275,12 @@ __device__ bool presort_dim_msd(const SCtx<D>& cx, int k, int vmin, int vmax, in
   const unsigned inc = (unsigned)warp_incl_scan((int)sum);
   const unsigned wmx = (unsigned)warp_max((int)mx);
   if (lane == 31) tmp[w] = (int)inc;
-  if (lane == 0) tmp[SS_NW + w] = (int)wmx;
+  if (lane == 0) tmp[NW + w] = (int)wmx;
   __syncthreads();
   unsigned run = inc - sum, big = 0;
-  for (int v = 0; v < SS_NW; ++v) {
+  for (int v = 0; v < NW; ++v) {
     if (v < w) run += (unsigned)tmp[v];
-    big = max(big, (unsigned)tmp[SS_NW + v]);
+    big = max(big, (unsigned)tmp[NW + v]);
   }
   if (big > (unsigned)MSD_MAX_BUCKET) {
     __syncthreads();  // every thread has read tmp before the caller reuses it
@@ -277,11 +293,11 @@ __device__ bool presort_dim_msd(const SCtx<D>& cx, int k, int vmin, int vmax, in
   }
   __syncthreads();
   uint16_t* binned = cx.list(D);
-  for (int i = tid; i < n; i += SS_THREADS)
+  for (int i = tid; i < n; i += NT)
     binned[atomicAdd(&hist[((unsigned)Xk[i] - (unsigned)vmin) >> shift], 1u)] = (uint16_t)i;
   __syncthreads();
   // hist[b] is now the end of bin b
-  for (int i = tid; i < n; i += SS_THREADS) {
+  for (int i = tid; i < n; i += NT) {
     const int v = binned[i];
     const int32_t kv = Xk[v];
     const unsigned b = ((unsigned)kv - (unsigned)vmin) >> shift;
@@ -834,14 +850,20 @@ __device__ void swarp_run(const Team& wt, const SCtx<D>& cx, STask tk, STask* st
 }
 
 // Drive the warps of the CTA over the root task.
-template <int D>
+//
+// Barriers: teams alive together are disjoint ranges of at least two warps, so
+// the id f / 2 + 1 tells them apart (a left child goes on with its parent's,
+// which is complete by then).  A CTA has ids 1 to 15 beside the one of
+// __syncthreads, so of 32 warps the last pair is not a team: warp 30 takes its
+// node alone and warp 31 is done.
+template <int D, int NW>
 __device__ void srun_tasks(const SCtx<D>& cx, STask root, int* sred, STask* wstack) {
   const int w = warp_id();
-  int f = 0, nw = SS_NW;
+  int f = 0, nw = NW;
   STask tk = root;
   bool have_task = true;
   while (nw > 1) {
-    const Team tm{f, nw, team_barrier(f, nw, SS_NW), nullptr, sred + f * SS_RED};
+    const Team tm{f, nw, NW == SS_NW ? team_barrier(f, nw, NW) : f / 2 + 1, nullptr, sred + f * SS_RED};
     SKids ch;
     if (!snode<D>(tm, cx, tk, ch)) {
       have_task = false;
@@ -867,6 +889,10 @@ __device__ void srun_tasks(const SCtx<D>& cx, STask root, int* sred, STask* wsta
     tk = skid(tk, ch, second);
     if (second) f += half;
     nw = half;
+    if (NW == 32 && f == 30) {
+      have_task = w == 30;
+      break;
+    }
   }
   __syncwarp();
   int sp0 = cx.ctl->wsp[w];
