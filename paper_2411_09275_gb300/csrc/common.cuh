@@ -66,8 +66,9 @@ struct DevStatus {
   int detail;
   uint32_t max_depth;
   int idflags;  // id-table flags of the running call (IDF_* in ids.cuh)
-  unsigned long long refused;  // number of the last query call whose coordinates were out of range
-  unsigned long long counters[8];
+  // numbers of the last query calls whose coordinates were out of range, by
+  // number % 16 (queries on an unchanging tree may overlap)
+  unsigned long long refused[16];
 };
 
 __device__ __forceinline__ void set_error(DevStatus* st, int code, int detail) {

@@ -13,9 +13,9 @@
 // parent's minus the old offset squared plus the new one squared (the same
 // number as the distance to the box that the splitters imply).
 //
-// What bounds it: instruction issue (68% of the issue slots busy with 8 lanes
-// a query, 15% of the DRAM bandwidth, half of the loads hit L2), about a
-// third of it list insertions; small batches are bound by the chain of
+// What bounds it: dependent loads (37% of the stalls with 4 lanes a query, 50%
+// of the L1's misses hit L2, 20% of the DRAM bandwidth) and instructions (the SMs
+// 60% busy, about a third of it list insertions); small batches are bound by the chain of
 // dependent loads down the tree (about 20 us for one 10-NN query in 1e6 2-D
 // points).  One thread per query (before) kept the stack, with the 2d bounds
 // of every waiting subspace, and the k entries in local memory.  10-NN, time

@@ -361,7 +361,7 @@ __global__ void k_query_check(const int32_t* c1, uint64_t n1, const int32_t* c2,
   }
   const unsigned b = coord_bits(c1, n1) | (c2 ? coord_bits(c2, n2) : 0);
   if (__any_sync(0xffffffffu, (b >> 30) != 0) && (threadIdx.x & 31) == 0) {
-    *(volatile unsigned long long*)&st->refused = call;
+    *(volatile unsigned long long*)&st->refused[call % 16] = call;
     *(volatile int*)&h->bad = 1;
   }
 }

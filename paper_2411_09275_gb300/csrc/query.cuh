@@ -59,7 +59,7 @@ class QueryCheck {
 };
 // In the searches: was the call refused?  (The same answer in all lanes.)
 __device__ __forceinline__ bool query_refused(const QueryArgs& a) {
-  const bool no = a.call && (pkd_failed(a.st) || *(volatile const unsigned long long*)&a.st->refused == a.call);
+  const bool no = a.call && (pkd_failed(a.st) || *(volatile const unsigned long long*)&a.st->refused[a.call % 16] == a.call);
   return __any_sync(0xffffffffu, no);
 }
 

@@ -128,3 +128,40 @@ def test_refused_queries_write_nothing_and_offsets_bound_the_ids():
             assert (out[:n] == ids).all().item()
     assert np.array_equal(t.range_count(gl[:50], gh[:50]).cpu().numpy().astype(np.uint64), o.range_count(lo[:50], hi[:50]))
     t.close()
+
+
+def test_refused_queries_that_overlap_write_nothing():
+    # two threads on streams of their own: one call's refusal must not hide the other's
+    import threading
+
+    import torch
+
+    pkd, t, o, X = _tree("uniform", 5000, 3, 32, 71)
+    bad = to_dev(np.full((64, 3), 1 << 30, np.int32))
+    outs, errors = [], []
+
+    def calls():
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            oi = torch.full((64, 5), -7, dtype=torch.int32, device="cuda")
+            od = torch.full((64, 5), -7, dtype=torch.int64, device="cuda")
+            for _ in range(200):
+                try:
+                    pkd.pkd_knn(t._h, bad, 5, oi, od, stream=s)
+                    errors.append("a refused call was served")
+                except pkd.PkdError as e:
+                    if e.code != pkd.PKD_EINVAL:
+                        errors.append(e.code)
+            s.synchronize()
+            outs.append((oi, od))
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=calls) for _ in range(2)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    torch.cuda.synchronize()
+    assert not errors and len(outs) == 2
+    assert all((oi == -7).all().item() and (od == -7).all().item() for oi, od in outs)
+    t.close()
