@@ -501,20 +501,53 @@ static void launch_smem_sorted2(const SmemArgs& a, uint32_t nblocks, size_t smb,
   launch_with_smem(k_smem_sorted<D, 2>, &set, nblocks, SS_NW * 32, smb, s, a);
 }
 
-// A second stream of the current device, created on first use.
-static cudaStream_t aux_stream() {
-  static std::mutex mu;
-  static std::map<int, cudaStream_t> streams;
+// The helper stream of this host thread for direct launches, on the current
+// device (created on first use, handed to another thread when this one ends).
+// Builds on different trees may run from several threads at once.  One stream
+// for all of them would order one build behind another's, and it would be part
+// of another thread's graph while that is recorded: what is launched on it then
+// goes into that graph, or invalidates it.  Recording has a stream of its own
+// for the same reason (capture_helper_stream).  A call waits for its work
+// before it returns, so a stream handed on is idle.
+static cudaStream_t helper_stream() {
+  struct Pool {
+    std::mutex mu;
+    std::map<int, std::vector<cudaStream_t>> idle;  // by device
+  };
+  static Pool* const pool = new Pool();  // outlives every thread
+  struct Mine {
+    std::map<int, cudaStream_t> by_dev;
+    Pool* pool;
+    ~Mine() {
+      std::lock_guard<std::mutex> lk(pool->mu);
+      for (auto& e : by_dev) pool->idle[e.first].push_back(e.second);
+    }
+  };
+  static thread_local Mine mine{{}, pool};
   int dev = 0;
   cudaGetDevice(&dev);
-  std::lock_guard<std::mutex> lk(mu);
-  auto it = streams.find(dev);
-  if (it != streams.end()) return it->second;
+  auto it = mine.by_dev.find(dev);
+  if (it != mine.by_dev.end()) return it->second;
   cudaStream_t st = nullptr;
-  cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
-  streams[dev] = st;
+  {
+    std::lock_guard<std::mutex> lk(pool->mu);
+    auto& idle = pool->idle[dev];
+    if (!idle.empty()) {
+      st = idle.back();
+      idle.pop_back();
+    }
+  }
+  if (!st && cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  mine.by_dev[dev] = st;
   return st;
 }
+
+// The second stream of a build that is being recorded (under flow_mutex): a
+// level that no loop has.
+static cudaStream_t capture_helper_stream() { return flow_stream(-1); }
 
 // Largest capacity of the presorted base case that lets two CTAs share an
 // SM (each gets half of the SM's shared memory, less the per-CTA reserve).
@@ -1648,10 +1681,11 @@ static BaseLists base_limits(int d, const BuildJob& job) {
 
 // Every small subproblem, in shared memory, one CTA (or warp) per entry of
 // the base lists: `q` is the stream, `list_blocks(w, per, max)` the grid of
-// the list whose length is control word w.
+// the list whose length is control word w, `helper` the second stream (not
+// created before it is needed).
 template <class LB, class RC>
 static int base_stage(const SmemArgs& sa, const BaseLists& L, const uint32_t* dctr, const uint32_t* hctr, int d, int nsm,
-                      cudaStream_t q, cudaStream_t aux, LB&& list_blocks, RC&& recorded) {
+                      cudaStream_t q, cudaStream_t (*helper)(), LB&& list_blocks, RC&& recorded) {
   const uint64_t cta_pts = *(unsigned long long*)(hctr + C_BASE_PTS);
   const uint64_t warp_pts = *(unsigned long long*)(hctr + C_BASE_PTS + 2);
   const uint64_t tiny_pts = *(unsigned long long*)(hctr + C_BASE_PTS + 4);
@@ -1683,7 +1717,10 @@ static int base_stage(const SmemArgs& sa, const BaseLists& L, const uint32_t* dc
     s1.cap = (int)L.cap;
     const uint32_t b1 = list_blocks(C_NBBASE, 1, 0);
     cudaEvent_t fork = nullptr, join = nullptr;
+    cudaStream_t aux = nullptr;
     if (b1) {
+      aux = helper();
+      if (!aux) return PKD_ECUDA;
       PKD_CUDA(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming));
       PKD_CUDA(cudaEventCreateWithFlags(&join, cudaEventDisableTiming));
       PKD_CUDA(cudaEventRecord(fork, q));
@@ -1800,7 +1837,7 @@ static int build_flat(TreeMem& t, const BuildJob& job, Scratch& sc) {
     counted = true;
   }
   auto none = [](cudaStream_t, int, uint32_t, uint32_t) { return PKD_OK; };
-  PKD_TRY(base_stage(sa, L, dctr, hctr, d, nsm, s, aux_stream(), bound, none));
+  PKD_TRY(base_stage(sa, L, dctr, hctr, d, nsm, s, helper_stream, bound, none));
   PKD_CUDA(cudaGetLastError());
   return PKD_OK;
 }
@@ -2084,7 +2121,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
       return mx ? std::min(b, mx) : b;
     };
     auto none = [](cudaStream_t, int, uint32_t, uint32_t) { return PKD_OK; };
-    PKD_TRY(base_stage(sa, L, dctr, hctr, d, nsm, s, aux_stream(), host_blocks, none));
+    PKD_TRY(base_stage(sa, L, dctr, hctr, d, nsm, s, helper_stream, host_blocks, none));
     PKD_CUDA(cudaGetLastError());
     return PKD_OK;
   };
@@ -2175,7 +2212,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
       ++nshape;
       return PKD_OK;
     };
-    if (e == PKD_OK) e = base_stage(sa, L, dctr, hctr, d, nsm, cs, aux_stream(), dev_blocks, record_shape);
+    if (e == PKD_OK) e = base_stage(sa, L, dctr, hctr, d, nsm, cs, capture_helper_stream, dev_blocks, record_shape);
     flow_capturing() = false;
     cudaGraph_t graph_h = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(cs, &graph_h);

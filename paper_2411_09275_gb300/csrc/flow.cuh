@@ -36,7 +36,8 @@ static __global__ void k_flow_cond(cudaGraphConditionalHandle h, const uint32_t*
 bool& flow_capturing();
 
 // A stream of the current device for graph level `level` (created on first
-// use; level 0 holds the top-level capture).
+// use; level 0 holds the top-level capture, -1 what it forks to).  Only
+// recording uses these streams, under flow_mutex().
 cudaStream_t flow_stream(int level);
 
 // Serialises captures: the level streams are shared by every host thread.

@@ -1,0 +1,98 @@
+"""Host threads that work on trees of their own, each on its own stream: what
+one thread's call does on the library's shared state (the streams and the lock
+of recorded builds, the kernels' shared-memory limits) never reaches another
+thread's tree.  Trees equal the oracle's after every call."""
+import threading
+
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2411_09275_gb300 import inputs as I
+from tests import treeutil as U
+from tests.gpuutil import ids_dev, oparams, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+def _together(*bodies):
+    """Run every body(stream) in a thread of its own; re-raise what one raised."""
+    import torch
+
+    torch.cuda.synchronize()
+    failed = []
+    start = threading.Barrier(len(bodies))
+
+    def run(body):
+        s = torch.cuda.Stream()
+        try:
+            with torch.cuda.stream(s):
+                start.wait(60)
+                body(s)
+                s.synchronize()
+        except BaseException as e:  # noqa: BLE001
+            failed.append(e)
+
+    threads = [threading.Thread(target=run, args=(b,)) for b in bodies]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join(300)
+    assert not any(th.is_alive() for th in threads)
+    if failed:
+        raise failed[0]
+
+
+def test_builds_that_record_beside_updates_of_another_tree():
+    # one thread builds trees of ever new sizes, so that each records its
+    # graph; the other's tree is rebuilt from the root by every update
+    # (alpha = 0), as one segment that runs on the direct build's second stream
+    import torch
+
+    from paper_2411_09275_gb300 import pkd
+
+    p = pkd.Params(d=3)
+    points = [I.uniform(9000 + 37 * i, 3, 9000 + i) for i in range(100)]
+    p0 = pkd.Params(d=3, alpha_num=0)
+    X = I.uniform(5000, 3, 3)
+    Q = np.concatenate([X[::100], I.uniform(200, 3, 4)])
+    o = O.OracleTree(X, None, oparams(p0))
+    batches, want = [], []
+    for i in range(100):
+        Y = I.uniform(50 + i, 3, 7000 + i)
+        yid = np.arange(5000 + 200 * i, 5000 + 200 * i + len(Y), dtype=np.uint32)
+        gone = np.concatenate([yid[::2], np.arange(40 * i, 40 * i + 20, dtype=np.uint32)])
+        batches.append((Y, yid, gone))
+        o.insert(Y, yid)
+        want.append(o.knn(Q, 5))
+        assert o.delete(gone) == len(gone)
+        want.append(o.knn(Q, 5))
+    builds, answers = [], []
+    dev_points = [to_dev(x) for x in points]
+    dev_batches = [(to_dev(Y), ids_dev(yid), ids_dev(gone)) for Y, yid, gone in batches]
+    gX, gQ = to_dev(X), to_dev(Q)
+    updated = []
+
+    def build(s):
+        for x in dev_points:
+            builds.append(pkd.Tree(x, None, p, s))
+
+    def update(s):
+        t = pkd.Tree(gX, None, p0, s)
+        updated.append(t)
+        for Y, yid, gone in dev_batches:
+            t.insert(Y, yid, s)
+            answers.append(t.knn(gQ, 5, s))
+            assert t.delete(gone, s) == gone.numel()
+            answers.append(t.knn(gQ, 5, s))
+
+    _together(build, update)
+    torch.cuda.synchronize()
+    for x, t in zip(points, builds):
+        U.assert_exports_equal(t.export(), O.OracleTree(x, None, oparams(p)).export())
+        t.close()
+    for (gi, gd), (wi, wd) in zip(answers, want):
+        assert np.array_equal(gd.cpu().numpy(), wd) and np.array_equal(gi.cpu().numpy().view(np.uint32), wi)
+    U.assert_exports_equal(updated[0].export(), o.export())
+    updated[0].close()
+    assert len(builds) == len(points) and len(answers) == len(want)
