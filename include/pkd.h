@@ -25,7 +25,13 @@
  *    host, a smaller one's are queued together.  Queries are asynchronous:
  *    their outputs are valid once `stream` has been synchronised.
  *  - A pkd_tree is not thread-safe: one call at a time per tree, except
- *    that queries on an unchanging tree may overlap.
+ *    that queries on an unchanging tree may overlap.  Threads may work on
+ *    trees of their own at once.  A call that records a build's graph (a tree
+ *    or forest with rounds whose sizes or buffers are new) must not coincide
+ *    with another thread's wait for the whole device (cudaDeviceSynchronize):
+ *    CUDA fails such a wait and ends the recording, and the build returns an
+ *    error.  Waits for streams and events are free of this, and so are this
+ *    library's own calls; with "graph_rounds" 0 nothing is recorded.
  *  - Return value 0 (PKD_OK) or one of the error codes below; device-side
  *    failures (a bound exceeded, a wait that ran out) are reported by the
  *    call that detects them, and leave the tree unusable: free it.

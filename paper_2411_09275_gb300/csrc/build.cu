@@ -1466,6 +1466,11 @@ std::mutex& flow_mutex() {
   return m;
 }
 
+cudaError_t device_wait() {
+  std::lock_guard<std::mutex> lk(flow_mutex());
+  return cudaDeviceSynchronize();
+}
+
 cudaStream_t flow_stream(int level) {
   static std::mutex mu;
   static std::map<std::pair<int, int>, cudaStream_t> streams;

@@ -269,6 +269,10 @@ struct BuildJob {
 };
 int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s);
 
+// Waits for the whole device, never while another thread records a graph
+// (CUDA forbids that: the wait fails and ends the recording).
+cudaError_t device_wait();
+
 // Builds whose rounds ran from one graph launch (since the library was loaded).
 int graph_builds();
 // ... of them, the builds that launched a graph recorded by an earlier build.

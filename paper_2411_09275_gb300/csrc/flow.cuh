@@ -74,6 +74,7 @@ inline int flow_cond_node(Flow& f, int w, cudaGraphConditionalNodeType type, cud
   PKD_CUDA(cudaGraphConditionalHandleCreate(h, g, 0, 0));
   PKD_LAUNCH(k_flow_cond<<<1, 1, 0, f.s>>>(*h, f.dctl + w));
   PKD_CUDA(cudaStreamGetCaptureInfo(f.s, &cs, nullptr, &g, &deps, nullptr, &nd));
+  if (cs != cudaStreamCaptureStatusActive) return PKD_EINTERNAL;  // ended meanwhile: deps are stale
   cudaGraphNodeParams np{};
   np.type = cudaGraphNodeTypeConditional;
   np.conditional.handle = *h;

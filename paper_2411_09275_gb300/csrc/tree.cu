@@ -452,7 +452,7 @@ void tree_touch(TreeMem& t, cudaStream_t s, bool noalloc) {
 
 void tree_wait_uses(TreeMem& t) {
   std::lock_guard<std::mutex> g(g_use_mu);
-  if (t.untracked) cudaDeviceSynchronize();
+  if (t.untracked) device_wait();
   for (auto& u : t.uses) {
     if (!t.untracked) cudaStreamWaitEvent(0, u.second, 0);
     cudaEventDestroy(u.second);
@@ -516,7 +516,7 @@ int download_tree(const TreeMem& t, HostTree& h, bool with_ids) {
   const uint64_t used = t.shared_cap + 2 * t.top;
   h.nodes.resize(used);
   h.ndim.resize(used);
-  PKD_CUDA(cudaDeviceSynchronize());
+  PKD_CUDA(device_wait());
   PKD_CUDA(cudaMemcpy(h.nodes.data(), t.nodes, used * sizeof(Node), cudaMemcpyDeviceToHost));
   PKD_CUDA(cudaMemcpy(h.ndim.data(), t.ndim, used, cudaMemcpyDeviceToHost));
   if (with_ids) {

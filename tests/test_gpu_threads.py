@@ -96,3 +96,36 @@ def test_builds_that_record_beside_updates_of_another_tree():
     U.assert_exports_equal(updated[0].export(), o.export())
     updated[0].close()
     assert len(builds) == len(points) and len(answers) == len(want)
+
+
+def test_builds_that_record_beside_exports_of_another_tree():
+    # an export waits for the whole device, which CUDA forbids while a stream
+    # is being recorded
+    from paper_2411_09275_gb300 import pkd
+
+    p = pkd.Params(d=2)
+    points = [I.uniform(30000 + 41 * i, 2, 600 + i) for i in range(80)]
+    X = I.uniform(20000, 2, 5)
+    t = pkd.Tree(to_dev(X), None, p)
+    dev_points = [to_dev(x) for x in points]
+    builds, exports, heights = [], [], []
+
+    def build(s):
+        for x in dev_points:
+            builds.append(pkd.Tree(x, None, p, s))
+
+    def export(s):
+        while len(builds) < len(points) and len(exports) < 5000:
+            exports.append(t.export())
+            heights.append(t.height)
+            del exports[1:-1]
+
+    _together(build, export)
+    want = O.OracleTree(X, None, oparams(p)).export()
+    assert len(builds) == len(points)
+    for e in exports:
+        U.assert_exports_equal(e, want)
+    for x, b in zip(points, builds):
+        U.assert_exports_equal(b.export(), O.OracleTree(x, None, oparams(p)).export())
+        b.close()
+    t.close()
