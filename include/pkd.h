@@ -308,6 +308,8 @@ const char* pkd_strerror(int code);
  *                default, sizes them by the points of those subtrees).  A
  *                list that overflows makes the update redo the flatten with
  *                room for every node of the tree, before any visible change.
+ *   "pause_rounds" testing: calls * 10000 + ms: that many rebuilds whose rounds
+ *                the host sequences sleep ms milliseconds before the first
  * Returns PKD_EINVAL for an unknown name or an out-of-range value. */
 int pkd_set_option(const char* name, int64_t value);
 

@@ -2110,6 +2110,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
 
   PKD_LAUNCH(k_ctl_init<<<1, 64, 0, s>>>(dctr, (uint32_t)nroots));
   auto host_rounds = [&]() {
+    test_pause(PAUSE_ROUNDS);
     PKD_TRY(classify(f));
     // the first round is certain when a segment is known to exceed one CTA;
     // the last read brings the base lists' lengths, for their exact grids
@@ -2137,7 +2138,7 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
     // { ... } ... IF(exact levels) { ... } ... }, then the base cases as
     // device-updatable kernel nodes whose grids k_base_shapes sets from the
     // lists' lengths (a node with an empty list is disabled).
-    std::lock_guard<std::mutex> lk(flow_mutex());
+    std::unique_lock<std::mutex> lk(flow_mutex());
     const auto rec0 = std::chrono::steady_clock::now();
     cudaStream_t cs = flow_stream(0);
     if (!cs) return PKD_ECUDA;
@@ -2186,7 +2187,10 @@ int run_build(TreeMem& t, const BuildJob& job, cudaStream_t s) {
     // positions are new), and recording, instantiating and destroying a graph
     // takes about 0.6 ms of host time, the host's reads of a rebuild's one or
     // two rounds 0.1: only a repeated one is recorded.
-    if (job.dsegs && !graph_seen(key)) return host_rounds();
+    if (job.dsegs && !graph_seen(key)) {
+      lk.unlock();  // the rounds wait for the device; other threads' builds do not wait for them
+      return host_rounds();
+    }
 
     int nshape = 0;
     cudaGraphNode_t shape_nodes[MAX_SHAPES] = {};

@@ -125,6 +125,12 @@ int cuda_err(cudaError_t e);
 // the next instead of being returned to the driver at every synchronisation.
 cudaMemPool_t mem_pool();
 
+// Testing: a thread that comes to one of these points sleeps there, as often and
+// as long as the option of that name says, so that a test can place another
+// thread's call in between.
+enum PausePoint { PAUSE_ROUNDS, PAUSE_POINTS };  // "pause_rounds": a rebuild whose rounds the host sequences
+void test_pause(PausePoint p);
+
 // Large blocks (tree arenas and node arrays) go through a small cache in
 // front of the pool: a freed block is kept with an event recorded on the
 // freeing stream and handed to the next request it fits (the requesting

@@ -10,6 +10,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "coords.cuh"
@@ -315,6 +316,19 @@ void big_free_zeroed(void* p, size_t zeroed, cudaStream_t s) {
 }
 
 void big_free(void* p, cudaStream_t s) { big_free_zeroed(p, 0, s); }
+
+// calls * PAUSE_CALL + milliseconds, counted down by the calls that sleep
+constexpr long long PAUSE_CALL = 10000, PAUSE_MAX = 1000 * PAUSE_CALL;
+static std::atomic<long long> g_pause[PAUSE_POINTS];
+
+void test_pause(PausePoint p) {
+  long long v = g_pause[p].load(std::memory_order_relaxed);
+  while (v >= PAUSE_CALL) {
+    if (!g_pause[p].compare_exchange_weak(v, v - PAUSE_CALL)) continue;
+    std::this_thread::sleep_for(std::chrono::milliseconds(v % PAUSE_CALL));
+    return;
+  }
+}
 
 static std::mutex g_pin_mu;
 static std::vector<void*> g_pin_free;
@@ -737,6 +751,9 @@ int pkd_set_option(const char* name, int64_t value) {
     if (value < -1) return PKD_EINVAL;
     knobs().fail_alloc_after = value;
     g_fail_budget.store(value);
+  } else if (n == "pause_rounds") {
+    if (value < 0 || value > PAUSE_MAX) return PKD_EINVAL;
+    g_pause[PAUSE_ROUNDS].store(value);
   } else if (n == "wait_cycles") {
     if (value < 0 || value > 4000000000000ll) return PKD_EINVAL;
     knobs().wait_cycles = value;

@@ -3,6 +3,7 @@ one thread's call does on the library's shared state (the streams and the lock
 of recorded builds, the kernels' shared-memory limits) never reaches another
 thread's tree.  Trees equal the oracle's after every call."""
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -10,7 +11,7 @@ import pytest
 import oracle as O
 from paper_2411_09275_gb300 import inputs as I
 from tests import treeutil as U
-from tests.gpuutil import ids_dev, oparams, to_dev
+from tests.gpuutil import ids_dev, knobs, oparams, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -129,3 +130,37 @@ def test_builds_that_record_beside_exports_of_another_tree():
         U.assert_exports_equal(b.export(), O.OracleTree(x, None, oparams(p)).export())
         b.close()
     t.close()
+
+
+def test_a_rebuild_that_waits_holds_up_no_other_build():
+    # the insert rebuilds its tree from the root (alpha = 0), more points than
+    # one CTA takes, and sleeps two seconds in front of the first round
+    from paper_2411_09275_gb300 import pkd
+
+    X, Y, Z = I.uniform(20000, 3, 11), I.uniform(100, 3, 12), I.uniform(40000, 3, 13)
+    p, p0 = pkd.Params(d=3), pkd.Params(d=3, alpha_num=0)
+    pkd.Tree(to_dev(Z), None, p).close()
+    t, o = pkd.Tree(to_dev(X), None, p0), O.OracleTree(X, None, oparams(p0))
+    gY, gZ, yid = to_dev(Y), to_dev(Z), np.arange(20000, 20100, dtype=np.uint32)
+    gyid = ids_dev(yid)
+    o.insert(Y, yid)
+    at, built = {}, []
+
+    def update(s):
+        at["start"] = time.monotonic()
+        t.insert(gY, gyid, s)
+        at["update"] = time.monotonic()
+
+    def build(s):
+        time.sleep(0.5)
+        built.append(pkd.Tree(gZ, None, p, s))
+        at["build"] = time.monotonic()
+
+    with knobs(pause_rounds=12000):
+        _together(update, build)
+    assert at["update"] - at["start"] >= 1.9  # the rebuild did sleep there
+    assert at["build"] < at["update"] - 0.5
+    U.assert_exports_equal(t.export(), o.export())
+    U.assert_exports_equal(built[0].export(), O.OracleTree(Z, None, oparams(p)).export())
+    t.close()
+    built[0].close()
