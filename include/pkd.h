@@ -310,6 +310,8 @@ const char* pkd_strerror(int code);
  *                room for every node of the tree, before any visible change.
  *   "pause_rounds" testing: calls * 10000 + ms: that many rebuilds whose rounds
  *                the host sequences sleep ms milliseconds before the first
+ *   "pause_smem" testing: the same in front of kernel launches with more shared
+ *                memory than the default limit
  * Returns PKD_EINVAL for an unknown name or an out-of-range value. */
 int pkd_set_option(const char* name, int64_t value);
 

@@ -456,21 +456,16 @@ __global__ void __launch_bounds__(WK_WARPS * 32, 4) k_smem_warp(SmemArgs a) {
 }
 
 // Launch of a shared-memory kernel with its dynamic shared memory.
-template <class K>
-static void launch_with_smem(K kern, int* set, uint32_t nblocks, int threads, size_t smb, cudaStream_t s,
-                             const SmemArgs& a) {
-  if (*set < (int)smb) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
-    *set = (int)smb;
-  }
+template <auto K>
+static void launch_with_smem(uint32_t nblocks, int threads, size_t smb, cudaStream_t s, const SmemArgs& a) {
+  allow_smem<K>(smb);
   if (nblocks == 0) return;
-  PKD_LAUNCH(kern<<<nblocks, threads, smb, s>>>(a));
+  PKD_LAUNCH(K<<<nblocks, threads, smb, s>>>(a));
 }
 
 template <int D>
 static void launch_smem_build(const SmemArgs& a, uint32_t nblocks, size_t smb, cudaStream_t s) {
-  static int set = 0;
-  launch_with_smem(k_smem_build<D>, &set, nblocks, SM_THREADS, smb, s, a);
+  launch_with_smem<k_smem_build<D>>(nblocks, SM_THREADS, smb, s, a);
 }
 
 static int smem_optin();
@@ -487,18 +482,15 @@ static void launch_smem_sorted(const SmemArgs& a, uint32_t nblocks, bool shared,
   if constexpr (D <= 5) {
     const size_t wide = sorted_layout(a.cap, D, SS_WIDE).total;
     if (!shared && wide <= (size_t)smem_optin()) {
-      static int set = 0;
-      launch_with_smem(k_smem_sorted<D, 1, SS_WIDE>, &set, nblocks, SS_WIDE * 32, wide, s, a);
+      launch_with_smem<k_smem_sorted<D, 1, SS_WIDE>>(nblocks, SS_WIDE * 32, wide, s, a);
       return;
     }
   }
-  static int set = 0;
-  launch_with_smem(k_smem_sorted<D, 1>, &set, nblocks, SS_NW * 32, sorted_layout(a.cap, D).total, s, a);
+  launch_with_smem<k_smem_sorted<D, 1, SS_NW>>(nblocks, SS_NW * 32, sorted_layout(a.cap, D).total, s, a);
 }
 template <int D>
 static void launch_smem_sorted2(const SmemArgs& a, uint32_t nblocks, size_t smb, cudaStream_t s) {
-  static int set = 0;
-  launch_with_smem(k_smem_sorted<D, 2>, &set, nblocks, SS_NW * 32, smb, s, a);
+  launch_with_smem<k_smem_sorted<D, 2, SS_NW>>(nblocks, SS_NW * 32, smb, s, a);
 }
 
 // The helper stream of this host thread for direct launches, on the current
@@ -571,22 +563,12 @@ static int sorted_cap_two_per_sm(int d) {
 
 template <int D>
 static void launch_smem_skel(const SmemArgs& a, uint32_t nblocks, size_t smb, cudaStream_t s) {
-  static int set = 0;
-  if (set < (int)smb) {
-    cudaFuncSetAttribute(k_smem_skel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
-    set = (int)smb;
-  }
-  PKD_LAUNCH(k_smem_skel<D><<<nblocks, SM_THREADS, smb, s>>>(a));
+  launch_with_smem<k_smem_skel<D>>(nblocks, SM_THREADS, smb, s, a);
 }
 
 template <int D>
 static void launch_smem_warp(const SmemArgs& a, uint32_t nblocks, size_t smb, cudaStream_t s) {
-  static int set = 0;
-  if (set < (int)smb) {
-    cudaFuncSetAttribute(k_smem_warp<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
-    set = (int)smb;
-  }
-  PKD_LAUNCH(k_smem_warp<D><<<nblocks, WK_WARPS * 32, smb, s>>>(a));
+  launch_with_smem<k_smem_warp<D>>(nblocks, WK_WARPS * 32, smb, s, a);
 }
 
 // ---------------------------------------------------------------------------

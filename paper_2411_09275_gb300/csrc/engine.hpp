@@ -5,7 +5,9 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <functional>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -112,6 +114,36 @@ void count_launch();
 // synchronises the stream and prints the wall time since the previous mark.
 void trace_mark(cudaStream_t s, const char* what);
 
+// Testing: a thread that comes to one of these points sleeps there, as often and
+// as long as the option of that name says, so that a test can place another
+// thread's call in between.
+enum PausePoint {
+  PAUSE_ROUNDS,  // "pause_rounds": a rebuild whose rounds the host sequences, in front of the first
+  PAUSE_SMEM,    // "pause_smem": a kernel with raised shared memory, in front of its launch
+  PAUSE_POINTS
+};
+void test_pause(PausePoint p);
+
+// Lets kernel K be launched with `bytes` of dynamic shared memory on the
+// current device.  The limit is the process's, so it is only ever raised, under
+// a lock: set to what each launch needs it could be lowered by another thread
+// between this thread's setting and its launch, which then fails.
+template <auto K>
+void allow_smem(size_t bytes) {
+  constexpr int DEVICES = 64;
+  static std::atomic<int> limit[DEVICES];
+  static std::mutex mu;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (limit[dev % DEVICES].load(std::memory_order_acquire) < (int)bytes) {
+    std::lock_guard<std::mutex> g(mu);
+    if (limit[dev % DEVICES].load(std::memory_order_relaxed) < (int)bytes &&
+        cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess)
+      limit[dev % DEVICES].store((int)bytes, std::memory_order_release);
+  }
+  test_pause(PAUSE_SMEM);
+}
+
 // Error helpers.
 int cuda_err(cudaError_t e);
 #define PKD_CUDA(x)                          \
@@ -124,12 +156,6 @@ int cuda_err(cudaError_t e);
 // release threshold is unlimited: memory freed by one build stays mapped for
 // the next instead of being returned to the driver at every synchronisation.
 cudaMemPool_t mem_pool();
-
-// Testing: a thread that comes to one of these points sleeps there, as often and
-// as long as the option of that name says, so that a test can place another
-// thread's call in between.
-enum PausePoint { PAUSE_ROUNDS, PAUSE_POINTS };  // "pause_rounds": a rebuild whose rounds the host sequences
-void test_pause(PausePoint p);
 
 // Large blocks (tree arenas and node arrays) go through a small cache in
 // front of the pool: a freed block is kept with an event recorded on the

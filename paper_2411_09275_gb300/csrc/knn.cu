@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(QTHREADS) k_knn(QueryArgs a) {
 template <int D, int G, int S, bool DEEP>
 static void launch_knn_as(const QueryArgs& a, cudaStream_t s) {
   constexpr int GPB = QTHREADS / G;
-  launch_query(k_knn<D, G, S, DEEP>, (a.nq + GPB - 1) / GPB, DEEP ? 0 : (size_t)GPB * a.cap * (12 + 4 * D), s, a);
+  launch_query<k_knn<D, G, S, DEEP>>((a.nq + GPB - 1) / GPB, DEEP ? 0 : (size_t)GPB * a.cap * (12 + 4 * D), s, a);
 }
 template <int D, bool DEEP>
 static void launch_knn_(const QueryArgs& a, cudaStream_t s) {

@@ -415,8 +415,8 @@ static void launch_report(const QueryArgs& a, const uint64_t* offsets, uint32_t*
   const uint64_t g = (a.nq + WPB - 1) / WPB;
   KTimer kt;
   ktimer_begin(kt, "range_report", a.nq, s);
-  if (a.deep) launch_query(k_range_report<D, true>, g, 0, s, a, offsets, ids, ids_cap);
-  else launch_query(k_range_report<D, false>, g, (size_t)WPB * a.cap * sizeof(uint2), s, a, offsets, ids,
+  if (a.deep) launch_query<k_range_report<D, true>>(g, 0, s, a, offsets, ids, ids_cap);
+  else launch_query<k_range_report<D, false>>(g, (size_t)WPB * a.cap * sizeof(uint2), s, a, offsets, ids,
                     ids_cap);
   ktimer_end(kt);
 }
@@ -427,8 +427,8 @@ static void launch_rc(const QueryArgs& a, cudaStream_t s) {
   const uint64_t g = (a.nq + WPB - 1) / WPB;
   KTimer kt;
   ktimer_begin(kt, "range_count", a.nq, s);
-  if (a.deep) launch_query(k_range_count<D, true>, g, 0, s, a);
-  else launch_query(k_range_count<D, false>, g, (size_t)WPB * a.cap * sizeof(uint2), s, a);
+  if (a.deep) launch_query<k_range_count<D, true>>(g, 0, s, a);
+  else launch_query<k_range_count<D, false>>(g, (size_t)WPB * a.cap * sizeof(uint2), s, a);
   ktimer_end(kt);
 }
 

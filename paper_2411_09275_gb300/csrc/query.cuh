@@ -114,10 +114,10 @@ int for_query_chunks(const TreeMem& t, const QueryArgs& a, int words, int extra,
 
 // Launches a kernel with `smb` bytes of dynamic shared memory (above 48 KiB
 // only for trees of a height far above the usual).
-template <class K, class... A>
-void launch_query(K kern, uint64_t blocks, size_t smb, cudaStream_t s, A... args) {
-  if (smb > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
-  PKD_LAUNCH((kern<<<(unsigned)blocks, QTHREADS, smb, s>>>(args...)));
+template <auto K, class... A>
+void launch_query(uint64_t blocks, size_t smb, cudaStream_t s, A... args) {
+  if (smb > 48 * 1024) allow_smem<K>(smb);
+  PKD_LAUNCH((K<<<(unsigned)blocks, QTHREADS, smb, s>>>(args...)));
 }
 
 }  // namespace pkd

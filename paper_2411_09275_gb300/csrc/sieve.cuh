@@ -563,11 +563,7 @@ template <int D>
 static void launch_scatter_tiles(const RoundArgs& r, uint32_t tiles, uint64_t pts, const char* fam,
                                  cudaStream_t s) {
   const size_t sm = scatter_smem(r.HN, r.NB, D, r.TILE);
-  static bool set = false;
-  if (!set) {
-    cudaFuncSetAttribute(k_scatter<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    set = true;
-  }
+  allow_smem<k_scatter<D>>(200 * 1024);
   const uint32_t grid = r.ntiles ? std::min<uint32_t>(tiles, (uint32_t)sm_count() * 2) : tiles;
   KTimer kt;
   ktimer_begin(kt, fam, pts, s);

@@ -609,11 +609,7 @@ static void launch_count(const RoundArgs& r, uint32_t tiles, uint64_t pts, const
     launch_count_tiles<D>(r, tiles, pts, fam, s);
     return;
   }
-  static size_t set = 0;
-  if (set < smb) {
-    cudaFuncSetAttribute(k_count_stream<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
-    set = smb;
-  }
+  allow_smem<k_count_stream<D>>(smb);
   const uint32_t grid = std::min<uint32_t>(tiles, (uint32_t)stream_sm_count() * 2);
   KTimer kt;
   ktimer_begin(kt, fam, pts, s);
@@ -628,11 +624,7 @@ static void launch_scatter(const RoundArgs& r, uint32_t tiles, uint64_t pts, con
     launch_scatter_tiles<D>(r, tiles, pts, fam, s);
     return;
   }
-  static size_t set = 0;
-  if (set < smb) {
-    cudaFuncSetAttribute(k_scatter_stream<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
-    set = smb;
-  }
+  allow_smem<k_scatter_stream<D>>(smb);
   const uint32_t grid = std::min<uint32_t>(tiles, (uint32_t)stream_sm_count() * 2);
   KTimer kt;
   ktimer_begin(kt, fam, pts, s);

@@ -625,10 +625,7 @@ template <int D>
 static void launch_route(const RouteArgs& a, const Seg* mid, const uint32_t* d_nmid, uint32_t nmid, const Seg* small,
                          const uint32_t* d_nsmall, uint32_t nsmall, cudaStream_t s) {
   const size_t per = skel_bytes(a.HN, a.NB), warps = per * WARP_TEAMS;
-  if (warps > 48 * 1024) {
-    cudaFuncSetAttribute(k_route<D, MID_TEAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)per);
-    cudaFuncSetAttribute(k_route<D, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)warps);
-  }
+  if (warps > 48 * 1024) allow_smem<k_route<D, 32>>(warps);  // (a CTA's one skeleton: 37 KB at lambda = 10)
   if (nmid) PKD_LAUNCH((k_route<D, MID_TEAM><<<nmid, MID_TEAM, per, s>>>(a, mid, d_nmid)));
   if (nsmall) {
     // persistent warps: each remembers the largest sizes that it has sent

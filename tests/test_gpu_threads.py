@@ -164,3 +164,62 @@ def test_a_rebuild_that_waits_holds_up_no_other_build():
     U.assert_exports_equal(built[0].export(), O.OracleTree(Z, None, oparams(p)).export())
     t.close()
     built[0].close()
+
+
+def test_searches_and_updates_with_different_shared_memory():
+    # stacks of trees of heights about 75 and 115, and skeletons of 9 and 10
+    # levels, take more than 48 KB of shared memory, each another amount
+    from paper_2411_09275_gb300 import pkd
+
+    def chain(batches):  # alpha = 1/2, always past the last point: one path grows
+        p = pkd.Params(d=3, phi=2, lam=2, sigma_log2=0, sigma_os=1, alpha_num=1, alpha_den=2)
+        X = np.zeros((8, 3), np.int32)
+        X[:, 0] = np.arange(8) * 7
+        t, o = pkd.Tree(to_dev(X), None, p), O.OracleTree(X, None, oparams(p))
+        for r in range(batches):
+            Y = np.zeros((3, 3), np.int32)
+            Y[:, 0] = 100 + 10 * r + np.array([3, 1, 2])
+            yid = np.arange(8 + 3 * r, 11 + 3 * r, dtype=np.uint32)
+            t.insert(to_dev(Y), ids_dev(yid))
+            o.insert(Y, yid)
+        return t, o
+
+    Q = I.uniform(9000, 3, 21)
+    Q[:, 0] %= 700
+    Q[:, 1:] %= 50
+    gQ = to_dev(Q)
+    pairs = [chain(36), chain(56)]
+    assert 66 <= pairs[0][0].height < 85 and 100 < pairs[1][0].height < 126
+    X = I.uniform(3000, 3, 22)
+    Y, yid = I.uniform(20, 3, 23), np.arange(3000, 3020, dtype=np.uint32)
+    gY, gyid = to_dev(Y), ids_dev(yid)
+    wide = []
+    for lam in (9, 10):
+        p = pkd.Params(d=3, lam=lam, phi=8)
+        wide.append((pkd.Tree(to_dev(X), None, p), O.OracleTree(X, None, oparams(p))))
+    answers = []
+
+    def search(k, wait):
+        def body(s):
+            time.sleep(wait)
+            answers.append((k, pairs[k][0].knn(gQ, 4, s)))
+        return body
+
+    def update(k, wait):
+        def body(s):
+            time.sleep(wait)
+            wide[k][0].insert(gY, gyid, s)
+        return body
+
+    # the larger one sleeps between the limit and its launch, the other runs meanwhile
+    for small, large in ((search(0, 0.3), search(1, 0)), (update(0, 0.3), update(1, 0))):
+        with knobs(pause_smem=10700):
+            _together(small, large)
+    for k, (gi, gd) in answers:
+        wi, wd = pairs[k][1].knn(Q, 4)
+        assert np.array_equal(gd.cpu().numpy(), wd) and np.array_equal(gi.cpu().numpy().view(np.uint32), wi)
+    for t, o in wide:
+        o.insert(Y, yid)
+        U.assert_exports_equal(t.export(), o.export())
+    for t, o in pairs + wide:
+        t.close()
