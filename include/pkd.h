@@ -312,6 +312,8 @@ const char* pkd_strerror(int code);
  *                the host sequences sleep ms milliseconds before the first
  *   "pause_smem" testing: the same in front of kernel launches with more shared
  *                memory than the default limit
+ *   "pause_query" testing: the same for queries, between their check and their
+ *                search
  * Returns PKD_EINVAL for an unknown name or an out-of-range value. */
 int pkd_set_option(const char* name, int64_t value);
 

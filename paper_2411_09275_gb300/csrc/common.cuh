@@ -61,14 +61,16 @@ enum DevErr : int {
   DERR_STATE = 5,     // an internal consistency check failed
 };
 
+constexpr int QUERY_SLOTS = 16;
+
 struct DevStatus {
   int err;
   int detail;
   uint32_t max_depth;
   int idflags;  // id-table flags of the running call (IDF_* in ids.cuh)
-  // numbers of the last query calls whose coordinates were out of range, by
-  // number % 16 (queries on an unchanging tree may overlap)
-  unsigned long long refused[16];
+  // query calls whose coordinates were out of range, by number, each in the slot
+  // that its call holds (queries on an unchanging tree may overlap)
+  unsigned long long refused[QUERY_SLOTS];
 };
 
 __device__ __forceinline__ void set_error(DevStatus* st, int code, int detail) {

@@ -59,6 +59,7 @@ struct TreeMem {
   bool scratch_dirty = false;       // a delete has set marks it has not cleared yet
   DevStatus* st = nullptr;          // device status word
   DevStatus* st_host = nullptr;     // pinned mirror
+  uint32_t query_slots = 0;         // slots of st->refused that a running call holds (atomic)
   IdTable ids;                      // id -> coordinates of the stored points
   int32_t* bbox = nullptr;          // stored bounding boxes (boxes.cu), node_cap * 2d
   uint64_t bbox_cap = 0;            // node slots bbox covers
@@ -120,6 +121,7 @@ void trace_mark(cudaStream_t s, const char* what);
 enum PausePoint {
   PAUSE_ROUNDS,  // "pause_rounds": a rebuild whose rounds the host sequences, in front of the first
   PAUSE_SMEM,    // "pause_smem": a kernel with raised shared memory, in front of its launch
+  PAUSE_QUERY,   // "pause_query": a query, between its check and its search
   PAUSE_POINTS
 };
 void test_pause(PausePoint p);

@@ -300,6 +300,7 @@ int pkd::knn_on(TreeMem& t, uint32_t root, const int32_t* queries, uint64_t q, i
   PKD_TRY_(check.begin(queries, q * (uint64_t)t.p.d, nullptr, 0));
   QueryArgs a{};
   a.call = check.call;
+  a.slot = check.slot;
   a.nodes = t.nodes;
   a.ndim = t.ndim;
   a.A = t.A;

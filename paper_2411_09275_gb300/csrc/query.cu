@@ -354,14 +354,14 @@ __global__ void k_scan64_apply(QueryArgs a, const uint64_t* in, uint64_t n, cons
 }
 
 __global__ void k_query_check(const int32_t* c1, uint64_t n1, const int32_t* c2, uint64_t n2, DevStatus* st,
-                              unsigned long long call, QueryHost* h) {
+                              unsigned long long call, int slot, QueryHost* h) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     h->err = st->err;
     h->detail = st->detail;
   }
   const unsigned b = coord_bits(c1, n1) | (c2 ? coord_bits(c2, n2) : 0);
   if (__any_sync(0xffffffffu, (b >> 30) != 0) && (threadIdx.x & 31) == 0) {
-    *(volatile unsigned long long*)&st->refused[call % 16] = call;
+    if (slot >= 0) *(volatile unsigned long long*)&st->refused[slot] = call;
     *(volatile int*)&h->bad = 1;
   }
 }
@@ -381,9 +381,17 @@ int QueryCheck::begin(const int32_t* c1, uint64_t n1, const int32_t* c2, uint64_
   if (!h) return PKD_ENOMEM;
   h->bad = 0;
   call = ++calls;
+  uint32_t held = __atomic_load_n(&t.query_slots, __ATOMIC_RELAXED);
+  while (~held & ((1u << QUERY_SLOTS) - 1u)) {
+    const int k = __builtin_ctz(~held);
+    if (__atomic_compare_exchange_n(&t.query_slots, &held, held | 1u << k, true, __ATOMIC_ACQUIRE, __ATOMIC_RELAXED)) {
+      slot = k;
+      break;
+    }
+  }
   KTimer kt;
   ktimer_begin(kt, "validate", n1 + (c2 ? n2 : 0), s);
-  PKD_LAUNCH(k_query_check<<<coord_blocks(n1), 256, 0, s>>>(c1, n1, c2, n2, t.st, call, (QueryHost*)h));
+  PKD_LAUNCH(k_query_check<<<coord_blocks(n1), 256, 0, s>>>(c1, n1, c2, n2, t.st, call, slot, (QueryHost*)h));
   ktimer_end(kt);
   if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess || cudaEventRecord(ev, s) != cudaSuccess) {
     cudaGetLastError();
@@ -391,19 +399,35 @@ int QueryCheck::begin(const int32_t* c1, uint64_t n1, const int32_t* c2, uint64_
     if (ev) cudaEventDestroy(ev);
     ev = nullptr;
   }
+  test_pause(PAUSE_QUERY);
+  if (slot < 0) {
+    call = 0;
+    return verdict();
+  }
   return PKD_OK;
 }
 
-int QueryCheck::end() {
+int QueryCheck::verdict() {
   if (ev) PKD_CUDA(cudaEventSynchronize(ev));
   if (h->bad) return PKD_EINVAL;
   return status_code(h->err, h->detail);
+}
+
+int QueryCheck::end() {
+  const int e = verdict();
+  if (slot >= 0 && h->bad) PKD_CUDA(cudaStreamSynchronize(s));  // the search has read its slot
+  ended = true;
+  return e;
 }
 
 QueryCheck::~QueryCheck() {
   if (ev) {
     cudaEventSynchronize(ev);  // the check writes to the block until then
     cudaEventDestroy(ev);
+  }
+  if (slot >= 0) {
+    if (!ended) cudaStreamSynchronize(s);
+    __atomic_fetch_and(&t.query_slots, ~(1u << slot), __ATOMIC_RELEASE);
   }
   if (h) pinned_put((void*)h);
 }
@@ -442,6 +466,7 @@ namespace {
 QueryArgs range_args(const TreeMem& t, const QueryCheck& check, const int32_t* lo, const int32_t* hi, uint64_t q) {
   QueryArgs a{};
   a.call = check.call;
+  a.slot = check.slot;
   a.nodes = t.nodes;
   a.ndim = t.ndim;
   a.A = t.A;

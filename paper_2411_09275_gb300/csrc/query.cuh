@@ -27,6 +27,7 @@ struct QueryArgs {
   DevStatus* st;
   const int32_t* box;  // stored bounding boxes (node slot * 2d), or null
   unsigned long long call;  // the search does nothing when this call was refused (0: checked before)
+  int slot;                 // where its refusal stands
   int cap;             // stack entries per query
   bool given_offsets;  // report: the offsets are the caller's (no verdict on the tree when they do not fit)
   uint32_t* deep;      // deep trees: the queries' stacks, one after another
@@ -38,6 +39,11 @@ struct QueryArgs {
 // for the check alone, so it costs the search one kernel instead of a round
 // trip to the host (a fill, a kernel, two copies and two waits before: 45 us
 // in front of the search, now about 5).
+// The refusal is the call's number in a slot of the status block that no other
+// call on the tree holds until this one returns, and a refused call returns
+// after its search.  (An accepted call's search may still run by then: it only
+// looks for its own number.)  With every slot taken the host waits for the check
+// before the search is queued.
 struct QueryHost {  // written by the check into pinned memory
   int err, detail, bad;
 };
@@ -50,16 +56,19 @@ class QueryCheck {
   int begin(const int32_t* c1, uint64_t n1, const int32_t* c2, uint64_t n2);
   int end();  // waits for the check: PKD_OK, PKD_EINVAL or the tree's error
   unsigned long long call = 0;
+  int slot = -1;
 
  private:
+  int verdict();
   TreeMem& t;
   cudaStream_t s;
+  bool ended = false;
   volatile QueryHost* h = nullptr;
   cudaEvent_t ev = nullptr;
 };
 // In the searches: was the call refused?  (The same answer in all lanes.)
 __device__ __forceinline__ bool query_refused(const QueryArgs& a) {
-  const bool no = a.call && (pkd_failed(a.st) || *(volatile const unsigned long long*)&a.st->refused[a.call % 16] == a.call);
+  const bool no = a.call && (pkd_failed(a.st) || *(volatile const unsigned long long*)&a.st->refused[a.slot] == a.call);
   return __any_sync(0xffffffffu, no);
 }
 

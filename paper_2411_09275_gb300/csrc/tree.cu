@@ -751,9 +751,9 @@ int pkd_set_option(const char* name, int64_t value) {
     if (value < -1) return PKD_EINVAL;
     knobs().fail_alloc_after = value;
     g_fail_budget.store(value);
-  } else if (n == "pause_rounds" || n == "pause_smem") {
+  } else if (n == "pause_rounds" || n == "pause_smem" || n == "pause_query") {
     if (value < 0 || value > PAUSE_MAX) return PKD_EINVAL;
-    g_pause[n == "pause_rounds" ? PAUSE_ROUNDS : PAUSE_SMEM].store(value);
+    g_pause[n == "pause_rounds" ? PAUSE_ROUNDS : (n == "pause_smem" ? PAUSE_SMEM : PAUSE_QUERY)].store(value);
   } else if (n == "wait_cycles") {
     if (value < 0 || value > 4000000000000ll) return PKD_EINVAL;
     knobs().wait_cycles = value;

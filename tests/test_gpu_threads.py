@@ -223,3 +223,72 @@ def test_searches_and_updates_with_different_shared_memory():
         U.assert_exports_equal(t.export(), o.export())
     for t, o in pairs + wide:
         t.close()
+
+
+def _asker(pkd, t, q, outs, k=5):
+    """A body that asks for k neighbours of q on t, its outputs marked first."""
+    import torch
+
+    def body(s):
+        n = q.shape[0]
+        oi = torch.full((n, k), -7, dtype=torch.int32, device="cuda")
+        od = torch.full((n, k), -7, dtype=torch.int64, device="cuda")
+        code = pkd.PKD_OK
+        try:
+            pkd.pkd_knn(t._h, q, k, oi, od, stream=s)
+        except pkd.PkdError as e:
+            code = e.code
+        s.synchronize()
+        outs.append((code, oi, od))
+
+    return body
+
+
+def test_a_refusal_stands_until_its_search_has_run():
+    # a refused call sleeps between its check and its search while 40 others
+    # are refused on the same tree
+    from paper_2411_09275_gb300 import pkd
+
+    t = pkd.Tree(to_dev(I.uniform(5000, 3, 31)), None, pkd.Params(d=3))
+    bad = to_dev(np.full((64, 3), 1 << 30, np.int32))
+    slow, others = [], []
+
+    def refused(s):
+        time.sleep(0.3)
+        for _ in range(40):
+            _asker(pkd, t, bad, others)(s)
+
+    with knobs(pause_query=11500):
+        _together(_asker(pkd, t, bad, slow), refused)
+    assert len(slow) == 1 and len(others) == 40
+    for code, oi, od in slow + others:
+        assert code == pkd.PKD_EINVAL
+        assert (oi == -7).all().item() and (od == -7).all().item()
+    t.close()
+
+
+@pytest.mark.parametrize("threads", [2, 16, 17, 40])
+def test_queries_in_flight_at_once(threads):
+    # every call sleeps between its check and its search, so that all are in
+    # flight together: more than there are slots for refusals, too
+    from paper_2411_09275_gb300 import pkd
+
+    X, Q = I.uniform(5000, 3, 41), I.uniform(64, 3, 42)
+    p = pkd.Params(d=3)
+    t, o = pkd.Tree(to_dev(X), None, p), O.OracleTree(X, None, oparams(p))
+    good = to_dev(Q)
+    bad = to_dev(np.full((64, 3), 1 << 30, np.int32))
+    wi, wd = o.knn(Q, 5)
+    served, refused = [], []
+    for _ in range(2):  # the slots are free again
+        with knobs(pause_query=threads * 10000 + 300):
+            _together(*[_asker(pkd, t, bad if i % 3 == 0 else good, refused if i % 3 == 0 else served)
+                        for i in range(threads)])
+    assert len(served) + len(refused) == 2 * threads
+    for code, oi, od in refused:
+        assert code == pkd.PKD_EINVAL
+        assert (oi == -7).all().item() and (od == -7).all().item()
+    for code, oi, od in served:
+        assert code == pkd.PKD_OK
+        assert np.array_equal(od.cpu().numpy(), wd) and np.array_equal(oi.cpu().numpy().view(np.uint32), wi)
+    t.close()
