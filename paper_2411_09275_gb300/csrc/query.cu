@@ -366,17 +366,18 @@ __global__ void k_query_check(const int32_t* c1, uint64_t n1, const int32_t* c2,
   }
 }
 
-int QueryCheck::begin(const int32_t* c1, uint64_t n1, const int32_t* c2, uint64_t n2) {
-  static std::atomic<unsigned long long> calls{0};
-  // A capturing stream is refused before anything is recorded on it, as the
-  // wait below would be: a graph must not keep the pinned block.
+int refuse_capture(cudaStream_t s) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   PKD_CUDA(cudaStreamIsCapturing(s, &cap));
-  if (cap != cudaStreamCaptureStatusNone) {
-    const cudaError_t e = cudaStreamSynchronize(s);  // ends the capture with an error
-    cudaGetLastError();
-    return e != cudaSuccess ? cuda_err(e) : PKD_ECUDA;
-  }
+  if (cap == cudaStreamCaptureStatusNone) return PKD_OK;
+  const cudaError_t e = cudaStreamSynchronize(s);  // ends the capture with an error
+  cudaGetLastError();
+  return e != cudaSuccess ? cuda_err(e) : PKD_ECUDA;
+}
+
+int QueryCheck::begin(const int32_t* c1, uint64_t n1, const int32_t* c2, uint64_t n2) {
+  static std::atomic<unsigned long long> calls{0};
+  PKD_TRY_(refuse_capture(s));
   h = (volatile QueryHost*)pinned_get();
   if (!h) return PKD_ENOMEM;
   h->bad = 0;

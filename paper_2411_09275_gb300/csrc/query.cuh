@@ -66,6 +66,11 @@ class QueryCheck {
   volatile QueryHost* h = nullptr;
   cudaEvent_t ev = nullptr;
 };
+// PKD_OK, or the error for a stream that is being captured: before anything is
+// recorded on it, as a call that waits for the stream could not return anything
+// else (and a graph must not keep the call's pinned blocks).
+int refuse_capture(cudaStream_t s);
+
 // In the searches: was the call refused?  (The same answer in all lanes.)
 __device__ __forceinline__ bool query_refused(const QueryArgs& a) {
   const bool no = a.call && (pkd_failed(a.st) || *(volatile const unsigned long long*)&a.st->refused[a.slot] == a.call);

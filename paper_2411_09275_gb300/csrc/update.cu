@@ -1160,6 +1160,7 @@ int pkd_batch_delete(pkd_tree* tc, const uint32_t* ids, uint64_t m, uint64_t* n_
   TreeMem& t = tc->m;
   if (m >= (1ull << 31)) return PKD_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
+  PKD_TRY_(refuse_capture(s));
   TreeTouch touch{&t, s};
   // ids -> coordinates: every LIVE id of the batch is taken once (repeats and
   // unknown or deleted ids are skipped) and staged for the sieve
