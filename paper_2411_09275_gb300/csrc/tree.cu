@@ -231,14 +231,20 @@ static void big_flush_locked() {
 static std::atomic<unsigned long long> g_allocs{0};
 static std::atomic<long long> g_fail_budget{-1};
 
-cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
-  *p = nullptr;
+// Whether fault injection lets one more allocation pass (counted).
+static bool count_alloc() {
   long long b = g_fail_budget.load();
-  while (b >= 0) {  // fault injection armed
-    if (b == 0) return cudaErrorMemoryAllocation;
+  while (b >= 0) {  // armed
+    if (b == 0) return false;
     if (g_fail_budget.compare_exchange_weak(b, b - 1)) break;
   }
   g_allocs.fetch_add(1, std::memory_order_relaxed);
+  return true;
+}
+
+cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
+  *p = nullptr;
+  if (!count_alloc()) return cudaErrorMemoryAllocation;
   return cudaMallocFromPoolAsync(p, bytes, mem_pool(), s);
 }
 
@@ -338,7 +344,7 @@ void* pinned_get() {
   if (g_pin_free.empty()) {
     constexpr size_t CHUNK = 256;  // blocks per chunk
     char* c = nullptr;
-    g_allocs.fetch_add(1, std::memory_order_relaxed);
+    if (!count_alloc()) return nullptr;
     if (cudaMallocHost((void**)&c, CHUNK * PINNED_BLOCK) != cudaSuccess) {
       cudaGetLastError();
       return nullptr;

@@ -1163,7 +1163,10 @@ int pkd_batch_delete(pkd_tree* tc, const uint32_t* ids, uint64_t m, uint64_t* n_
   PKD_TRY_(refuse_capture(s));
   TreeTouch touch{&t, s};
   // ids -> coordinates: every LIVE id of the batch is taken once (repeats and
-  // unknown or deleted ids are skipped) and staged for the sieve
+  // unknown or deleted ids are skipped) and staged for the sieve; whatever
+  // refuses the call after that gives them back
+  PinnedBlock hb;
+  if (!hb.p) return PKD_ENOMEM;
   Scratch sc{s, {}};
   const int d = t.p.d;
   int32_t* wc;
@@ -1176,21 +1179,20 @@ int pkd_batch_delete(pkd_tree* tc, const uint32_t* ids, uint64_t m, uint64_t* n_
   PKD_TRY(dev_fill(cnt, 0, 4, s));
   Pts W{wc, wid, m};
   ids_take(t, ids, m, W, wslots, cnt, s);
-  PinnedBlock hb;
-  if (!hb.p) return PKD_ENOMEM;
   PKD_CUDA(cudaMemcpyAsync(hb.p, cnt, 4, cudaMemcpyDeviceToHost, s));
   int fl = 0;
   PKD_TRY(read_idflags(t, s, &fl));  // synchronises s
-  PKD_TRY(status_code(t.st_host->err, t.st_host->detail));
+  int e = status_code(t.st_host->err, t.st_host->detail);
   const uint32_t taken = *(const uint32_t*)hb.p;
-  if (fl) {
+  if (e == PKD_OK && fl) e = PKD_EINTERNAL;
+  if (e != PKD_OK) {
     ids_restore(t, wslots, taken, s);
-    return PKD_EINTERNAL;
+    return e;
   }
   stat_items("delete_gather", taken);
   if (taken == 0) return PKD_OK;
   uint64_t removed = 0;
-  int e = run_update(t, nullptr, nullptr, &W, taken, false, &removed, nullptr, s);
+  e = run_update(t, nullptr, nullptr, &W, taken, false, &removed, nullptr, s);
   if (e == PKD_OK && removed != taken) {
     fprintf(stderr, "pkd: delete removed %llu points for %u live ids\n", (unsigned long long)removed, taken);
     e = PKD_EINTERNAL;

@@ -1,6 +1,10 @@
 """Calls that are refused leave nothing behind: on a stream that is being captured
-nothing is launched or allocated."""
+nothing is launched or allocated, and a delete that finds no memory for its
+counters (the library's pinned blocks used up) gives the ids it took back."""
 import ctypes as C
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -48,3 +52,42 @@ def test_calls_on_a_capturing_stream_record_nothing():
     assert t.delete(ids, s) == o.delete(gone) == len(gone)
     U.assert_exports_equal(t.export(), o.export())
     t.close()
+
+
+_FRESH = r"""
+import sys
+import numpy as np
+sys.path.insert(0, sys.argv[1])
+import oracle as O
+from paper_2411_09275_gb300 import inputs as I, pkd
+from tests import treeutil as U
+from tests.gpuutil import ids_dev, knobs, oparams, to_dev
+
+# each of 256 trees keeps one pinned block, which is what the first allocation
+# of them holds: the delete's own is a new allocation
+X = I.uniform(3000, 3, 5)
+p = pkd.Params(d=3)
+gX = to_dev(X)
+trees = [pkd.Tree(gX, None, p) for _ in range(256)]
+t, o = trees[0], O.OracleTree(X, None, oparams(p))
+gone = np.arange(0, 3000, 3, dtype=np.uint32)
+before, fails = t.export(), 0
+for k in range(200):
+    try:
+        with knobs(fail_alloc_after=k):
+            n = t.delete(ids_dev(gone))
+        break
+    except pkd.PkdError as e:
+        assert e.code == pkd.PKD_ENOMEM, e.code
+        fails += 1
+        U.assert_exports_equal(t.export(), before)
+assert n == o.delete(gone) == len(gone), n
+U.assert_exports_equal(t.export(), o.export())
+print("RESULT ok", fails)
+"""
+
+
+def test_a_delete_without_memory_for_its_counters_keeps_the_ids():
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _FRESH, root], capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0 and "RESULT ok" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
