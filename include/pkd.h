@@ -21,8 +21,8 @@
  *    test counts the kernels leave in device memory, so the host does not
  *    wait between rounds (option "graph_rounds").  The rebuilds inside a
  *    batch update run the same way or are sequenced by the host; the routing
- *    rounds of a batch of more than 4096 points read their counts on the
- *    host, a smaller one's are queued together.  Queries are asynchronous:
+ *    rounds of a batch of more than 4096 points (or into a tree of height 126
+ *    or more) read their counts on the host, others are queued together.  Queries are asynchronous:
  *    their outputs are valid once `stream` has been synchronised.
  *  - A pkd_tree is not thread-safe: one call at a time per tree, except
  *    that queries on an unchanging tree may overlap.  Threads may work on

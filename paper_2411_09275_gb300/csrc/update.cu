@@ -782,8 +782,11 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
   // the tree's height / lambda, are queued one after another on bounds of
   // their lists' lengths, and the host reads the counters once at the end.
   // A larger one reads them after every round, for the next round's sieve
-  // and list sizes (about 20 us each).
-  const bool queued = m <= MID_ITEM;
+  // and list sizes (about 20 us each), and so does one into a tree too tall for
+  // the searches' stacks in shared memory: its rounds are counted by the tallest
+  // path, which few batches go down, and the bounds on the lists grow with it
+  // (4096 points at a height of 1e5: 3.3 GB and 17000 rounds).
+  const bool queued = m <= MID_ITEM && query_height_ok(t);
   const uint32_t height = t.st_host->max_depth;  // an upper bound
   const int max_rounds = (int)std::max<uint64_t>(1, ((uint64_t)height + lam - 1) / lam);
   const uint32_t ctl_words = (uint32_t)(max_rounds + 3) * CTL_STRIDE;
@@ -831,11 +834,11 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
                                              (int)CTL_STRIDE + (nbig ? R_BIG : (nmid ? R_MID : R_SMALL))));
   RouteRound all{};  // queued rounds share their lists
   if (queued) {
-    // a point's path has at most `height` inner nodes
-    all.stay_cap = (uint32_t)(m * std::max<uint32_t>(height, 1));
+    // a point's path has at most `height` inner nodes, and a node is listed once
+    all.stay_cap = (uint32_t)std::min<uint64_t>(m * std::max<uint32_t>(height, 1), t.node_cap);
     PKD_TRY(sc.get(&all.stay, all.stay_cap));
     if (!insert) {
-      all.aux_cap = (uint32_t)(m * (height + 1ull));
+      all.aux_cap = (uint32_t)std::min<uint64_t>(m * (height + 1ull), t.node_cap);
       PKD_TRY(sc.get(&all.auxs, all.aux_cap));
     }
     all.ctl = rc(max_rounds + 1);
@@ -891,10 +894,10 @@ static int run_update(TreeMem& t, const int32_t* coords, const uint32_t* ids, co
       ra.aux_cap = all.aux_cap;
     } else {
       RouteRound R{};
-      R.stay_cap = (uint32_t)std::min<uint64_t>(m * (uint64_t)lam, nitems * (uint64_t)(NB - 1));
+      R.stay_cap = (uint32_t)std::min({m * (uint64_t)lam, nitems * (uint64_t)(NB - 1), t.node_cap});
       PKD_TRY(sc.get(&R.stay, R.stay_cap));
       if (!insert) {
-        R.aux_cap = (uint32_t)std::min<uint64_t>(m * (uint64_t)(lam + 1), nitems * (uint64_t)(HN - 1));
+        R.aux_cap = (uint32_t)std::min({m * (uint64_t)(lam + 1), nitems * (uint64_t)(HN - 1), t.node_cap});
         PKD_TRY(sc.get(&R.auxs, R.aux_cap));
       }
       R.ctl = rc(r);
