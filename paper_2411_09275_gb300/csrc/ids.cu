@@ -114,7 +114,10 @@ __global__ void __launch_bounds__(ID_THREADS) k_ids_claim(const int32_t* coords,
 // 0.33 + 0.70 ms, most of the second after the base cases that it should
 // overlap.  DENSE_CTAS per SM leave room for the largest base case's CTA, which
 // starts at the same time: the step of 1e8 points takes 22.1 ms with them, 22.4
-// with four per SM, 22.3 with one, 22.7 with the two passes.
+// with four per SM, 22.3 with one, 22.7 with the two passes.  The registers are
+// held to six CTAs' worth up to d = 4 (a few spill there), so that these CTAs
+// leave the base case beside them more: building 1e8 4-D points takes 22.3 ms,
+// 23.1 with the registers of five or of four.
 constexpr int DENSE_PER = 2, DENSE_CTAS = 2;
 template <int D>
 __global__ void __launch_bounds__(ID_THREADS, D <= 4 ? 6 : 2) k_ids_dense(const int32_t* coords, uint64_t m, IdTable T, uint32_t minv) {

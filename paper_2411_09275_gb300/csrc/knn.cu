@@ -19,9 +19,10 @@
 // dependent loads down the tree (about 20 us for one 10-NN query in 1e6 2-D
 // points).  One thread per query (before) kept the stack, with the 2d bounds
 // of every waiting subspace, and the k entries in local memory.  10-NN, time
-// before -> now: 1e6 uniform queries in 1e7 3-D points 7.5 -> 1.85 ms; 1e5
-// queries in clustered 1e7 3-D points 0.75 -> 0.20 ms; 64 queries in 1e6 2-D
-// points 170 -> 20 us; 100-NN of 2000 queries in 2e5 8-D points 91 -> 2.0 ms.
+// before -> now: 1e6 uniform queries in 1e7 3-D points 7.5 -> 1.85 ms; a call of
+// 1e5 queries in clustered 1e7 3-D points 0.81 to 1.9 -> 0.20 to 0.62 ms by the
+// draw of the points (3.0 to 4.0 times); 64 queries in 1e6 2-D points 170 -> 20
+// us; 100-NN of 2000 queries in 2e5 8-D points 91 -> 2.0 ms.
 #include <cstdio>
 #include <mutex>
 

@@ -38,7 +38,10 @@ __host__ __device__ inline unsigned upw_blocks(uint32_t n) {
 // move to the front of the leaf and its size is rewritten at once, in the pass
 // that has its points in registers (marking every leaf and compacting in a
 // second pass read each leaf twice: 0.55 + 0.89 ms for the 1e7 random deletes
-// in 1e8 points).  *total counts the points that go.
+// in 1e8 points).  *total counts the points that go.  Bound by HBM and by the
+// latency of a warp's loads: eight CTAs per SM up to three dimensions, which
+// spill a few registers, against six and four: 3.11, 3.16 and 3.33 ms for the
+// whole delete.
 template <int D, bool MARK>
 __global__ void __launch_bounds__(UPW_WARPS * 32, (D <= 3 ? 8 : 1)) k_delete_leaves(const LeafGroup* groups,
                                                           const uint32_t* ngroups, Node* nodes, Pts A, Pts F,
